@@ -568,22 +568,24 @@ void grid_take(Bump& B, GridLaunch* G, const GridSizes& z) {
   const size_t as = z.fp64 ? 16 : 8;         // exact sum
   GridHaloState* st = B.take<GridHaloState>((size_t)z.n_grid);
   GridCtl* ctl = B.take<GridCtl>(1);
+  uint32_t* hist = B.take<uint32_t>((size_t)z.n_tiles * 256);   // behind ctl: the bin counts in it are cleared with it
   char* rec = B.take<char>(z.nf * 2 * v4);
-  char* ka = B.take<char>(z.nf * es);
-  char* kb = B.take<char>(z.nf * es);
-  uint32_t* va = B.take<uint32_t>(z.nf);
-  uint32_t* vb = B.take<uint32_t>(z.nf);
-  char* wr = B.take<char>(z.nf * v4);
+  // the radix sort's keys and positions, the radial order and the final
+  // pass's masses: one block, which the bins' records overlay
+  const size_t ke = align_up(z.nf * es, 256), ve = align_up(z.nf * 4, 256), re = align_up(z.nf * v4, 256);
+  char* blk = B.take<char>(2 * ke + 2 * ve + re + z.nf * as);
+  char *ka = blk, *kb = blk + ke;
+  uint32_t *va = (uint32_t*)(blk + 2 * ke), *vb = (uint32_t*)(blk + 2 * ke + ve);
+  char* wr = blk + 2 * ke + 2 * ve;
+  char* mc = wr + re;
   char* ms = B.take<char>(z.masses ? z.nf * es : 0);
   char* uth = B.take<char>(z.gas ? z.nf * es : 0);
   uint32_t* vx = B.take<uint32_t>(z.nf);
-  char* mc = B.take<char>(z.nf * as);
   char* rcp = B.take<char>(z.nf * es);
   int2* trg = B.take<int2>((size_t)z.n_tiles);
   int* th = B.take<int>((size_t)z.n_tiles);
   int* ht0 = B.take<int>((size_t)z.n_grid + 1);
   int* big = B.take<int>((size_t)std::max(1, z.n_big));
-  uint32_t* hist = B.take<uint32_t>((size_t)z.n_tiles * 256);
   uint32_t* dbase = B.take<uint32_t>((size_t)z.n_grid * 256);
   const size_t n_sub = (size_t)z.n_tiles * (GRID_TILE / GRID_SUB);
   char* agm = B.take<char>(2 * n_sub * as);
@@ -604,16 +606,26 @@ void grid_take(Bump& B, GridLaunch* G, const GridSizes& z) {
   G->agg_m = agm; G->agg_r = agr; G->agg_c = agc; G->pre_m = prm_; G->pre_r = prr; G->pre_c = prc;
   G->work = work;
   G->rem_mask = rmask;
+  G->wr_radix = wr;
+  // the block has 2 es + 8 + v4 + as bytes per candidate: 40 (72 in FP64),
+  // the records 2 v4 and the masses es of them: 36 (72)
+  G->rec_b = blk;
+  G->ms_b = blk + 2 * v4 * z.nf;
+  G->rank = (uint16_t*)rcp;
+  G->bin_n = hist;
+  G->bin_at = (uint32_t*)prc;
+  G->wr_bins = rec;
+  G->vr_bins = rec + z.nf * v4;
   G->tile_mv = tmv; G->skip = skip; G->max_halo_tiles = z.max_halo_tiles; G->n_halos = z.n_grid; G->n_flat = (long long)z.nf; G->n_tiles = z.n_tiles;
   G->fp64 = z.fp64 ? 1 : 0;
 }
 
-// Per-call device resets of the class's control words and halo states
-// (before grid_prepare).
+// Per-call device resets of the class's control words, halo states and bin
+// counts (before grid_bins; before grid_prepare with key_and set to all ones).
 int grid_reset(const GridLaunch& G, cudaStream_t s) {
-  AHF_CUDA(cudaMemsetAsync(G.state, 0, sizeof(GridHaloState) * (size_t)G.n_halos, s));
-  AHF_CUDA(cudaMemsetAsync(G.ctl, 0, sizeof(GridCtl), s));
-  AHF_CUDA(cudaMemsetAsync(&G.ctl->key_and, 0xff, sizeof(unsigned long long), s));
+  // states, control words and bin counts lie back to back
+  char* end = (char*)G.bin_n + (size_t)G.n_tiles * 2 * 128;
+  AHF_CUDA(cudaMemsetAsync(G.state, 0, (size_t)(end - (char*)G.state), s));
   return AHF_OK;
 }
 
@@ -633,34 +645,53 @@ int run_grid(ahf_ctx* c, GridLaunch& G, const ahf_params* prm, cudaStream_t s, i
   // the passes stage the stream through tensor copies (mixed mode, a uniform
   // mass, no gas) when the device takes them
   G.wait_limit = c->wait_limit;
-  G.use_tma = 0;
-  if (!G.fp64 && !G.ms && !G.uth) {
-    if (c->tma_grid < 0) c->tma_grid = grid_tma_grid(c->device);
-    G.tma_grid = c->tma_grid;
-    if (G.tma_grid > 0 && grid_wr_map(G, (G.n_flat + 7) / 8)) G.use_tma = 1;
-  }
-  AHF_CUDA(cudaMemcpyAsync(c->flag_host, &G.ctl->key_or, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-  AHF_CUDA(cudaStreamSynchronize(s));
-  c->stats.host_syncs += 1;
-  unsigned long long orb, andb;
-  std::memcpy(&orb, c->flag_host, 8);
-  std::memcpy(&andb, c->flag_host + 2, 8);
-  AHF_CUDA(grid_sort(G, s, orb, andb));
+  auto streams = [&](bool bins) {
+    G.wr = bins ? G.wr_bins : G.wr_radix;
+    G.vr = bins ? G.vr_bins : nullptr;
+    G.use_tma = 0;
+    if (!G.fp64 && !G.ms && !G.uth) {
+      if (c->tma_grid < 0) c->tma_grid = grid_tma_grid(c->device);
+      G.tma_grid = c->tma_grid;
+      if (G.tma_grid > 0 && grid_wr_map(G, (G.n_flat + 7) / 8)) G.use_tma = 1;
+    }
+  };
+  streams(true);
+  AHF_CUDA(grid_bins(G, s));
   c->stats.launches += G.sort_launches;
   if ((rc = phase_end(c, PH_GRID_SORT, s))) return rc;
   if ((rc = phase_begin(c, PH_GRID_ITER, s, G.n_halos, G.n_flat))) return rc;
-  for (int pass = 1; pass <= prm->max_iter;) {
+  bool radix = false;
+  for (int pass = 1;;) {
     const int n = std::min(chunk, prm->max_iter - pass + 1);
     for (int i = 0; i < n; ++i) {
       AHF_CUDA(grid_iterate(G, pass++, s));
       c->stats.launches += 3;
       c->stats.grid_iterations += 1;
     }
-    if (pass > prm->max_iter) break;
-    AHF_CUDA(cudaMemcpyAsync(c->flag_host + 4, &G.ctl->work_n[pass & 1], sizeof(int), cudaMemcpyDeviceToHost, s));
+    // work_n and the bins' overflow word
+    AHF_CUDA(cudaMemcpyAsync(c->flag_host, G.ctl, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
     AHF_CUDA(cudaStreamSynchronize(s));
     c->stats.host_syncs += 1;
-    if (c->flag_host[4] == 0) break;
+    if (!radix && c->flag_host[2]) {
+      // a radial bin overflowed (the passes above had no active halo): the
+      // radix sort orders any radii
+      radix = true;
+      pass = 1;
+      streams(false);
+      if ((rc = grid_reset(G, s))) return rc;
+      AHF_CUDA(cudaMemsetAsync(&G.ctl->key_and, 0xff, sizeof(unsigned long long), s));
+      AHF_CUDA(grid_prepare(G, s));
+      AHF_CUDA(cudaMemcpyAsync(c->flag_host, &G.ctl->key_or, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+      AHF_CUDA(cudaStreamSynchronize(s));
+      c->stats.host_syncs += 1;
+      unsigned long long orb, andb;
+      std::memcpy(&orb, c->flag_host, 8);
+      std::memcpy(&andb, c->flag_host + 2, 8);
+      AHF_CUDA(grid_sort(G, s, orb, andb));
+      c->stats.launches += 2 + G.sort_launches;
+      continue;
+    }
+    if (pass > prm->max_iter || c->flag_host[pass & 1] == 0) break;
   }
   if ((rc = phase_end(c, PH_GRID_ITER, s))) return rc;
   if ((rc = phase_begin(c, PH_GRID_FINISH, s, G.n_halos, G.n_flat))) return rc;
@@ -875,9 +906,6 @@ int unbind_pass(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64
     G.rows.factor = dfac;
     G.rows.factor_f = dfacf;
     G.rows.n_bins = n_bins;
-    if ((rc = phase_begin(c, PH_GRID_SORT, s, n_grid, (long long)nf))) return rc;
-    AHF_CUDA(grid_prepare(G, s));
-    c->stats.launches += 2;
   }
   if ((rc = pin_release(c, s))) return rc;
   if (c->trace) {
@@ -1010,6 +1038,7 @@ int unbind_pass(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64
   } else {
     if ((rc = enqueue_onchip(s, false))) return rc;
     if (n_grid) {
+      if ((rc = phase_begin(c, PH_GRID_SORT, s, n_grid, (long long)nf))) return rc;
       if ((rc = run_grid(c, G, prm, s, c->pass_chunk))) return rc;
       if (push) {
         AHF_CUDA(launch_push(*push, hd + n_onchip, n_grid, P.hd[(size_t)n_onchip].count, s));
@@ -1234,8 +1263,6 @@ int plain_impl(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64_
       continue;
     }
     if ((rc = phase_begin(c, PH_GRID_SORT, s, 1, d.count))) return rc;
-    AHF_CUDA(grid_prepare(G, s));
-    c->stats.launches += 2;
     // the plain form reads the change flag after every pass
     if ((rc = run_grid(c, G, prm, s, 1))) return rc;
   }

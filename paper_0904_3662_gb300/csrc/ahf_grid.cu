@@ -8,14 +8,14 @@
 //   prepare  one coalesced read of the candidates: recentring, sphere test,
 //            radius key, and a 32-byte record per candidate, (w, r) and
 //            (v, m) with w = v + H d (64 bytes in the all-FP64 mode)
-//   sort     segmented stable LSD radix sort of (key, position) with 8-bit
-//            digits (tile histograms, per-(halo, digit) scans over tiles,
-//            digit bases, a scatter ranked by warp ballots and staged in
-//            shared memory so that each digit's run is written contiguously);
-//            the last pass gathers each member's record once and writes the
-//            radial-order stream (w, r) (+ m), so no later step touches the
-//            particle store
-//   init     exact sums of the initial set per tile and per halo, v_bulk
+//   sort     members distributed into radial bins by rank of arrival (counted
+//            by the prepare), each bin then ordered on chip by one CTA, which
+//            writes the radial-order streams (w, r), (v, m), so no later step
+//            touches the particle store.  Radii that the bins cannot hold
+//            (hundreds equal, a thin shell in a void) take a segmented stable LSD
+//            radix sort of (key, position) with 8-bit digits instead
+//   init     exact sums of the initial set per sub-tile (with the bins) and per
+//            halo, v_bulk
 //   passes   ONE streaming kernel per iteration: each tile takes the exact
 //            prefix sums M(<r) and sum m/r of the tiles before it from the
 //            tile prefixes of the current set, evaluates phi (Appendix A),
@@ -34,6 +34,7 @@
 // Exact sums: long long fixed point in the mixed mode (the same scales and
 // bits as the on-chip classes), __int128 in the all-FP64 mode, where a
 // 64-bit quantum would limit large haloes to ~1e-11 relative in sum m/r.
+#include <algorithm>
 #include <atomic>
 #include <cstdint>
 
@@ -46,7 +47,7 @@ constexpr int T = GRID_THREADS;         // 256
 constexpr int TILE = GRID_TILE;         // 2048
 constexpr int IPT = TILE / T;           // 8 elements per thread
 constexpr int NWARP = T / 32;
-static_assert(T == 256, "one thread per byte digit in the histograms and scans");
+static_assert(T == 256 && GRID_TILE == 2048, "one thread per byte digit in the histograms and scans");
 
 // Precision of the per-particle arithmetic.  float: the mixed mode (FP32
 // radius key, FP32 phi and escape test).  double: the all-FP64 mode (FP64
@@ -250,6 +251,8 @@ __device__ __forceinline__ X block_excl(X x, X* red) {
 
 __device__ __forceinline__ uint32_t key_of(float r) { return __float_as_uint(r); }
 __device__ __forceinline__ unsigned long long key_of(double r) { return (unsigned long long)__double_as_longlong(r); }
+__device__ __forceinline__ float radius_of_key(uint32_t k) { return __uint_as_float(k); }
+__device__ __forceinline__ double radius_of_key(unsigned long long k) { return __longlong_as_double((long long)k); }
 __device__ __forceinline__ int exp_of_bits(unsigned long long b, float) { return (int)((b >> 23) & 0xff) - 127; }
 __device__ __forceinline__ int exp_of_bits(unsigned long long b, double) { return (int)((b >> 52) & 0x7ff) - 1023; }
 __device__ __forceinline__ unsigned long long abs_bits(float x) { return __float_as_uint(fabsf(x)); }
@@ -261,6 +264,13 @@ __device__ __forceinline__ double rinv_real(double r, const ParamsDev& P) {
   const double rr = fmax(r, P.r_soft);
   return rr > 0.0 ? 1.0 / rr : 0.0;
 }
+// rinv_real(r, P) > 0, without the division
+__device__ __forceinline__ bool rinv_positive(float r, const ParamsDev& P) { return fmaxf(r, P.r_soft_f) > 0.0f; }
+__device__ __forceinline__ bool rinv_positive(double r, const ParamsDev& P) { return fmax(r, P.r_soft) > 0.0; }
+__device__ __forceinline__ unsigned long long bits_of(float x) { return __float_as_uint(x); }
+__device__ __forceinline__ unsigned long long bits_of(double x) { return (unsigned long long)__double_as_longlong(x); }
+__device__ __forceinline__ float real_of_bits(unsigned long long b, float) { return __uint_as_float((uint32_t)b); }
+__device__ __forceinline__ double real_of_bits(unsigned long long b, double) { return __longlong_as_double((long long)b); }
 __device__ __forceinline__ float phi_real(float M, float ri, float S, const ParamsDev& P) { return phi_of(M, ri, S, P.Gf); }
 __device__ __forceinline__ double phi_real(double M, double ri, double S, const ParamsDev& P) {
   return __dmul_rn(-P.G, __fma_rn(M, ri, S));
@@ -330,6 +340,49 @@ __device__ __forceinline__ void store_low_byte_hist(const GridLaunch& L, int t, 
   L.tile_hist[(size_t)t0 * 256 + (size_t)threadIdx.x * th + (t - t0)] = h[threadIdx.x];
 }
 
+// The largest m, m / max(r, r_soft) and |m v_k| of a thread's members (the
+// scales of the exact sums follow from their exponents).  With one mass for all
+// only the smallest radius and the largest |v_k| are kept: rounding is monotone,
+// so m0 times their values is the largest of the products, and the reciprocal
+// and three products per candidate fall away.
+template <typename R>
+struct Maxima {
+  using Key = typename Prec<R>::Key;
+  Key m = 0, a = 0, v = 0;                 // uniform mass: a = complement of the smallest r's bits, v = |v| bits
+  __device__ __forceinline__ void add(const ParamsDev& P, bool masses, R mass, R r, const R vel[3]) {
+    if (masses) {
+      m = max(m, (Key)abs_bits(mass));
+      a = max(a, (Key)abs_bits(mass * rinv_real(r, P)));
+#pragma unroll
+      for (int k = 0; k < 3; ++k) v = max(v, (Key)abs_bits(mul_rn(mass, vel[k])));
+    } else {
+      // (a radius of zero has a reciprocal of zero unless softened: left out)
+      if (rinv_positive(r, P)) a = max(a, (Key)~(Key)bits_of(r));
+#pragma unroll
+      for (int k = 0; k < 3; ++k) v = max(v, (Key)abs_bits(vel[k]));
+    }
+  }
+  // The warp's maxima, in every lane.
+  __device__ __forceinline__ void warp(const ParamsDev& P, bool masses, const ParticlesDev& p, int n,
+                                       unsigned long long& mm, unsigned long long& mr, unsigned long long& mv) {
+    for (int o = 16; o > 0; o >>= 1) {
+      m = max(m, __shfl_xor_sync(FULL_MASK, m, o));
+      a = max(a, __shfl_xor_sync(FULL_MASK, a, o));
+      v = max(v, __shfl_xor_sync(FULL_MASK, v, o));
+    }
+    mm = m;
+    mr = a;
+    mv = v;
+    if (!masses) {
+      const R m0 = sizeof(R) == 4 ? (R)p.m0f : (R)p.m0;
+      const bool any = __any_sync(FULL_MASK, n > 0);
+      mm = any ? abs_bits(m0) : 0ull;
+      mr = a ? abs_bits(m0 * rinv_real(real_of_bits((Key)~a, R()), P)) : 0ull;
+      mv = abs_bits(mul_rn(m0, real_of_bits(v, R())));
+    }
+  }
+};
+
 // The CTA's key range, per-halo maxima and member count merged into the call's
 // words.  Every thread passes its warp's reduced values; the CTA reduces them
 // once more and thread 0 issues an atomic only where it can change the word
@@ -372,9 +425,303 @@ __device__ __forceinline__ void merge_prepare(const GridLaunch& L, int k, unsign
   if (n) atomicAdd((unsigned long long*)&st->n_member, (unsigned long long)n);
 }
 
+// ---- distribution over radial bins -----------------------------------------------
+//
+// The radial order needs no comparison sort of a whole halo.  A halo of th
+// tiles gets 2 th bins of radius (1,024 candidates each on average, cut into 512
+// parts; a halo of one tile is one bin), monotone in r.  The prepare counts each member in its bin and keeps
+// its rank of arrival; a scan of the bins' counts gives every bin its first
+// position; one scatter moves each member's record to its bin; and one CTA per
+// bin orders it on chip and writes the radial-order streams.  Against the radix
+// sort below (a histogram, two scans and a scatter per key byte, then a random
+// gather of every record) each record moves twice, as one full 32-byte sector.
+//
+// The bins follow the halo's own distribution: a strided sample of its
+// candidates is counted in 1,024 cells (256 for small haloes) of equal width in
+// the bits of r (so logarithmic in r) from below its smallest radius up to its largest, and each
+// cell gets parts of bins in proportion to its count (and a little more, so
+// that no cell is left without), a member's place within its cell taken as
+// linear in the bits of r.  Radii beyond the largest sampled one get tail parts
+// in intervals that double in width.  The sample only balances the bins; the
+// order does not depend on it.
+//
+// Measured against the radix sort for every halo (whole calls): 64 hosts of
+// 1.5e8 candidates 13.2 -> 12.2 ms; 3,000 haloes in FP64 (keys of 8 bytes) 2.70 ->
+// 2.11 ms; 11,000 candidates in FP64 590 -> 432 us; 3 hosts of 4e6 with gas 0.84 ->
+// 0.75 ms.  The prepare is bound by its integer arithmetic and the latency of
+// the counting atomics, the scatter by DRAM (two thirds of its peak), the
+// ordering by issue slots (65 % busy).
+//
+// A bin holds BIN_MAX members at most (its CTA's shared memory).  When one would
+// hold more (thousands of equal radii, a thin shell in a void), or a part so
+// many that ordering it by counting would be slow, ctl->overflow is set, every
+// later kernel of the attempt returns at once and the host runs the radix sort
+// instead.
+
+constexpr int CELLS = 1024;              // at most
+constexpr int SAMPLE_T = 1024;
+constexpr int SAMPLE_PT = 32;            // sampled candidates per thread
+constexpr int SAMPLE_MAX = SAMPLE_T * SAMPLE_PT;
+constexpr int TAILS = 32;                // tail intervals
+constexpr int PARTS = 512;               // parts of a bin
+constexpr uint32_t TAB_UNIT = 2u;        // bin tables count in halves of a part (below 2^32 for any halo)
+constexpr uint32_t NO_RANK = 0xffffu;    // rank of a non-member
+static_assert(PARTS == 2 * T, "two parts a thread");
+constexpr int BIN_MAX = 3072;            // members of a bin
+constexpr uint32_t PART_MAX = 512u;      // members of a part
+constexpr int BIN_PAD = 32;              // words between bins' counters: atomics on one 128-byte line queue
+constexpr int AGG_BINS = 512;            // halo's bins up to which a CTA counts in shared memory first
+
+// Bins of a halo of th tiles; its first is 2 t0.
+__host__ __device__ __forceinline__ int halo_bins(int th) { return th > 1 ? 2 * th : th; }
+
+__device__ __forceinline__ bool bins_overflowed(const GridLaunch& L) { return __ldcg(&L.ctl->overflow) != 0; }
+
+// The key a bin is found from: the bits of r as a float (rounding a double
+// radius is monotone).
+__device__ __forceinline__ uint32_t bin_key(float r) { return __float_as_uint(r); }
+__device__ __forceinline__ uint32_t bin_key(double r) { return __float_as_uint(__double2float_rn(r)); }
+
+// Candidates sampled of n: an eighth, 512 to SAMPLE_MAX of them.
+__device__ __forceinline__ int sample_size(long long n) {
+  return (int)min(n, max(512ll, min((long long)SAMPLE_MAX, n >> 3)));
+}
+// Parts of one tail interval: four times the candidates expected beyond the
+// largest of the sample, at two to a part.  TAILS intervals stay below half
+// of a halo's parts (2,048 at least).
+__device__ __forceinline__ uint32_t tail_parts(long long n) {
+  const int S = sample_size(n);
+  return S > 0 ? 2u * (uint32_t)(n / S) : 1u;
+}
+
+// Cells of a halo of th tiles.
+__host__ __device__ __forceinline__ int map_cells(int th) { return th >= 8 ? CELLS : 256; }
+// Its table of cells, behind the bins' counters in tile_hist (192 words a tile).
+__device__ __forceinline__ uint32_t* bin_table(const GridLaunch& L, int t0) {
+  return L.tile_hist + (size_t)L.n_tiles * 2 * BIN_PAD + (size_t)t0 * (256 - 2 * BIN_PAD);
+}
+
+// A halo's map from keys to parts (PARTS to a bin): `cells` cells of 2^sh keys from
+// k0 on, ending with the largest sampled key kx; tail intervals of 2^gs keys,
+// then doubling.
+struct BinMap {
+  uint32_t k0, kx, tb, main;             // main: parts before the tails
+  int sh, gs, cells;
+};
+
+// The map of halo k and its cells' first parts (in units of 1 / TAB_UNIT; the last
+// entry: main) into shared memory.
+__device__ __forceinline__ BinMap load_bin_map(const GridLaunch& L, int k, int t0, long long n, int th, uint32_t* tab) {
+  const GridHaloState& S = L.state[k];
+  BinMap M;
+  M.k0 = S.bin_k0;
+  M.kx = S.bin_kx;
+  M.sh = S.bin_shifts & 255;
+  M.gs = S.bin_shifts >> 8;
+  M.tb = tail_parts(n);
+  M.main = (uint32_t)halo_bins(th) * PARTS - TAILS * M.tb;
+  M.cells = map_cells(th);
+  const uint32_t* src = bin_table(L, t0);
+  if (th > 1)
+    for (int c = threadIdx.x; c < M.cells; c += T) tab[c] = src[c];
+  if (threadIdx.x == 0) tab[M.cells] = M.main * TAB_UNIT;
+  return M;
+}
+
+// Part of a key (monotone in it): its cell, then linear within the cell; keys
+// below the first cell go to part 0.
+__device__ __forceinline__ uint32_t part_of(uint32_t key, const BinMap& M, const uint32_t* tab) {
+  if (key > M.kx) {
+    const uint32_t x = key - M.kx - 1u, y = x >> M.gs;
+    const int i = y == 0u ? 0 : 32 - __clz(y);
+    const int w = i == 0 ? M.gs : M.gs + i - 1;        // the interval's width
+    const uint32_t lo = i == 0 ? x : x - (1u << w);
+    return M.main + (uint32_t)i * M.tb + (uint32_t)(((unsigned long long)lo * M.tb) >> w);
+  }
+  const uint32_t x = key > M.k0 ? key - M.k0 : 0u;
+  const uint32_t c = min(x >> M.sh, (uint32_t)M.cells - 1u);
+  const uint32_t lo = min(x - (c << M.sh), (1u << M.sh) - 1u);
+  const uint32_t b0 = tab[c], w = tab[c + 1] - b0;
+  return min((b0 + (uint32_t)(((unsigned long long)w * lo) >> M.sh)) / TAB_UNIT, M.main - 1u);
+}
+
+static_assert(CELLS == SAMPLE_T && 8 * (256 - 2 * BIN_PAD) >= CELLS && 2 * (256 - 2 * BIN_PAD) >= 256, "bin tables");
+
+// The sample's keys, one candidate per thread, to rec_b at the halo's base, and
+// their extremes.  CTA b of halo k: from a grid of (b, k), or of the tiles, of
+// which each halo's first ones serve (whichever grid is the smaller).
+template <typename R, int CT>
+__global__ void __launch_bounds__(T) g_sample(GridLaunch L) {
+  const int k = gridDim.y > 1 ? blockIdx.y : L.tile_halo[blockIdx.x];
+  const int t0 = L.halo_tile0[k], th = L.halo_tile0[k + 1] - t0;
+  if (th <= 1) return;                   // one bin: no map
+  const HaloDev& H = L.halos[k];
+  const long long n = H.count;
+  const int S = sample_size(n);
+  const int b = gridDim.y > 1 ? blockIdx.x : blockIdx.x - t0;
+  if (b >= (S + T - 1) / T) return;      // (at most th shares: S is an eighth of n, or 512 of two tiles)
+  const int j = b * T + threadIdx.x;
+  uint32_t key = KEY_NONMEMBER;
+  const bool in = j < S;
+  if (in) {
+    // groups of 8 neighbours (one or two sectors per array), evenly spread
+    const long long groups = (S + 7) >> 3;
+    long long pi = H.offset + min(((j >> 3) * n) / groups + (j & 7), n - 1);
+    if (L.out.member_idx) pi = L.out.member_idx[pi];
+    if (pi >= 0 && pi < L.p.n) {
+      if constexpr (sizeof(R) == 4) {
+        float d[3];
+        long long f[3];
+        offset_of<CT>(L.p, pi, H, d, f);
+        if (member_of<CT>(L.p, pi, H, d, f)) key = bin_key(radius_of(d));
+      } else {
+        double d[3];
+        offset_f64<CT>(L.p, pi, H, L.frame.box, d);
+        const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])), __dmul_rn(d[2], d[2]));
+        if (r2 <= H.R2) key = bin_key(sqrt(r2));
+      }
+    }
+    ((uint32_t*)L.rec_b)[H.gbase + j] = key;
+  }
+  const bool mem = key != KEY_NONMEMBER;
+  const uint32_t km = __reduce_max_sync(FULL_MASK, mem ? key : 0u);
+  const uint32_t kn = __reduce_max_sync(FULL_MASK, mem ? ~key : 0u);
+  if ((threadIdx.x & 31) == 0 && kn) {
+    atomicMax(&L.state[k].bin_kx, km);
+    atomicMax(&L.state[k].bin_k0, kn);   // the complement of the smallest key
+  }
+}
+
+// One CTA per halo: the sample's cells and the table.
+__global__ void __launch_bounds__(SAMPLE_T) g_bin_map(GridLaunch L) {
+  __shared__ uint32_t cell[CELLS];
+  __shared__ uint32_t wt[SAMPLE_T / 32];
+  const int k = blockIdx.x;
+  const HaloDev& H = L.halos[k];
+  const long long n = H.count;
+  const int th = L.halo_tile0[k + 1] - L.halo_tile0[k];
+  if (th <= 1) return;
+  const int S = sample_size(n);
+  const uint32_t* skey = (const uint32_t*)L.rec_b + H.gbase;
+  const uint32_t kx = L.state[k].bin_kx, kn = min(~L.state[k].bin_k0, kx);
+  const int cells = map_cells(th), log_cells = cells == CELLS ? 10 : 8;
+  cell[threadIdx.x] = 0u;
+  // the cells end with the largest sampled key and start a quarter of the
+  // sampled range and two octaves below the smallest
+  const uint32_t range = kx - kn;
+  const uint32_t want = range + (range >> 2) + (2u << 23);        // < 2^32
+  const int sh = 32 - log_cells - __clz(want - 1u);               // cells << sh >= want
+  const uint32_t span = (uint32_t)min((unsigned long long)cells << sh, 0xffffffffull);
+  const uint32_t k0 = kx + 1u > span ? kx + 1u - span : 0u;
+  __syncthreads();
+#pragma unroll 8
+  for (int j = threadIdx.x; j < S; j += SAMPLE_T) {
+    const uint32_t key = skey[j];
+    if (key != KEY_NONMEMBER) atomicAdd(&cell[min((key > k0 ? key - k0 : 0u) >> sh, (uint32_t)cells - 1u)], 1u);
+  }
+  __syncthreads();
+  const int c = threadIdx.x, lane = c & 31, warp = c >> 5;
+  // weight of a cell with m samples: m + 3 sqrt(m) + 4 (scaled down for small
+  // samples), an upper estimate, so that the bins of cells a few samples fell in
+  // rarely hold more than their share
+  uint32_t w = 0u;
+  if (c < cells) {
+    const float m = (float)cell[c];
+    w = (uint32_t)(64.0f * (m + 3.0f * sqrtf(m))) + max(1u, (uint32_t)S / 128u);
+  }
+  const uint32_t inc = warp_inclusive_scan(w, lane);
+  if (lane == 31) wt[warp] = inc;
+  __syncthreads();
+  if (c < cells) {
+    uint32_t base = inc - w, tot = 0;
+    for (int v = 0; v < SAMPLE_T / 32; ++v) {
+      const uint32_t x = wt[v];
+      if (v < warp) base += x;
+      tot += x;
+    }
+    const unsigned long long all = ((unsigned long long)halo_bins(th) * PARTS - TAILS * tail_parts(n)) * TAB_UNIT;
+    bin_table(L, L.halo_tile0[k])[c] = (uint32_t)((all * base) / tot);
+    if (c == 0) {
+      // the tails start with a quarter of the spacing of the last cells' samples
+      const uint32_t cx = min((kx - k0) >> sh, (uint32_t)cells - 1u);
+      const uint32_t sp = (1u << sh) / (cell[cx] + (cx ? cell[cx - 1] : 0u) + 1u);
+      GridHaloState& st = L.state[k];
+      st.bin_k0 = k0;
+      st.bin_shifts = sh | (max(0, 29 - __clz(max(sp, 1u))) << 8);
+    }
+  }
+}
+
+// Bin of a member and its rank of arrival there, for the members a CTA holds at
+// one step: `bin` their bins (relative to the halo's first), mem false for
+// none.  One bin: a warp's members take consecutive ranks (one atomic per
+// warp); AGG_BINS at most: counted in shared memory first (scnt, zero before and
+// reused as the bins' bases), one global atomic per bin met.  (With more bins
+// each member's atomic is issued where its bin is found: bin_rank_now.)
+template <int N>
+__device__ __forceinline__ void bin_ranks(uint32_t* cnt, int nb, const bool mem[N], const uint32_t bin[N], uint32_t rk[N],
+                                          uint32_t* scnt) {
+  if (nb == 1) {
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const unsigned m = __ballot_sync(FULL_MASK, mem[q]);
+      uint32_t base = 0;
+      if ((threadIdx.x & 31) == 0 && m) base = atomicAdd(cnt, (uint32_t)__popc(m));
+      base = __shfl_sync(FULL_MASK, base, 0);
+      rk[q] = base + __popc(m & lanemask_lt());
+    }
+  } else if (nb <= AGG_BINS) {
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (mem[q]) rk[q] = atomicAdd(&scnt[bin[q]], 1u);
+    __syncthreads();
+    for (int c = threadIdx.x; c < nb; c += T) {
+      const uint32_t v = scnt[c];
+      if (v) scnt[c] = atomicAdd(&cnt[(size_t)c * BIN_PAD], v);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (mem[q]) rk[q] += scnt[bin[q]];
+  }
+}
+__device__ __forceinline__ uint32_t bin_rank_now(uint32_t* cnt, int nb, uint32_t bin) {
+  return nb > AGG_BINS ? atomicAdd(&cnt[(size_t)bin * BIN_PAD], 1u) : 0u;
+}
+
+// The tile's sub-tile sums of the initial set (copy 1) and its sum m v zeroed,
+// for the CTAs that will add to them.
+template <typename R>
+__device__ __forceinline__ void zero_sums(const GridLaunch& L, int t) {
+  using Acc = typename Prec<R>::Acc;
+  if (threadIdx.x < GRID_TILE / GRID_SUB) {
+    const size_t u = (size_t)(L.n_tiles + t) * (GRID_TILE / GRID_SUB) + threadIdx.x;
+    ((Acc*)L.agg_m)[u] = 0;
+    ((Acc*)L.agg_r)[u] = 0;
+    L.agg_c[u] = 0;
+  }
+  if (threadIdx.x < 3) A<Acc>(L.tile_mv[3 * (size_t)t + threadIdx.x]) = 0;
+}
+
+// The ranks of a thread's candidates (element q T + thread of the tile; rank
+// NO_RANK for a non-member).
+template <int N>
+__device__ __forceinline__ void store_ranks(const GridLaunch& L, int2 tr, const bool mem[N], const uint32_t rk[N]) {
+  bool over = false;
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    const int e = q * T + threadIdx.x;
+    if (e < tr.y) L.rank[(size_t)tr.x + e] = (uint16_t)(mem[q] ? min(rk[q], NO_RANK) : NO_RANK);
+    over |= mem[q] && rk[q] >= (uint32_t)BIN_MAX;
+  }
+  if (over) L.ctl->overflow = 1;
+}
+
 // Mixed precision: the on-chip classes' float offsets (exact recentring),
 // membership and radius; the record holds w = v + H d and r, then v and m.
-template <int CT>
+// BINS: each member is counted in its radial bin and its rank of arrival kept;
+// otherwise the keys and the first digit's histogram of the radix sort.
+template <int CT, bool BINS>
 __global__ void __launch_bounds__(T, 4) g_prepare_mixed(GridLaunch L) {
   const int t = blockIdx.x;
   const int2 tr = L.tile_range[t];
@@ -383,8 +730,16 @@ __global__ void __launch_bounds__(T, 4) g_prepare_mixed(GridLaunch L) {
   const ParamsDev& P = L.prm;
   uint32_t* key_a = (uint32_t*)L.key_a;
   float4* rec = (float4*)L.rec;
-  __shared__ uint32_t h0[256];
-  h0[threadIdx.x] = 0u;
+  __shared__ uint32_t h0[CELLS + 1];
+  __shared__ uint32_t scnt[BINS ? AGG_BINS : 1];
+  const int t0 = L.halo_tile0[k], th = L.halo_tile0[k + 1] - t0;
+  BinMap BM;
+  if (BINS) {
+    BM = load_bin_map(L, k, t0, H.count, th, h0);
+    zero_sums<float>(L, t);
+    if (halo_bins(th) <= AGG_BINS)
+      for (int c = threadIdx.x; c < halo_bins(th); c += T) scnt[c] = 0u;
+  } else h0[threadIdx.x] = 0u;
   Cand<CT> c[IPT];
   bool ok[IPT];
 #pragma unroll
@@ -405,12 +760,16 @@ __global__ void __launch_bounds__(T, 4) g_prepare_mixed(GridLaunch L) {
     }
   }
   uint32_t orb = 0, andb = 0xffffffffu;
-  unsigned long long mxm = 0, mxr = 0, mxv = 0;
+  Maxima<float> mx;
   int nmem = 0;
-  __syncthreads();                       // h0 zeroed
+  uint32_t* cnt = L.bin_n + (size_t)t0 * 2 * BIN_PAD;
+  const int nb = halo_bins(th);
+  __syncthreads();                       // h0 is ready
+  uint32_t bin[IPT], rk[IPT];
 #pragma unroll
   for (int q = 0; q < IPT; ++q) {
     const int e = q * T + threadIdx.x;
+    bin[q] = 0u;
     if (e >= tr.y) continue;
     const long long g = (long long)tr.x + e;
     uint32_t key = KEY_NONMEMBER;
@@ -418,7 +777,8 @@ __global__ void __launch_bounds__(T, 4) g_prepare_mixed(GridLaunch L) {
       float d[3];
       long long f[3];
       cand_offset<CT>(c[q], H, d, f);
-      if (cand_member<CT>(c[q], H, d, f)) {
+      ok[q] = cand_member<CT>(c[q], H, d, f);
+      if (ok[q]) {
         const float r = radius_of(d);
         const float m = cand_mass<CT>(L.p, c[q]);
         float v[3];
@@ -426,34 +786,44 @@ __global__ void __launch_bounds__(T, 4) g_prepare_mixed(GridLaunch L) {
         rec[2 * g] = make_float4(fmaf(P.Hf, d[0], v[0]), fmaf(P.Hf, d[1], v[1]), fmaf(P.Hf, d[2], v[2]), r);
         rec[2 * g + 1] = make_float4(v[0], v[1], v[2], m);
         key = key_of(r);
-        mxm = max(mxm, abs_bits(m));
-        mxr = max(mxr, abs_bits(m * rinv_real(r, P)));
-#pragma unroll
-        for (int a = 0; a < 3; ++a) mxv = max(mxv, abs_bits(mul_rn(m, v[a])));
+        if (BINS && th > 1) {
+          bin[q] = part_of(bin_key(r), BM, h0) / PARTS;
+          rk[q] = bin_rank_now(cnt, nb, bin[q]);
+        }
+        mx.add(P, L.p.m != nullptr, m, r, v);
         ++nmem;
       }
     }
     if (L.out.removed_iter) L.out.removed_iter[H.offset + (g - H.gbase)] = key == KEY_NONMEMBER ? -1 : 0;
-    key_a[g] = key;
-    atomicAdd(&h0[key & 0xffu], 1u);
-    orb |= key;
-    andb &= key;
+    if (!BINS) {
+      key_a[g] = key;
+      atomicAdd(&h0[key & 0xffu], 1u);
+      orb |= key;
+      andb &= key;
+    }
   }
-  __syncthreads();
-  store_low_byte_hist(L, t, k, h0);
-  for (int o = 16; o > 0; o >>= 1) {
-    orb |= __shfl_xor_sync(FULL_MASK, orb, o);
-    andb &= __shfl_xor_sync(FULL_MASK, andb, o);
-    mxm = max(mxm, __shfl_xor_sync(FULL_MASK, mxm, o));
-    mxr = max(mxr, __shfl_xor_sync(FULL_MASK, mxr, o));
-    mxv = max(mxv, __shfl_xor_sync(FULL_MASK, mxv, o));
+  if (BINS) {
+    bin_ranks<IPT>(cnt, nb, ok, bin, rk, scnt);
+    store_ranks<IPT>(L, tr, ok, rk);
+  } else {
+    __syncthreads();
+    store_low_byte_hist(L, t, k, h0);
   }
+  if (!BINS) {
+    for (int o = 16; o > 0; o >>= 1) {
+      orb |= __shfl_xor_sync(FULL_MASK, orb, o);
+      andb &= __shfl_xor_sync(FULL_MASK, andb, o);
+    }
+  }
+  unsigned long long mxm, mxr, mxv;
+  mx.warp(P, L.p.m != nullptr, L.p, nmem, mxm, mxr, mxv);
   nmem = __reduce_add_sync(FULL_MASK, nmem);
-  merge_prepare(L, k, orb, (unsigned long long)andb | 0xffffffff00000000ull, mxm, mxr, mxv, nmem);
+  if (BINS) merge_prepare(L, k, 0ull, ~0ull, mxm, mxr, mxv, nmem);
+  else merge_prepare(L, k, orb, (unsigned long long)andb | 0xffffffff00000000ull, mxm, mxr, mxv, nmem);
 }
 
 // All-FP64 mode: d = x - c in FP64 (minimum image), r^2 = (dx^2 + dy^2) + dz^2.
-template <int CT>
+template <int CT, bool BINS>
 __global__ void __launch_bounds__(T) g_prepare_f64(GridLaunch L) {
   const int t = blockIdx.x;
   const int2 tr = L.tile_range[t];
@@ -462,12 +832,30 @@ __global__ void __launch_bounds__(T) g_prepare_f64(GridLaunch L) {
   const ParamsDev& P = L.prm;
   unsigned long long* key_a = (unsigned long long*)L.key_a;
   D4* rec = (D4*)L.rec;
-  unsigned long long orb = 0, andb = ~0ull, mxm = 0, mxr = 0, mxv = 0;
+  unsigned long long orb = 0, andb = ~0ull;
+  Maxima<double> mx;
   int nmem = 0;
-  __shared__ uint32_t h0[256];
-  h0[threadIdx.x] = 0u;
+  __shared__ uint32_t h0[CELLS + 1];
+  __shared__ uint32_t scnt[BINS ? AGG_BINS : 1];
+  const int t0 = L.halo_tile0[k], th = L.halo_tile0[k + 1] - t0;
+  BinMap BM;
+  if (BINS) {
+    BM = load_bin_map(L, k, t0, H.count, th, h0);
+    zero_sums<double>(L, t);
+    if (halo_bins(th) <= AGG_BINS)
+      for (int c = threadIdx.x; c < halo_bins(th); c += T) scnt[c] = 0u;
+  } else h0[threadIdx.x] = 0u;
   __syncthreads();
-  for (int e = threadIdx.x; e < tr.y; e += T) {
+  bool mem[IPT];
+  uint32_t bin[IPT], rk[IPT];
+  uint32_t* cnt = L.bin_n + (size_t)t0 * 2 * BIN_PAD;
+  const int nb = halo_bins(th);
+#pragma unroll
+  for (int j = 0; j < IPT; ++j) {
+    const int e = j * T + threadIdx.x;
+    mem[j] = false;
+    bin[j] = 0u;
+    if (e >= tr.y) continue;
     const long long g = (long long)tr.x + e;
     const long long slot = H.offset + (g - H.gbase);
     long long pi = slot;
@@ -501,37 +889,46 @@ __global__ void __launch_bounds__(T) g_prepare_f64(GridLaunch L) {
         rec[2 * g] = a;
         rec[2 * g + 1] = b;
         key = key_of(r);
-        mxm = max(mxm, abs_bits(m));
-        mxr = max(mxr, abs_bits(m * rinv_real(r, P)));
-#pragma unroll
-        for (int q = 0; q < 3; ++q) mxv = max(mxv, abs_bits(mul_rn(m, v[q])));
+        mem[j] = true;
+        if (BINS && th > 1) {
+          bin[j] = part_of(bin_key(r), BM, h0) / PARTS;
+          rk[j] = bin_rank_now(cnt, nb, bin[j]);
+        }
+        mx.add(P, L.p.m != nullptr, m, r, v);
         ++nmem;
       }
     }
     if (L.out.removed_iter) L.out.removed_iter[slot] = key == ~0ull ? -1 : 0;
-    key_a[g] = key;
-    atomicAdd(&h0[(uint32_t)key & 0xffu], 1u);
-    orb |= key;
-    andb &= key;
+    if (!BINS) {
+      key_a[g] = key;
+      atomicAdd(&h0[(uint32_t)key & 0xffu], 1u);
+      orb |= key;
+      andb &= key;
+    }
   }
-  __syncthreads();
-  store_low_byte_hist(L, t, k, h0);
-  for (int o = 16; o > 0; o >>= 1) {
-    orb |= __shfl_xor_sync(FULL_MASK, orb, o);
-    andb &= __shfl_xor_sync(FULL_MASK, andb, o);
-    mxm = max(mxm, __shfl_xor_sync(FULL_MASK, mxm, o));
-    mxr = max(mxr, __shfl_xor_sync(FULL_MASK, mxr, o));
-    mxv = max(mxv, __shfl_xor_sync(FULL_MASK, mxv, o));
+  if (BINS) {
+    bin_ranks<IPT>(cnt, nb, mem, bin, rk, scnt);
+    store_ranks<IPT>(L, tr, mem, rk);
+  } else {
+    __syncthreads();
+    store_low_byte_hist(L, t, k, h0);
   }
+  if (!BINS) {
+    for (int o = 16; o > 0; o >>= 1) {
+      orb |= __shfl_xor_sync(FULL_MASK, orb, o);
+      andb &= __shfl_xor_sync(FULL_MASK, andb, o);
+    }
+  }
+  unsigned long long mxm, mxr, mxv;
+  mx.warp(P, L.p.m != nullptr, L.p, nmem, mxm, mxr, mxv);
   nmem = __reduce_add_sync(FULL_MASK, nmem);
-  merge_prepare(L, k, orb, andb, mxm, mxr, mxv, nmem);
+  if (BINS) merge_prepare(L, k, 0ull, ~0ull, mxm, mxr, mxv, nmem);
+  else merge_prepare(L, k, orb, andb, mxm, mxr, mxv, nmem);
 }
 
+// The scales of a halo's exact sums and the start of its bookkeeping.
 template <typename R>
-__global__ void g_scales(GridLaunch L) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= L.n_halos) return;
-  GridHaloState& s = L.state[k];
+__device__ __forceinline__ void halo_scales(GridHaloState& s) {
   const long long n = s.n_member;
   s.s_m = acc_scale<R>(exp_of_bits(s.mass_max_bits, R()), n);
   s.s_mr = acc_scale<R>(exp_of_bits(s.mr_max_bits, R()), n);
@@ -543,6 +940,114 @@ __global__ void g_scales(GridLaunch L) {
   s.part_iter = 0;
   s.band = 0;
   s.k_first = 0x7fffffffffffffffll;
+}
+
+template <typename R>
+__global__ void g_scales(GridLaunch L) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < L.n_halos) halo_scales<R>(L.state[k]);
+}
+
+// One CTA per halo: the first position of each of its bins (the exclusive
+// prefix of their counts), and its scales.
+template <typename R>
+__global__ void __launch_bounds__(T) g_bin_base(GridLaunch L) {
+  __shared__ uint32_t red[NWARP];
+  __shared__ uint32_t carry;
+  const int k = blockIdx.x;
+  const int b0 = 2 * L.halo_tile0[k], b1 = b0 + halo_bins(L.halo_tile0[k + 1] - L.halo_tile0[k]);
+  if (threadIdx.x == 0) {
+    carry = 0u;
+    halo_scales<R>(L.state[k]);
+  }
+  // four consecutive bins per thread and round
+  for (int b = b0; b < b1; b += 4 * T) {
+    uint32_t v[4], s = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int i = b + 4 * (int)threadIdx.x + j;
+      v[j] = i < b1 ? L.bin_n[(size_t)i * BIN_PAD] : 0u;
+      s += v[j];
+    }
+    uint32_t run = block_excl(s, red) + carry;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int i = b + 4 * (int)threadIdx.x + j;
+      if (i < b1) L.bin_at[i] = run;
+      run += v[j];
+    }
+    __syncthreads();
+    if (threadIdx.x == T - 1) carry = run;
+    __syncthreads();
+  }
+}
+
+// 32 bytes to one sector (a 32-byte aligned address) as one store.
+__device__ __forceinline__ void store_sector(void* p, float4 a, float4 b) {
+  unsigned long long g;
+  asm("cvta.to.global.u64 %0, %1;" : "=l"(g) : "l"(p));
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(g), "f"(a.x), "f"(a.y), "f"(a.z), "f"(a.w),
+               "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
+               : "memory");
+}
+
+// A member's record by bin: (w, r) and (v, candidate position).
+__device__ __forceinline__ void put_binned(const GridLaunch& L, long long dst, float4 a, float4 b, uint32_t pos) {
+  b.w = __uint_as_float(pos);
+  store_sector((float4*)L.rec_b + 2 * dst, a, b);
+}
+__device__ __forceinline__ void put_binned(const GridLaunch& L, long long dst, D4 a, D4 b, uint32_t pos) {
+  b.w = __longlong_as_double((long long)pos);
+  D4* r = (D4*)L.rec_b + 2 * dst;
+  r[0] = a;
+  r[1] = b;
+}
+__device__ __forceinline__ uint32_t binned_pos(float x) { return __float_as_uint(x); }
+__device__ __forceinline__ uint32_t binned_pos(double x) { return (uint32_t)__double_as_longlong(x); }
+
+// Each member of a candidate tile to its bin: the bin's first position plus
+// its rank.
+template <typename R>
+__global__ void __launch_bounds__(T, sizeof(R) == 4 ? 4 : 2) g_place(GridLaunch L) {
+  using V4 = typename Prec<R>::V4;
+  __shared__ uint32_t tab[CELLS + 1];
+  if (bins_overflowed(L)) return;
+  const int t = blockIdx.x;
+  const int2 tr = L.tile_range[t];
+  const int k = L.tile_halo[t];
+  const long long gb = L.halos[k].gbase;
+  const int t0 = L.halo_tile0[k], th = L.halo_tile0[k + 1] - t0;
+  const BinMap BM = load_bin_map(L, k, t0, L.halos[k].count, th, tab);
+  const V4* __restrict__ rec = (const V4*)L.rec;
+  // batches of GB candidates, every load of a batch issued before its first use
+  constexpr int GB = sizeof(R) == 4 ? 4 : 2;
+  uint32_t rk[IPT];
+#pragma unroll
+  for (int q = 0; q < IPT; ++q) {
+    const int e = q * T + threadIdx.x;
+    rk[q] = e < tr.y ? L.rank[(size_t)tr.x + e] : NO_RANK;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int b = 0; b < IPT; b += GB) {
+    V4 ra[GB], rq[GB];
+#pragma unroll
+    for (int j = 0; j < GB; ++j) {
+      if (rk[b + j] != NO_RANK) {
+        const long long g = (long long)tr.x + (b + j) * T + threadIdx.x;
+        ra[j] = rec[2 * g];
+        rq[j] = rec[2 * g + 1];
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < GB; ++j) {
+      if (rk[b + j] == NO_RANK) continue;
+      const uint32_t bn = th > 1 ? part_of(bin_key(ra[j].w), BM, tab) / PARTS : 0u;
+      const long long dst = gb + L.bin_at[2 * t0 + bn] + rk[b + j];
+      if (L.ms) ((R*)L.ms_b)[dst] = rq[j].w;
+      put_binned(L, dst, ra[j], rq[j], (uint32_t)((long long)tr.x + (b + j) * T + threadIdx.x - gb));
+    }
+  }
 }
 
 // ---- segmented radix sort ------------------------------------------------------------
@@ -866,6 +1371,63 @@ __device__ __forceinline__ void atomic_acc(AccSlot& s, __int128 v) {
   atomicAdd((unsigned long long*)&s.w[1], hi + carry);
 }
 
+// The same on a plain array of sums.
+__device__ __forceinline__ void atomic_add_acc(long long* p, long long v) {
+  atomicAdd((unsigned long long*)p, (unsigned long long)v);
+}
+__device__ __forceinline__ void atomic_add_acc(__int128* p, __int128 v) { atomic_acc(*(AccSlot*)p, v); }
+
+// The map of a halo of one bin, from its own keys: 256 cells between the
+// extreme keys, parts by the cells' counts.  `cell`: 256 zeroed words, left zero.
+template <typename Key, int NE>
+__device__ __forceinline__ BinMap one_bin_map(const Key key[NE], int n, uint32_t* cell, uint32_t* tab, uint32_t* red) {
+  __shared__ uint32_t ext[2];
+  __shared__ uint32_t total;
+  if (threadIdx.x == 0) {
+    ext[0] = 0x7f800000u;
+    ext[1] = 0u;
+  }
+  __syncthreads();
+  uint32_t a = 0x7f800000u, b = 0u;
+#pragma unroll
+  for (int j = 0; j < NE; ++j) {
+    if (j * T + (int)threadIdx.x < n) {
+      const uint32_t x = bin_key(radius_of_key(key[j]));
+      a = min(a, x);
+      b = max(b, x);
+    }
+  }
+  a = __reduce_min_sync(FULL_MASK, a);
+  b = __reduce_max_sync(FULL_MASK, b);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(&ext[0], a);
+    atomicMax(&ext[1], b);
+  }
+  __syncthreads();
+  BinMap M;
+  M.k0 = ext[0];
+  M.kx = 0xffffffffu;                    // no tails
+  M.tb = 0u;
+  M.main = PARTS;
+  M.cells = 256;
+  const uint32_t range = ext[1] > ext[0] ? ext[1] - ext[0] : 0u;
+  M.sh = max(0, 24 - __clz(max(range, 1u)));             // 256 << sh > range
+  M.gs = 0;
+#pragma unroll
+  for (int j = 0; j < NE; ++j)
+    if (j * T + (int)threadIdx.x < n) atomicAdd(&cell[(bin_key(radius_of_key(key[j])) - M.k0) >> M.sh], 1u);
+  __syncthreads();
+  const uint32_t w = 16u * cell[threadIdx.x] + 1u;
+  cell[threadIdx.x] = 0u;
+  const uint32_t base = block_excl(w, red);
+  if (threadIdx.x == 255) total = base + w;
+  __syncthreads();
+  tab[threadIdx.x] = (PARTS * TAB_UNIT * base) / total;  // base <= 16 BIN_MAX + 256
+  if (threadIdx.x == 0) tab[256] = PARTS * TAB_UNIT;
+  __syncthreads();
+  return M;
+}
+
 // v_bulk = sum m v / sum m of the current set, into the halo state.
 template <typename R>
 __device__ __forceinline__ void set_vbulk(GridHaloState& S, typename Prec<R>::Acc m,
@@ -968,7 +1530,7 @@ __global__ void __launch_bounds__(HT) g_halo(GridLaunch L, int pass) {
   __shared__ int s_kept;                   // sub-tiles of the halo on the next list
   const int k = blockIdx.x;
   GridHaloState& S = L.state[k];
-  if (!INIT && !S.active) return;
+  if (INIT ? bins_overflowed(L) : !S.active) return;
   const int n_sub = L.n_tiles * SPT;
   const int cp = (pass + 1) & 1;
   const Acc* am = (const Acc*)L.agg_m + (size_t)cp * n_sub;
@@ -1217,6 +1779,163 @@ __global__ void __launch_bounds__(HT) g_halo(GridLaunch L, int pass) {
   }
 }
 
+// A bin ordered, one CTA each: its members counted in the bin's 512 parts in
+// shared memory, their keys moved there, and each member's place in its part
+// found by counting the members before it in (r, candidate).  Then, in
+// radial order, the streams (w, r), (v, m), the position (and mass, thermal
+// energy), the exact sum m v, and the sub-tiles' sums of the initial set.
+template <typename R>
+__global__ void __launch_bounds__(T, 3) g_bin_sort(GridLaunch L) {
+  using V4 = typename Prec<R>::V4;
+  using Key = typename Prec<R>::Key;
+  using Acc = typename Prec<R>::Acc;
+  constexpr int NE = BIN_MAX / T;        // members per thread
+  extern __shared__ __align__(16) unsigned char dyn[];
+  Key* skey = reinterpret_cast<Key*>(dyn);                       // [BIN_MAX]
+  uint16_t* sidx = reinterpret_cast<uint16_t*>(skey + BIN_MAX);  // [BIN_MAX] slot -> source
+  uint16_t* sout = sidx + BIN_MAX;                               // [BIN_MAX] place -> source
+  uint16_t* spart = sout + BIN_MAX;                              // [BIN_MAX] slot -> part
+  __shared__ uint32_t tab[CELLS + 1];
+  __shared__ uint32_t pcnt[PARTS + 1];
+  __shared__ uint32_t red[NWARP];
+  __shared__ Acc racc[NWARP];
+  // (another CTA may set the word meanwhile: one decision for the CTA)
+  if (__syncthreads_or(bins_overflowed(L))) return;
+  const int bin = blockIdx.x, t = bin >> 1;
+  const int k = L.tile_halo[t];
+  const HaloDev& H = L.halos[k];
+  const GridHaloState& S = L.state[k];
+  const int t0 = L.halo_tile0[k], th = L.halo_tile0[k + 1] - t0;
+  if (th == 1 && (bin & 1)) return;      // one bin
+  const int n = (int)L.bin_n[(size_t)bin * BIN_PAD];
+  BinMap BM;
+  if (th > 1) BM = load_bin_map(L, k, t0, H.count, th, tab);
+  pcnt[threadIdx.x] = 0u;
+  pcnt[threadIdx.x + T] = 0u;
+  Acc smv[3] = {0, 0, 0};
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t at = L.bin_at[bin];
+  const long long g0 = H.gbase + at;     // first flat position of the bin
+  const V4* __restrict__ rb = (const V4*)L.rec_b + 2 * g0;
+  uint32_t slot[NE];                     // part << 16 | rank of arrival in it
+  {
+    Key key[NE];
+#pragma unroll
+    for (int j = 0; j < NE; ++j) {
+      if (j * T >= n) break;
+      const int i = j * T + threadIdx.x;
+      if (i < n) key[j] = key_of(rb[2 * i].w);
+    }
+    __syncthreads();
+    if (th == 1) BM = one_bin_map<Key, NE>(key, n, pcnt, tab, red);
+    const uint32_t first = (uint32_t)PARTS * (uint32_t)(bin - 2 * t0);
+#pragma unroll
+    for (int j = 0; j < NE; ++j) {
+      if (j * T >= n) break;
+      const int i = j * T + threadIdx.x;
+      if (i < n) {
+        const uint32_t q = min(part_of(bin_key(radius_of_key(key[j])), BM, tab) - first, (uint32_t)PARTS - 1u);
+        slot[j] = (q << 16) | atomicAdd(&pcnt[q], 1u);
+      }
+    }
+    __syncthreads();
+    const uint32_t v0 = pcnt[2 * threadIdx.x], v1 = pcnt[2 * threadIdx.x + 1];
+    if (max(v0, v1) > PART_MAX) L.ctl->overflow = 1;
+    const uint32_t ex = block_excl(v0 + v1, red);
+    __syncthreads();
+    pcnt[2 * threadIdx.x] = ex;
+    pcnt[2 * threadIdx.x + 1] = ex + v0;
+    if (threadIdx.x == T - 1) pcnt[PARTS] = ex + v0 + v1;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < NE; ++j) {
+      if (j * T >= n) break;
+      const int i = j * T + threadIdx.x;
+      if (i < n) {
+        const uint32_t q = pcnt[slot[j] >> 16] + (slot[j] & 0xffffu);
+        skey[q] = key[j];
+        sidx[q] = (uint16_t)i;
+        spart[q] = (uint16_t)(slot[j] >> 16);
+      }
+    }
+  }
+  __syncthreads();
+  // in slot order: a warp's members are in neighbouring parts
+  for (int own = threadIdx.x; own < n; own += T) {
+    const uint32_t p = spart[own];
+    const uint32_t a = pcnt[p], z = pcnt[p + 1];
+    if (z - a > PART_MAX) continue;      // the overflow word is set: nothing of this attempt is used
+    const Key key = skey[own];
+    uint32_t q = a, ties = 0u;
+    for (uint32_t x = a; x < z; ++x) {
+      const Key kx = skey[x];
+      q += kx < key ? 1u : 0u;
+      ties += kx == key ? 1u : 0u;
+    }
+    const uint32_t ip = sidx[own];
+    if (ties > 1u) {                     // equal radii: in candidate order
+      const uint32_t pos = binned_pos(rb[2 * ip + 1].w);
+      for (uint32_t x = a; x < z; ++x)
+        if (skey[x] == key && binned_pos(rb[2 * (uint32_t)sidx[x] + 1].w) < pos) ++q;
+    }
+    sout[q] = (uint16_t)ip;
+  }
+  __syncthreads();
+  // the streams in radial order, a warp taking rows of 32; sums by sub-tile
+  const int s_m = S.s_m, s_r = S.s_mr, s_v = S.s_mv;
+  const R m0 = sizeof(R) == 4 ? (R)L.p.m0f : (R)L.p.m0;
+  const Acc mfix0 = fixp(m0, s_m);
+  V4* vr = (V4*)L.vr;
+  const size_t sub0 = (size_t)L.n_tiles * SPT + (size_t)t0 * SPT;   // copy 1
+  // rows aligned to 32 positions of the halo, so that none straddles two sub-tiles
+  const int lead = (int)(at & 31u);
+  const int rows = (n + lead + 31) >> 5;
+  for (int row = warp; row < rows; row += NWARP) {
+    const int e = row * 32 - lead + lane;
+    const bool in = e >= 0 && e < n;
+    Acc a = 0, b = 0;
+    if (in) {
+      const int i = sout[e];
+      const V4 x = rb[2 * i];
+      V4 y = rb[2 * i + 1];
+      const uint32_t p = binned_pos(y.w);
+      const long long dst = g0 + e;
+      const R m = L.ms ? ((const R*)L.ms_b)[g0 + i] : m0;
+      y.w = m;
+      ((V4*)L.wr)[dst] = x;
+      vr[dst] = y;
+      L.val_x[dst] = p;
+      if (L.ms) ((R*)L.ms)[dst] = m;
+      if (L.uth) {
+        const long long slot = H.offset + p;
+        const long long pi = L.out.member_idx ? L.out.member_idx[slot] : slot;
+        ((R*)L.uth)[dst] = (R)(L.p.coord_type == AHF_COORD_F64 ? __ldg((const double*)L.p.u_th + pi)
+                                                               : (double)__ldg((const float*)L.p.u_th + pi));
+      }
+      a = L.ms ? (Acc)fixp(m, s_m) : mfix0;
+      b = fixp(m * rinv_real(x.w, L.prm), s_r);
+      smv[0] += fixr(mul_rn(m, y.x), s_v);
+      smv[1] += fixr(mul_rn(m, y.y), s_v);
+      smv[2] += fixr(mul_rn(m, y.z), s_v);
+    }
+    const int c = __popc(__ballot_sync(FULL_MASK, in));
+    if (L.ms) a = wsum(a);
+    else a = mfix0 * (Acc)c;
+    b = wsum(b);
+    if (lane == 0 && c) {
+      const size_t u = sub0 + ((at + (uint32_t)max(row * 32 - lead, 0)) / SUB);
+      atomic_add_acc((Acc*)L.agg_m + u, a);
+      atomic_add_acc((Acc*)L.agg_r + u, b);
+      atomicAdd(&L.agg_c[u], c);
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const Acc x = block_sum(smv[a], racc);
+    if (threadIdx.x == 0) atomic_acc(L.tile_mv[3 * (size_t)t + a], x);
+  }
+}
+
 // ---- one unbinding pass -----------------------------------------------------------------
 
 constexpr int EPL = SUB / 32;            // 8 consecutive elements per lane
@@ -1418,6 +2137,7 @@ __global__ void __launch_bounds__(T) g_removed(GridLaunch L, int pass) {
   const int4* list = L.work + (size_t)(pass & 1) * L.n_tiles * SPT;
   V4* wr = (V4*)L.wr;
   const V4* rec = (const V4*)L.rec;
+  const V4* vr = (const V4*)L.vr;        // radial order, or NULL (radix sort): by candidate
   const R m0 = sizeof(R) == 4 ? (R)L.p.m0f : (R)L.p.m0;
   // 32 listed sub-tiles per step: lane j checks entry i0 + j's flags (32
   // bytes), then the warp takes the flagged ones one after another
@@ -1457,7 +2177,7 @@ __global__ void __launch_bounds__(T) g_removed(GridLaunch L, int pass) {
       V4 vm[EPL];
 #pragma unroll
       for (int e = 0; e < EPL; ++e)
-        if ((rem >> e) & 1u) vm[e] = rec[2 * (H.gbase + pos[e]) + 1];  // (v, m) of the candidate
+        if ((rem >> e) & 1u) vm[e] = vr ? vr[g0 + e] : rec[2 * (H.gbase + pos[e]) + 1];  // (v, m)
 #pragma unroll
       for (int e = 0; e < EPL; ++e) {
         if (!((rem >> e) & 1u)) continue;
@@ -1913,16 +2633,62 @@ __global__ void __launch_bounds__(T) g_rows_f64(GridLaunch L) {
 
 inline int blocks_for(int n, int b) { return (n + b - 1) / b; }
 
+template <typename R, bool BINS>
+void launch_prepare(const GridLaunch& L, cudaStream_t s) {
+  const bool f64 = L.p.coord_type == AHF_COORD_F64;
+  if constexpr (sizeof(R) == 4) {
+    if (f64) g_prepare_mixed<AHF_COORD_F64, BINS><<<L.n_tiles, T, 0, s>>>(L);
+    else g_prepare_mixed<AHF_COORD_F32_REL, BINS><<<L.n_tiles, T, 0, s>>>(L);
+  } else {
+    if (f64) g_prepare_f64<AHF_COORD_F64, BINS><<<L.n_tiles, T, 0, s>>>(L);
+    else g_prepare_f64<AHF_COORD_F32_REL, BINS><<<L.n_tiles, T, 0, s>>>(L);
+  }
+}
+
+template <typename R>
+void launch_halo_init(const GridLaunch& L, cudaStream_t s) {
+  if (L.max_halo_tiles > 64) g_halo<R, true, HT_BIG><<<L.n_halos, HT_BIG, 0, s>>>(L, 0);
+  else g_halo<R, true, HT_SMALL><<<L.n_halos, HT_SMALL, 0, s>>>(L, 0);
+}
+
+// The distribution into radial bins (see g_sample).
+template <typename R>
+cudaError_t bins_t(GridLaunch& L, cudaStream_t s) {
+  L.sort_passes = 0;
+  L.sort_launches = 0;
+  if (L.n_tiles == 0) {
+    g_scales<R><<<blocks_for(L.n_halos, 128), 128, 0, s>>>(L);
+    L.sort_launches = 1;
+    return cudaGetLastError();
+  }
+  constexpr size_t smem = (size_t)BIN_MAX * (sizeof(typename Prec<R>::Key) + 6);
+  static std::atomic<unsigned long long> attrs_set{0};
+  cudaError_t e = cudaSuccess;
+  if (first_use_on_device(attrs_set)) {
+    e = cudaFuncSetAttribute(g_bin_sort<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    mark_used_on_device(attrs_set);
+  }
+  if (L.max_halo_tiles > 1) {
+    const int shares = std::min(L.max_halo_tiles, SAMPLE_MAX / T);
+    const bool by_halo = L.n_halos > 1 && L.n_halos <= 65535 && (long long)shares * L.n_halos < L.n_tiles;
+    const dim3 grid = by_halo ? dim3((unsigned)shares, (unsigned)L.n_halos) : dim3((unsigned)L.n_tiles);
+    if (L.p.coord_type == AHF_COORD_F64) g_sample<R, AHF_COORD_F64><<<grid, T, 0, s>>>(L);
+    else g_sample<R, AHF_COORD_F32_REL><<<grid, T, 0, s>>>(L);
+    g_bin_map<<<L.n_halos, SAMPLE_T, 0, s>>>(L);
+  }
+  launch_prepare<R, true>(L, s);
+  g_bin_base<R><<<L.n_halos, T, 0, s>>>(L);
+  g_place<R><<<L.n_tiles, T, 0, s>>>(L);
+  g_bin_sort<R><<<2 * L.n_tiles, T, smem, s>>>(L);
+  launch_halo_init<R>(L, s);
+  L.sort_launches = 5 + (L.max_halo_tiles > 1 ? 2 : 0);
+  return cudaGetLastError();
+}
+
 template <typename R>
 cudaError_t prepare_t(const GridLaunch& L, cudaStream_t s) {
-  if (L.n_tiles == 0) {
-  } else if (sizeof(R) == 4) {
-    if (L.p.coord_type == AHF_COORD_F64) g_prepare_mixed<AHF_COORD_F64><<<L.n_tiles, T, 0, s>>>(L);
-    else g_prepare_mixed<AHF_COORD_F32_REL><<<L.n_tiles, T, 0, s>>>(L);
-  } else {
-    if (L.p.coord_type == AHF_COORD_F64) g_prepare_f64<AHF_COORD_F64><<<L.n_tiles, T, 0, s>>>(L);
-    else g_prepare_f64<AHF_COORD_F32_REL><<<L.n_tiles, T, 0, s>>>(L);
-  }
+  if (L.n_tiles > 0) launch_prepare<R, false>(L, s);
   g_scales<R><<<blocks_for(L.n_halos, 128), 128, 0, s>>>(L);
   return cudaGetLastError();
 }
@@ -1967,8 +2733,7 @@ cudaError_t sort_t(GridLaunch& L, cudaStream_t s, unsigned long long or_bits, un
   if (nd == 0) g_fill_identity<R><<<L.n_tiles, T, 0, s>>>(L);
   L.sort_launches += (nd == 0 ? 1 : 0) + 2;
   g_sums<R><<<(int)(((long long)L.n_tiles * SPT + NWARP - 1) / NWARP), T, 0, s>>>(L);
-  if (L.max_halo_tiles > 64) g_halo<R, true, HT_BIG><<<L.n_halos, HT_BIG, 0, s>>>(L, 0);
-  else g_halo<R, true, HT_SMALL><<<L.n_halos, HT_SMALL, 0, s>>>(L, 0);
+  launch_halo_init<R>(L, s);
   return cudaGetLastError();
 }
 
@@ -2057,6 +2822,8 @@ bool grid_wr_map(GridLaunch& L, long long n_rows) {
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+
+cudaError_t grid_bins(GridLaunch& L, cudaStream_t s) { return L.fp64 ? bins_t<double>(L, s) : bins_t<float>(L, s); }
 
 cudaError_t grid_prepare(const GridLaunch& L, cudaStream_t s) {
   return L.fp64 ? prepare_t<double>(L, s) : prepare_t<float>(L, s);

@@ -96,11 +96,11 @@ struct GridHaloState {
   int status;
   int active;
   int s_m, s_mr, s_mv;               // fixed-point scales
-  int pad0, pad;
+  uint32_t bin_k0, bin_kx;           // radius keys where the halo's bin cells start and end
   AccSlot rem_mv[3];                 // exact sum m v of what the current pass removed
   long long band_pass;               // band tests of the current pass
   float vbulk[3];                    // v_bulk of the current set (mixed precision)
-  float pad2;
+  int bin_shifts;                    // log2 of the cells' width, then << 8 of the first tail's
   double vbulk_d[3];                 // v_bulk of the current set (all-FP64 mode)
   AccSlot m_init;                    // exact sum of the members' masses (before any pass)
   double mrem;                       // mass the halo lost before the current pass
@@ -123,7 +123,8 @@ struct SkipRec {
 // Device control words of one multi-CTA call.
 struct GridCtl {
   int work_n[2];                     // sub-tiles to process in the passes of each parity
-  int pad0[2];
+  int overflow;                      // a radial bin would hold more members than it can
+  int pad0;
   unsigned long long key_or, key_and;  // OR and AND of every radius key
   int pad[8];
 };
@@ -203,6 +204,16 @@ struct GridLaunch {
                            // as float4 / 4 doubles, by candidate position
   void *key_a, *key_b;     // radius keys: uint32 / uint64
   uint32_t *val_a, *val_b; // candidate positions riding along the sort
+  // the distribution into radial bins; these overlay arrays not in use then
+  uint16_t* rank;          // rank of arrival in the bin per candidate
+  void* rec_b;             // 2 per member, by bin: (w, r), (v, candidate position)
+  void* ms_b;              // masses by bin
+  uint32_t *bin_n, *bin_at;  // per bin (two per tile): members (a 128-byte line each, in
+                           // tile_hist), first position in the halo
+  void* vr;                // radial order: (v, m); NULL after the radix sort (then by
+                           // candidate, in rec)
+  void *wr_bins, *vr_bins; // wr and vr after the bins (in rec, which the bins are done with)
+  void* wr_radix;          // wr after the radix sort
   void* wr;                // radial order: (w.x, w.y, w.z, r), r's sign bit = removed
   void* ms;                // radial order masses (float / double), NULL for a uniform mass
   void* uth;               // gas: thermal energy in radial order (float / double), or NULL
@@ -214,7 +225,8 @@ struct GridLaunch {
   int2* tile_range;        // (first flat index, length)
   int* tile_halo;
   int* halo_tile0;         // first tile of each halo (n_halos + 1)
-  uint32_t* tile_hist;     // n_tiles * 256, per halo digit-major
+  uint32_t* tile_hist;     // n_tiles * 256: bin counts and bin tables (radix sort: digit
+                           // counts, per halo digit-major)
   uint32_t* digit_base;    // n_halos * 256
   int* big_halos;          // haloes of more than 256 tiles (digit scans spread over CTAs)
   int n_big;
@@ -236,8 +248,8 @@ struct GridLaunch {
                            // haloes for the passes of each parity: (sub-tile, halo, first
                            // flat element, members in it)
   int iter_grid;           // CTAs of the persistent iteration pass
-  int sort_passes;         // radix passes the last grid_sort launched
-  int sort_launches;       // and its kernel launches
+  int sort_passes;         // radix passes the last grid_sort launched (0: bins)
+  int sort_launches;       // kernel launches of the last grid_bins or grid_sort
   ProfileRows rows;        // rows.prof != NULL: profile rows from the final pass
 };
 
@@ -252,6 +264,10 @@ int grid_tma_grid(int device);
 // Fill L.wr_map for the stream L.wr of n_rows 8-element rows; false if the
 // tensor map cannot be made (the passes then read the stream directly).
 bool grid_wr_map(GridLaunch &L, long long n_rows);
+// The radial order by distribution into bins: gather, streams, sums of the
+// initial set.  Sets ctl->overflow (and leaves no halo active) when a bin
+// cannot hold its members; then grid_reset, grid_prepare and grid_sort.
+cudaError_t grid_bins(GridLaunch &L, cudaStream_t s);
 cudaError_t grid_prepare(const GridLaunch &L, cudaStream_t s);
 // Radix passes over the bits where the keys differ (or_bits ^ and_bits);
 // the last pass also lays out the radial-order streams.  Then the sums of
