@@ -1469,23 +1469,32 @@ int hier_impl(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64_t
   if ((rc = validate_slots(halos, n_halos, n_slots, member_idx != nullptr))) return rc;
   // scratch outside the workspace (the levels' unbinding calls lay that out anew)
   Bump sz{nullptr, 0, 0};
-  auto layout = [&](Bump& B, HierLaunch* L, int** lvl, int** anc) {
+  // chunks of the largest level
+  std::vector<int64_t> level_chunks((size_t)max_depth + 1, 0);
+  for (int64_t h = 0; h < n_halos; ++h)
+    level_chunks[(size_t)depth[(size_t)h]] += std::max<int64_t>(1, (halos[h].count + HIER_CHUNK - 1) / HIER_CHUNK);
+  const int64_t max_chunks = *std::max_element(level_chunks.begin(), level_chunks.end());
+  if (max_chunks >= (1ll << 31)) return fail(AHF_ERR_INVALID, "a level above 2^31 chunks");
+  // per level, one upload: its haloes, every halo's ancestor, the chunks
+  const size_t n_tab = 2 * (size_t)n_halos + 2 * (size_t)max_chunks;
+  int* d_tab = nullptr;
+  auto layout = [&](Bump& B, HierLaunch* L) {
     long long* owner = B.take<long long>((size_t)std::max<int64_t>(p->n, 1));
     long long* mem = B.take<long long>((size_t)std::max<int64_t>(n_slots, 1));
     long long* cmap = B.take<long long>((size_t)std::max<int64_t>(n_slots, 1));
     int* rem = B.take<int>((size_t)std::max<int64_t>(n_slots, 1));
     ahf_result* rl = B.take<ahf_result>((size_t)n_halos);
     ahf_halo* hd = B.take<ahf_halo>((size_t)n_halos);
-    int* lv = B.take<int>((size_t)n_halos);
-    int* an = B.take<int>((size_t)n_halos);
+    int* tab = B.take<int>(n_tab);
+    int* ck = B.take<int>((size_t)max_chunks);
     long long* kept = B.take<long long>((size_t)n_halos);
     if (L) {
       L->owner = owner; L->members = mem; L->cand_map = cmap; L->rem_level = rem; L->res_level = rl;
-      L->halos = hd; L->level = lv; L->anc = an; L->kept = kept;
-      *lvl = lv; *anc = an;
+      L->halos = hd; L->kept = kept; L->chunk_kept = ck;
+      d_tab = tab;
     }
   };
-  layout(sz, nullptr, nullptr, nullptr);
+  layout(sz, nullptr);
   if (sz.used + 4096 > c->hier_bytes) {
     if (c->last_valid) AHF_CUDA(cudaEventSynchronize(c->last));
     if (c->hier) cudaFree(c->hier);
@@ -1499,9 +1508,7 @@ int hier_impl(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64_t
   }
   Bump B{(char*)c->hier, 0, c->hier_bytes};
   HierLaunch L{};
-  int* d_level = nullptr;
-  int* d_anc = nullptr;
-  layout(B, &L, &d_level, &d_anc);
+  layout(B, &L);
   L.member_idx = (const long long*)member_idx;
   L.n_particles = p->n;
   L.res = out;
@@ -1511,7 +1518,7 @@ int hier_impl(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64_t
   if (c->last_valid) AHF_CUDA(cudaStreamWaitEvent(s, c->last, 0));
   if (p->n) AHF_CUDA(cudaMemsetAsync(L.owner, 0xff, sizeof(long long) * (size_t)p->n, s));
   AHF_CUDA(cudaMemcpyAsync((void*)L.halos, halos, sizeof(ahf_halo) * (size_t)n_halos, cudaMemcpyHostToDevice, s));
-  std::vector<int> level, anc((size_t)n_halos);
+  std::vector<int> level, tab;
   std::vector<long long> kept;
   std::vector<ahf_halo> lh;
   int64_t launches = 0, syncs = 0;
@@ -1520,16 +1527,31 @@ int hier_impl(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64_t
     for (int64_t h = 0; h < n_halos; ++h)
       if (depth[(size_t)h] == d) level.push_back((int)h);
     if (level.empty()) continue;
+    const int nl = (int)level.size();
+    const size_t nc = (size_t)level_chunks[(size_t)d];
+    tab.resize((size_t)nl + (size_t)n_halos + 2 * nc);
+    std::copy(level.begin(), level.end(), tab.begin());
+    int* anc = tab.data() + nl;
     for (int64_t t = 0; t < n_halos; ++t) {
       int64_t a = t;
       while (a >= 0 && depth[(size_t)a] > d) a = parent[a];
-      anc[(size_t)t] = depth[(size_t)t] > d ? (int)a : -1;
+      anc[t] = depth[(size_t)t] > d ? (int)a : -1;
     }
-    const int nl = (int)level.size();
-    AHF_CUDA(cudaMemcpyAsync(d_level, level.data(), sizeof(int) * (size_t)nl, cudaMemcpyHostToDevice, s));
-    AHF_CUDA(cudaMemcpyAsync(d_anc, anc.data(), sizeof(int) * (size_t)n_halos, cudaMemcpyHostToDevice, s));
+    int *cl = anc + n_halos, *co = cl + nc;
+    for (int i = 0; i < nl; ++i) {
+      const int64_t n = std::max<int64_t>(1, (halos[level[(size_t)i]].count + HIER_CHUNK - 1) / HIER_CHUNK);
+      for (int64_t o = 0; o < n; ++o) {
+        *cl++ = i;
+        *co++ = (int)o;
+      }
+    }
+    AHF_CUDA(cudaMemcpyAsync(d_tab, tab.data(), sizeof(int) * tab.size(), cudaMemcpyHostToDevice, s));
+    L.level = d_tab;
+    L.anc = d_tab + nl;
+    L.chunk_level = L.anc + n_halos;
+    L.chunk_ord = L.chunk_level + nc;
     L.rank = max_depth - d;
-    AHF_CUDA(launch_hier_compact(L, nl, s));
+    AHF_CUDA(launch_hier_compact(L, (int)nc, s));
     kept.assign((size_t)nl, 0);
     AHF_CUDA(cudaMemcpyAsync(kept.data(), L.kept, sizeof(long long) * (size_t)nl, cudaMemcpyDeviceToHost, s));
     AHF_CUDA(cudaStreamSynchronize(s));
@@ -1543,8 +1565,8 @@ int hier_impl(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64_t
                           removed_iter ? (int32_t*)L.rem_level : nullptr, s)))
       return rc;
     launches += c->stats.launches;
-    AHF_CUDA(launch_hier_scatter(L, nl, s));
-    launches += 2;
+    AHF_CUDA(launch_hier_scatter(L, (int)nc, s));
+    launches += 3;
   }
   c->stats.launches = launches;
   c->stats.host_syncs += syncs;

@@ -335,7 +335,7 @@ struct HierLaunch {
   long long *owner;                // [n_particles]: level rank << 32 | halo, -1 none
   const int *anc;                  // [n_halos]: ancestor on this level, -1
   long long *members;              // [n_slots] compacted member lists
-  long long *cand_map;             // [n_slots] compacted position -> candidate slot
+  long long *cand_map;             // [n_slots] candidate slot -> compacted position, -1 dropped
   long long *kept;                 // [n_level] kept candidates
   const ahf_result *res_level;     // [n_level]
   ahf_result *res;                 // caller's records
@@ -343,9 +343,14 @@ struct HierLaunch {
   int *removed_iter;               // caller's, or NULL
   const long long *bound_idx;      // caller's
   int rank;                        // 0 for the deepest level, growing outwards
+  // chunks of HIER_CHUNK candidates of the level's haloes (one at least each):
+  // the halo's position in `level`, the chunk's in the halo, its kept candidates
+  const int *chunk_level, *chunk_ord;
+  int *chunk_kept;
 };
-cudaError_t launch_hier_compact(const HierLaunch &L, int n_level, cudaStream_t s);
-cudaError_t launch_hier_scatter(const HierLaunch &L, int n_level, cudaStream_t s);
+constexpr int HIER_CHUNK = 2048;
+cudaError_t launch_hier_compact(const HierLaunch &L, int n_chunks, cudaStream_t s);
+cudaError_t launch_hier_scatter(const HierLaunch &L, int n_chunks, cudaStream_t s);
 
 // Cross-identification of two catalogues by xi = N_shared^2 / (N_1 N_2).
 constexpr int MATCH_TABLE = 2048;        // distinct second-catalogue haloes one halo may meet
