@@ -705,12 +705,14 @@ struct GridTables {
   std::vector<int> tile_halo;
   std::vector<int> halo_tile0;
   std::vector<int> big;        // haloes of more than 256 tiles
+  int n_cta = 0;               // leading haloes of more than GRID_WARP_TILES tiles
 };
 
 void build_tiles(const Plan& P, int first, int n, GridTables& T) {
   T.tile_range.clear();
   T.tile_halo.clear();
   T.big.clear();
+  T.n_cta = 0;
   T.halo_tile0.assign((size_t)n + 1, 0);
   for (int k = 0; k < n; ++k) {
     const HaloDev& d = P.hd[(size_t)first + k];
@@ -720,7 +722,9 @@ void build_tiles(const Plan& P, int first, int n, GridTables& T) {
       T.tile_range.push_back(make_int2((int)(d.gbase + o), (int)len));
       T.tile_halo.push_back(k);
     }
-    if ((int)T.tile_range.size() - T.halo_tile0[k] > 256) T.big.push_back(k);
+    const int th = (int)T.tile_range.size() - T.halo_tile0[k];
+    if (th > 256) T.big.push_back(k);
+    if (th > GRID_WARP_TILES) T.n_cta = k + 1;           // (largest first)
   }
   T.halo_tile0[n] = (int)T.tile_range.size();
 }
@@ -901,6 +905,7 @@ int unbind_pass(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64
     if ((rc = grid_reset(G, s))) return rc;
     G.p = pd; G.frame = P.frame; G.prm = prd; G.out = O;
     G.iter_grid = grid_pass_ctas(c, fp64);
+    G.n_cta_halos = T.n_cta;
     // profile rows of this class from its final pass
     G.rows.prof = prof;
     G.rows.factor = dfac;
@@ -1235,6 +1240,7 @@ int plain_impl(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64_
     G.n_tiles = (int)tr.size();
     G.n_flat = d.count;
     G.n_big = G.n_tiles > 256 ? 1 : 0;
+    G.n_cta_halos = G.n_tiles > GRID_WARP_TILES ? 1 : 0;
     char* pin = nullptr;
     if ((rc = pin_acquire(c, pin_need, &pin))) return rc;
     size_t po = 0;

@@ -1503,14 +1503,172 @@ __global__ void __launch_bounds__(T) g_sums(GridLaunch L) {
   }
 }
 
+// A halo's bookkeeping, by one thread, after the initial sums (INIT) or after
+// pass `pass`: iterations, particle-iterations, band tests, sum m v, v_bulk,
+// convergence (Sect. 2.1, Appendix A: the loop ends when an iteration removes
+// nothing), from the sums M, Rr and the count C of the set left (mvs: sum m v of
+// the members, INIT only).  Returns whether the halo goes on.
+template <typename R, bool INIT>
+__device__ __forceinline__ int halo_update(const GridLaunch& L, GridHaloState& S, int pass,
+                                           typename Prec<R>::Acc M, typename Prec<R>::Acc Rr, long long C,
+                                           const typename Prec<R>::Acc mvs[3], float vb[3]) {
+  using Acc = typename Prec<R>::Acc;
+  Acc mv[3];
+  int active;
+  if (INIT) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) mv[q] = mvs[q];
+    active = C > 0 ? 1 : 0;
+  } else {
+    const long long alive = S.n_alive;
+    S.part_iter += alive;
+    S.band += S.band_pass;
+    S.band_pass = 0;
+    S.n_iter = pass;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      mv[q] = Ald<Acc>(S.mv[q]) - Ald<Acc>(S.rem_mv[q]);
+      A<Acc>(S.rem_mv[q]) = 0;
+    }
+    active = 1;
+    if (C == alive) {
+      active = 0;
+    } else if (C == 0) {
+      active = 0;
+      S.status |= AHF_HALO_EMPTY;
+    } else if (pass >= L.prm.max_iter) {
+      active = 0;
+      S.status |= AHF_HALO_NOT_CONVERGED;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) A<Acc>(S.mv[q]) = mv[q];
+  A<Acc>(S.m_tot) = M;
+  A<Acc>(S.t_tot) = Rr;
+  S.n_alive = C;
+  if (active && (INIT || !L.prm.vbulk_initial)) set_vbulk<R>(S, M, mv);
+  S.active = active;
+  // the mass lost so far (exact sums), for the skip records and test
+  if (INIT) A<Acc>(S.m_init) = M;
+  S.mrem = INIT ? 0.0 : dfix(Ald<Acc>(S.m_init) - M, S.s_m);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) vb[q] = sizeof(R) == 4 ? S.vbulk[q] : (float)S.vbulk_d[q];
+  return active;
+}
+
+// Whether sub-tile u, last tested as `rc` says, may stay out of the next pass;
+// if so its sums carry over to the copy that pass would have written.  It may
+// while its members can neither be removed nor fall in the band: since that
+// test each member's 2|phi| fell by at most 2 G dM / max(r, r_soft) (the halo
+// lost mass dM, each removed particle's term at most m / r of the member's own
+// radius), and its |u|^2 rose by at most 2 |u| dv + dv^2 (v_bulk moved by dv); the
+// record's margin (slack 2^-16 of 2|phi| for the float rounding of both tests)
+// must exceed that, with 2^-10 more on the bound for its own rounding.
+template <typename R>
+__device__ __forceinline__ bool skips(const GridLaunch& L, int u, int pass, const SkipRec& rc, double mrem, float vb0,
+                                      float vb1, float vb2) {
+  using Acc = typename Prec<R>::Acc;
+  const float dm = (float)(mrem - rc.mrem) * (1.0f + 0x1p-20f);
+  const float reff = fmaxf(rc.rin, L.prm.r_soft_f);
+  const float ax = vb0 - rc.vb[0], ay = vb1 - rc.vb[1], az = vb2 - rc.vb[2];
+  const float vmag =
+      fabsf(vb0) + fabsf(vb1) + fabsf(vb2) + fabsf(rc.vb[0]) + fabsf(rc.vb[1]) + fabsf(rc.vb[2]);
+  const float dv = sqrtf(fmaf(az, az, fmaf(ay, ay, ax * ax))) * (1.0f + 0x1p-20f) + vmag * 0x1p-20f;
+  const float bound =
+      ((2.0f * L.prm.Gf) * dm / reff + dv * fmaf(2.0f, rc.umax, dv)) * (1.0f + 0x1p-10f);
+  if (!(reff > 0.0f && isfinite(bound) && rc.margin > bound)) return false;
+  const size_t n_sub = (size_t)L.n_tiles * SPT;
+  const size_t a = (size_t)((pass + 1) & 1) * n_sub + u, b = (size_t)(pass & 1) * n_sub + u;
+  ((Acc*)L.agg_m)[b] = ((const Acc*)L.agg_m)[a];
+  ((Acc*)L.agg_r)[b] = ((const Acc*)L.agg_r)[a];
+  L.agg_c[b] = L.agg_c[a];
+  return true;
+}
+
+// A halo of at most GRID_WARP_TILES tiles (32 sub-tiles), by one warp, a sub-tile per
+// lane: g_halo's work without a CTA's barriers.  3,000 haloes in FP64 (2,900 of
+// them this small) took 36 us a pass with one CTA each.
+static_assert(GRID_WARP_TILES * SPT == 32, "a sub-tile per lane");
+template <typename R, bool INIT>
+__device__ __forceinline__ void halo_warp(const GridLaunch& L, int k, int pass) {
+  using Acc = typename Prec<R>::Acc;
+  GridHaloState& S = L.state[k];
+  if (!INIT && !S.active) return;
+  const int lane = threadIdx.x & 31;
+  const int n_sub = L.n_tiles * SPT;
+  const size_t cp = (size_t)((pass + 1) & 1) * n_sub;
+  const int t0 = L.halo_tile0[k], th = L.halo_tile0[k + 1] - t0;
+  const int u = t0 * SPT + lane;
+  const long long nm = S.n_member;
+  const int nu = (int)((nm + SUB - 1) / SUB);            // sub-tiles holding members
+  SkipRec rc;
+  if (!INIT && lane < nu) rc = L.skip[u];
+  Acc m = 0, r = 0;
+  int c = 0;
+  if (lane < nu) {
+    m = ((const Acc*)L.agg_m)[cp + u];
+    r = ((const Acc*)L.agg_r)[cp + u];
+    c = L.agg_c[cp + u];
+  }
+  const Acc im = wscan(m, lane), ir = wscan(r, lane);
+  const int ic = (int)wscan((uint32_t)c, lane);
+  if ((lane % SPT) == 0 && lane / SPT < th) {
+    ((Acc*)L.pre_m)[t0 + lane / SPT] = im - m;
+    ((Acc*)L.pre_r)[t0 + lane / SPT] = ir - r;
+    L.pre_c[t0 + lane / SPT] = ic - c;
+  }
+  const Acc M = shfl_idx_x(im, 31), Rr = shfl_idx_x(ir, 31);
+  const long long C = __shfl_sync(FULL_MASK, ic, 31);
+  Acc mvs[3] = {0, 0, 0};
+  if (INIT) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      if (lane < th) mvs[q] = Ald<Acc>(L.tile_mv[3 * (size_t)(t0 + lane) + q]);
+      mvs[q] = wsum(mvs[q]);
+    }
+  }
+  float vb[3] = {0.0f, 0.0f, 0.0f};
+  int active = 0;
+  double mrem = 0.0;
+  if (lane == 0) {
+    active = halo_update<R, INIT>(L, S, pass, M, Rr, C, mvs, vb);
+    mrem = S.mrem;
+  }
+  active = __shfl_sync(FULL_MASK, active, 0);
+  if (!active) return;
+  mrem = __shfl_sync(FULL_MASK, mrem, 0);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) vb[q] = __shfl_sync(FULL_MASK, vb[q], 0);
+  bool keep = lane < nu;
+  if (!INIT && keep && skips<R>(L, u, pass, rc, mrem, vb[0], vb[1], vb[2])) keep = false;
+  const unsigned bal = __ballot_sync(FULL_MASK, keep);
+  if (bal == 0u) {
+    // every sub-tile left out: the next pass would remove nothing
+    if (!INIT && lane == 0) {
+      S.part_iter += S.n_alive;
+      S.n_iter = pass + 1;
+      S.active = 0;
+    }
+    return;
+  }
+  int base = 0;
+  if (lane == 0) base = atomicAdd(&L.ctl->work_n[(pass + 1) & 1], __popc(bal));
+  base = __shfl_sync(FULL_MASK, base, 0);
+  if (keep) {
+    int4* list = L.work + (size_t)((pass + 1) & 1) * n_sub;
+    list[base + __popc(bal & lanemask_lt())] =
+        make_int4(u, k, (int)(L.halos[k].gbase + (long long)lane * SUB), (int)min((long long)SUB, nm - (long long)lane * SUB));
+  }
+}
+
 // Per halo, after the initial sums (INIT, pass 0) or after pass `pass`: the
 // tiles' sums of the set left (copy (pass + 1) & 1 of the sub-tile sums),
 // their exclusive prefix over the halo (for the next pass and the final one),
-// the totals, and the halo's bookkeeping: iterations, particle-iterations,
-// band tests, sum m v, v_bulk, convergence (Sect. 2.1, Appendix A: the loop
-// ends when an iteration removes nothing).  Each thread takes a run of
-// consecutive tiles; the runs' sums are scanned over the CTA.
+// the totals, and the halo's bookkeeping (halo_update).  Each thread takes a run
+// of consecutive tiles; the runs' sums are scanned over the CTA.
 // The sub-tiles of the haloes still active are listed for the next pass.
+// The haloes are in order of size: the first L.n_cta_halos take a CTA each, the
+// others (GRID_WARP_TILES tiles at most) a warp each.
 template <typename R, bool INIT, int HT>
 __global__ void __launch_bounds__(HT) g_halo(GridLaunch L, int pass) {
   if (gave_up(L)) return;
@@ -1528,9 +1686,15 @@ __global__ void __launch_bounds__(HT) g_halo(GridLaunch L, int pass) {
   __shared__ float s_vb[3];                // the skip test's halo input
   __shared__ int s_wn[NW], s_wb[NW];       // kept sub-tiles per warp, their list positions
   __shared__ int s_kept;                   // sub-tiles of the halo on the next list
+  if (INIT && bins_overflowed(L)) return;
+  if (blockIdx.x >= L.n_cta_halos) {
+    const int kw = L.n_cta_halos + (blockIdx.x - L.n_cta_halos) * NW + (threadIdx.x >> 5);
+    if (kw < L.n_halos) halo_warp<R, INIT>(L, kw, pass);
+    return;
+  }
   const int k = blockIdx.x;
   GridHaloState& S = L.state[k];
-  if (INIT ? bins_overflowed(L) : !S.active) return;
+  if (!INIT && !S.active) return;
   const int n_sub = L.n_tiles * SPT;
   const int cp = (pass + 1) & 1;
   const Acc* am = (const Acc*)L.agg_m + (size_t)cp * n_sub;
@@ -1645,46 +1809,7 @@ __global__ void __launch_bounds__(HT) g_halo(GridLaunch L, int pass) {
     for (int q = 0; q < 3; ++q) mvs[q] = block_sum_n<Acc, HT>(mvs[q], racc);
   }
   if (threadIdx.x == 0) {
-    Acc mv[3];
-    int active;
-    if (INIT) {
-#pragma unroll
-      for (int q = 0; q < 3; ++q) mv[q] = mvs[q];
-      active = C > 0 ? 1 : 0;
-    } else {
-      const long long alive = S.n_alive;
-      S.part_iter += alive;
-      S.band += S.band_pass;
-      S.band_pass = 0;
-      S.n_iter = pass;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        mv[q] = Ald<Acc>(S.mv[q]) - Ald<Acc>(S.rem_mv[q]);
-        A<Acc>(S.rem_mv[q]) = 0;
-      }
-      active = 1;
-      if (C == alive) {
-        active = 0;
-      } else if (C == 0) {
-        active = 0;
-        S.status |= AHF_HALO_EMPTY;
-      } else if (pass >= L.prm.max_iter) {
-        active = 0;
-        S.status |= AHF_HALO_NOT_CONVERGED;
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 3; ++q) A<Acc>(S.mv[q]) = mv[q];
-    A<Acc>(S.m_tot) = M;
-    A<Acc>(S.t_tot) = Rr;
-    S.n_alive = C;
-    if (active && (INIT || !L.prm.vbulk_initial)) set_vbulk<R>(S, M, mv);
-    S.active = active;
-    // the mass lost so far (exact sums), for the skip records and test
-    if (INIT) A<Acc>(S.m_init) = M;
-    S.mrem = INIT ? 0.0 : dfix(Ald<Acc>(S.m_init) - M, S.s_m);
-#pragma unroll
-    for (int q = 0; q < 3; ++q) s_vb[q] = sizeof(R) == 4 ? S.vbulk[q] : (float)S.vbulk_d[q];
+    const int active = halo_update<R, INIT>(L, S, pass, M, Rr, C, mvs, s_vb);
     // the halo's sub-tiles holding members go on the next pass's list
     s_nw = active ? (int)((S.n_member + SUB - 1) / SUB) : 0;
     s_kept = 0;
@@ -1697,7 +1822,6 @@ __global__ void __launch_bounds__(HT) g_halo(GridLaunch L, int pass) {
     int4* list = L.work + (size_t)((pass + 1) & 1) * n_sub;
     const double mrem = S.mrem;
     const float vb0 = s_vb[0], vb1 = s_vb[1], vb2 = s_vb[2];
-    const float two_g = 2.0f * L.prm.Gf, rsoft = L.prm.r_soft_f;
     // RB sub-tiles per thread and round, their records loaded together
     constexpr int RB = 4;
     for (int j0 = 0; j0 < nw; j0 += RB * HT) {
@@ -1714,29 +1838,7 @@ __global__ void __launch_bounds__(HT) g_halo(GridLaunch L, int pass) {
         const int j = j0 + r * HT + threadIdx.x;
         const int u = t0 * SPT + j;
         if (INIT || !keep[r]) continue;
-        // a sub-tile tested in an earlier pass stays out while its members
-        // can neither be removed nor fall in the band: since that test each
-        // member's 2|phi| fell by at most 2 G dM / max(r, r_soft) (the
-        // halo lost mass dM, each removed particle's term at most m / r of
-        // the member's own radius), and its |u|^2 rose by at most
-        // 2 |u| dv + dv^2 (v_bulk moved by dv); the record's margin (slack
-        // 2^-16 of 2|phi| for the float rounding of both tests) must exceed
-        // that, with 2^-10 more on the bound for its own rounding
-        const float dm = (float)(mrem - rc[r].mrem) * (1.0f + 0x1p-20f);
-        const float reff = fmaxf(rc[r].rin, rsoft);
-        const float ax = vb0 - rc[r].vb[0], ay = vb1 - rc[r].vb[1], az = vb2 - rc[r].vb[2];
-        const float vmag = fabsf(vb0) + fabsf(vb1) + fabsf(vb2) + fabsf(rc[r].vb[0]) + fabsf(rc[r].vb[1]) +
-                           fabsf(rc[r].vb[2]);
-        const float dv = sqrtf(fmaf(az, az, fmaf(ay, ay, ax * ax))) * (1.0f + 0x1p-20f) + vmag * 0x1p-20f;
-        const float bound = (two_g * dm / reff + dv * fmaf(2.0f, rc[r].umax, dv)) * (1.0f + 0x1p-10f);
-        if (reff > 0.0f && isfinite(bound) && rc[r].margin > bound) {
-          keep[r] = false;
-          // its sums carry over to the copy the next pass would have written
-          const size_t a = (size_t)((pass + 1) & 1) * n_sub + u, b = (size_t)(pass & 1) * n_sub + u;
-          ((Acc*)L.agg_m)[b] = ((const Acc*)L.agg_m)[a];
-          ((Acc*)L.agg_r)[b] = ((const Acc*)L.agg_r)[a];
-          L.agg_c[b] = L.agg_c[a];
-        }
+        if (skips<R>(L, u, pass, rc[r], mrem, vb0, vb1, vb2)) keep[r] = false;
       }
       // list positions: a warp scan of the warps' counts, one reservation per round
       unsigned bal[RB];
@@ -2139,14 +2241,17 @@ __global__ void __launch_bounds__(T) g_removed(GridLaunch L, int pass) {
   const V4* rec = (const V4*)L.rec;
   const V4* vr = (const V4*)L.vr;        // radial order, or NULL (radix sort): by candidate
   const R m0 = sizeof(R) == 4 ? (R)L.p.m0f : (R)L.p.m0;
-  // 32 listed sub-tiles per step: lane j checks entry i0 + j's flags (32
-  // bytes), then the warp takes the flagged ones one after another
+  // `share` listed sub-tiles per step (32, fewer when the list would leave
+  // warps without any: 43 sub-tiles of one halo were two warps' work, 27 us in
+  // FP64): lane j checks entry i0 + j's flags (32 bytes), then the warp takes the
+  // flagged ones one after another
   const int nwarps = (gridDim.x * T) >> 5;
-  for (int i0 = ((blockIdx.x * T + threadIdx.x) >> 5) * 32; i0 < n; i0 += nwarps * 32) {
+  const int share = min(32, (n + nwarps - 1) / nwarps);
+  for (int i0 = ((blockIdx.x * T + threadIdx.x) >> 5) * share; i0 < n; i0 += nwarps * share) {
     const int ij = i0 + lane;
     int4 wj = make_int4(0, 0, 0, 0);
     bool any = false;
-    if (ij < n) {
+    if (ij < n && lane < share) {
       wj = list[ij];
       const uint4* mk = (const uint4*)(L.rem_mask + (size_t)wj.x * 32);
       const uint4 m0 = mk[0], m1 = mk[1];
@@ -2645,10 +2750,15 @@ void launch_prepare(const GridLaunch& L, cudaStream_t s) {
   }
 }
 
+// CTAs of g_halo: one per large halo, then one warp per small one.
+int halo_ctas(const GridLaunch& L, int threads) {
+  return L.n_cta_halos + blocks_for(L.n_halos - L.n_cta_halos, threads / 32);
+}
+
 template <typename R>
 void launch_halo_init(const GridLaunch& L, cudaStream_t s) {
-  if (L.max_halo_tiles > 64) g_halo<R, true, HT_BIG><<<L.n_halos, HT_BIG, 0, s>>>(L, 0);
-  else g_halo<R, true, HT_SMALL><<<L.n_halos, HT_SMALL, 0, s>>>(L, 0);
+  if (L.max_halo_tiles > 64) g_halo<R, true, HT_BIG><<<halo_ctas(L, HT_BIG), HT_BIG, 0, s>>>(L, 0);
+  else g_halo<R, true, HT_SMALL><<<halo_ctas(L, HT_SMALL), HT_SMALL, 0, s>>>(L, 0);
 }
 
 // The distribution into radial bins (see g_sample).
@@ -2755,8 +2865,8 @@ cudaError_t iterate_t(const GridLaunch& L, int pass, cudaStream_t s) {
   else g_pass<R, false, true><<<L.iter_grid, T, 0, s>>>(L, pass);
   if (unif) g_removed<R, true><<<L.iter_grid, T, 0, s>>>(L, pass);
   else g_removed<R, false><<<L.iter_grid, T, 0, s>>>(L, pass);
-  if (L.max_halo_tiles > 64) g_halo<R, false, HT_BIG><<<L.n_halos, HT_BIG, 0, s>>>(L, pass);
-  else g_halo<R, false, HT_SMALL><<<L.n_halos, HT_SMALL, 0, s>>>(L, pass);
+  if (L.max_halo_tiles > 64) g_halo<R, false, HT_BIG><<<halo_ctas(L, HT_BIG), HT_BIG, 0, s>>>(L, pass);
+  else g_halo<R, false, HT_SMALL><<<halo_ctas(L, HT_SMALL), HT_SMALL, 0, s>>>(L, pass);
   return cudaGetLastError();
 }
 

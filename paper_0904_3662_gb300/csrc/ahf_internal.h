@@ -231,6 +231,7 @@ struct GridLaunch {
   int* big_halos;          // haloes of more than 256 tiles (digit scans spread over CTAs)
   int n_big;
   int max_halo_tiles;      // tiles of the largest halo
+  int n_cta_halos;         // leading haloes of more than GRID_WARP_TILES tiles
   // per sub-tile of GRID_SUB elements (GRID_TILE / GRID_SUB per tile), two
   // copies by pass parity (pass p reads copy p & 1 and writes the other): the
   // exact sums (m, m/r as long long / __int128) and count of its alive members
@@ -256,6 +257,7 @@ struct GridLaunch {
 constexpr int GRID_TILE = 2048;
 constexpr int GRID_THREADS = 256;
 constexpr int GRID_SUB = 256;      // elements of a sub-tile (one warp's share of a pass)
+constexpr int GRID_WARP_TILES = 32 * GRID_SUB / GRID_TILE;  // tiles of a halo one warp keeps the books of
 
 // CTAs of the multi-CTA class's persistent iteration pass that fit on
 // `device` at once.
