@@ -1350,7 +1350,7 @@ int props_impl(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64_
   L.props = props;
   AHF_CUDA(launch_properties(L, s));
   reset_stats(c);
-  c->stats.launches = (n_chunks > 0 ? 2 : 0) + 1;
+  c->stats.launches = (n_chunks > 0 ? (p->m ? 2 : 1) : 0) + 1;
   return end_call(c, s);
 }
 
