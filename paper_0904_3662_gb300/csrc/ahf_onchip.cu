@@ -7,10 +7,10 @@
 //            each member's offset, mass and velocity to its 32-byte record
 //   sort     stable LSD radix sort of the keys, once: the centre is fixed and
 //            particles only leave, so the survivors of every later iteration
-//            stay in radial order.  One CTA ranks 5-bit digits by counting
-//            (count_sort); a cluster ranks 8-bit digits by lane matching, each
-//            CTA holding a contiguous chunk of the order, the scatter writing
-//            into the owner CTA's shared memory.
+//            stay in radial order.  One CTA distributes (dist_sort; count_sort
+//            for dozens of equal radii); a cluster ranks 8-bit digits by lane
+//            matching, each CTA holding a contiguous chunk of the order, the
+//            scatter writing into the owner CTA's shared memory.
 //   fill     sorted SoA from the records: radius, mass, w = v + H d; exact
 //            sum m v
 //   iterate  scan of the exact M(<r) and sum m/r prefixes ->
@@ -37,11 +37,6 @@ namespace cg = cooperative_groups;
 
 namespace ahf {
 namespace {
-
-// Swizzled shared-memory position of element p for a blocked arrangement of
-// ipt = mask + 1 consecutive elements per thread: conflict-free both for
-// per-thread runs and for warp-striped access.
-__device__ __forceinline__ int sw(int p, int mask) { return p ^ ((p >> 5) & mask); }
 
 template <int CS>
 struct Cl {
@@ -96,7 +91,7 @@ struct Smem {
   long long scan_base[NW][3];
   long long tot[3];
   uint32_t or_bits, and_bits, max_m, max_mr, max_mv;
-  uint32_t max_key;             // largest member key (single-CTA sort)
+  uint32_t max_key, min_key;    // extreme member keys (single-CTA sort)
   int n_member;
   long long acc[4];             // block accumulators (m v or removed m, m v)
   int acc_n, acc_band;
@@ -207,15 +202,14 @@ __device__ __forceinline__ void cluster_exchange(Smem<NT>& S, Xchg& X, int rank,
 
 // Stable LSD radix sort of the halo's keys, 8-bit digits, skipping the digits
 // in which all keys agree.  Each CTA of the cluster holds `nloc` elements of a
-// chunk of `chunk` positions, in order; the result keeps that partition, with
-// element p of a CTA at sw(p, mask).  Every pass scatters (key, value) pairs
+// chunk of `chunk` positions, in order; the result keeps that partition.  Every pass scatters (key, value) pairs
 // as one 8-byte store into the owner CTA's shared memory (the two arrays of a
 // buffer, kA|vA or kB|vB, hold CAP interleaved pairs between passes); a local
 // pass splits the final pairs into the other buffer.  Returns 0 if the result
 // is in (kA, vA), 1 if in (kB, vB) (the same in every CTA).
 template <int NT, int IPT, int CS>
 __device__ int cluster_radix_sort(uint32_t* kA, uint32_t* vA, uint32_t* kB, uint32_t* vB, uint16_t* hist, Smem<NT>& S,
-                                  Xchg& X, int nloc, int chunk, uint32_t diff, int mask, int rank) {
+                                  Xchg& X, int nloc, int chunk, uint32_t diff, int rank) {
   constexpr int NW = NT / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int passes[4], np = 0;
@@ -223,8 +217,8 @@ __device__ int cluster_radix_sort(uint32_t* kA, uint32_t* vA, uint32_t* kB, uint
     if ((diff >> (8 * d)) & 0xffu) passes[np++] = d;
   if (np == 0) {
     for (int p = threadIdx.x; p < nloc; p += NT) {
-      kB[sw(p, mask)] = kA[p];
-      vB[sw(p, mask)] = vA[p];
+      kB[p] = kA[p];
+      vB[p] = vA[p];
     }
     __syncthreads();
     return 1;
@@ -313,17 +307,19 @@ __device__ int cluster_radix_sort(uint32_t* kA, uint32_t* vA, uint32_t* kB, uint
     pin = pout;
     pout = t;
   }
-  // split this CTA's sorted pairs into the other buffer, swizzled
+  // split this CTA's sorted pairs into the other buffer
   uint32_t* ko = reinterpret_cast<uint32_t*>(pout);
   uint32_t* vo = ko + IPT * NT;
   for (int p = threadIdx.x; p < nloc; p += NT) {
     const uint2 x = pin[p];
-    ko[sw(p, mask)] = x.x;
-    vo[sw(p, mask)] = x.y;
+    ko[p] = x.x;
+    vo[p] = x.y;
   }
   __syncthreads();
   return pout == pA ? 0 : 1;
 }
+
+constexpr int SORT_CELLS = 512;     // cells of the single-CTA radial sort
 
 template <int NT, int CS>
 constexpr int min_blocks() { return CS > 1 ? 1 : (NT <= 128 ? 6 : (NT <= 256 ? 2 : 1)); }
@@ -363,14 +359,12 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
     }
     const int lo = rank * chunk;
     const int nloc = max(0, min(n_cand - lo, chunk));
-    int ipt = 1;
-    while (ipt * NT < chunk) ipt <<= 1;
-    const int mask = ipt - 1;
     prefetch_candidates<CT>(L.p, L.out.member_idx, H.offset + lo, H.offset + lo + nloc, tid);
     if (tid == 0) {
       S.or_bits = 0u; S.and_bits = 0xffffffffu;
       S.max_m = 0u; S.max_mr = 0u; S.max_mv = 0u;
       S.max_key = 0u;
+      S.min_key = 0xffffffffu;
       S.n_member = 0;
       S.acc[0] = S.acc[1] = S.acc[2] = S.acc[3] = 0;
       S.acc_n = 0; S.acc_band = 0;
@@ -379,7 +373,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
 
     // ---- gather: key = radius bits of members, candidate position as value ----
     {
-      uint32_t orb = 0u, andb = 0xffffffffu, mxm = 0u, mxr = 0u, mxv = 0u, kmx = 0u;
+      uint32_t orb = 0u, andb = 0xffffffffu, mxm = 0u, mxr = 0u, mxv = 0u, kmx = 0u, kmn = 0xffffffffu;
       int nmem = 0;
       for (int i = tid; i < nloc; i += NT) {
         const int j = lo + i;
@@ -413,16 +407,13 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
         }
         // members start bound (removal overwrites with its iteration)
         if (L.out.removed_iter) L.out.removed_iter[slot] = key == KEY_NONMEMBER ? -1 : 0;
-        // one CTA sorts runs of ipt consecutive positions (swizzled), a
-        // cluster contiguous chunks; the single-CTA sort's key range is
-        // the members' (non-members get a key just above it)
-        const int wpos = CS == 1 ? sw(i, mask) : i;
-        kA[wpos] = key;
-        vA[wpos] = (uint32_t)j;
+        kA[i] = key;
+        if constexpr (CS > 1) vA[i] = (uint32_t)j;
         if (CS > 1 || key != KEY_NONMEMBER) {
           orb |= key;
           andb &= key;
           kmx = max(kmx, key);
+          kmn = min(kmn, key);
         }
       }
       orb = __reduce_or_sync(FULL_MASK, orb);
@@ -431,9 +422,15 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
       mxr = __reduce_max_sync(FULL_MASK, mxr);
       mxv = __reduce_max_sync(FULL_MASK, mxv);
       nmem = __reduce_add_sync(FULL_MASK, nmem);
-      if constexpr (CS == 1) kmx = __reduce_max_sync(FULL_MASK, kmx);
+      if constexpr (CS == 1) {
+        kmx = __reduce_max_sync(FULL_MASK, kmx);
+        kmn = __reduce_min_sync(FULL_MASK, kmn);
+      }
       if (lane == 0) {
-        if constexpr (CS == 1) atomicMax(&S.max_key, kmx);
+        if constexpr (CS == 1) {
+          atomicMax(&S.max_key, kmx);
+          atomicMin(&S.min_key, kmn);
+        }
         atomicOr(&S.or_bits, orb);
         atomicAnd(&S.and_bits, andb);
         atomicMax(&S.max_m, mxm);
@@ -477,22 +474,28 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
     // ---- radial sort (once) ----
     int which;
     if constexpr (CS == 1) {
-      uint32_t diff = 0u, sub = 0u;
-      if (n_mem > 0) {
-        diff = S.or_bits ^ S.and_bits;
-        if (n_mem < n_cand) {
+      which = 0;
+      uint32_t* aux = reinterpret_cast<uint32_t*>(hist);
+      uint32_t* wtot = reinterpret_cast<uint32_t*>(&S.red[0][0]);
+      // (the counts' last word, cnt[CAP], is ex2's first)
+      if (n_mem > 0 && !dist_sort<NT, SORT_CELLS>(kA, vA, kB, vB, vA, reinterpret_cast<uint32_t*>(ex1), aux, wtot,
+                                                  nullptr, nloc, n_mem, S.min_key, S.max_key, tid)) {
+        for (int i = tid; i < nloc; i += NT) vA[i] = (uint32_t)i;
+        uint32_t diff = S.or_bits ^ S.and_bits, sub = 0u;
+        if (n_mem < n_cand) {              // non-members get a key just above the members'
           sub = S.max_key + 1u;
           diff = (S.or_bits | sub) ^ (S.and_bits & sub);
         }
+        __syncthreads();
+        which = count_sort<NT, (run_length(CAP, NT) + 3) / 4 * 4>(kA, vA, kB, vB, aux, wtot, nloc,
+                                                                   run_length(nloc, NT), diff, sub, tid);
       }
-      which = count_sort<NT, IPT>(kA, vA, kB, vB, reinterpret_cast<uint32_t*>(hist),
-                                  reinterpret_cast<uint32_t*>(&S.red[0][0]), nloc, mask, diff, sub, tid);
     } else {
       which = cluster_radix_sort<NT, IPT, CS>(kA, vA, kB, vB, hist, S, X, nloc, chunk, S.or_bits ^ S.and_bits,
-                                              mask, rank);
+                                              rank);
     }
     if (tid == 0 && rank == 0) trace_mark(L.trace, H.index, 2);
-    float* rr = (float*)(which ? kB : kA);         // radius, sorted, swizzled
+    float* rr = (float*)(which ? kB : kA);         // radius, sorted
     uint32_t* jj = which ? vB : vA;                // candidate position
     float* mm = (float*)(which ? kA : kB);         // mass; sign bit = removed
     float* wx = (float*)(which ? vA : vB);
@@ -501,11 +504,12 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
 
     // ---- fill: m and w = v + H d in the radial order, and the exact sum m v
     // of the members (the sorted candidates re-read from the store, mostly L2)
+    const int ipt = run_length(nmem_loc, NT);
     const int p0 = tid * ipt;
     {
       long long smv[3] = {0, 0, 0};
       for (int p = tid; p < nmem_loc; p += NT) {
-        const int q = sw(p, mask);
+        const int q = p;
         const int j = (int)jj[q];
         float dfl[3], v[3], m;
         if (L.rec) {
@@ -553,7 +557,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
     for (int k = 0; k < ipt; ++k) {
       const int p = p0 + k;
       if (p < nmem_loc) {
-        const int q = sw(p, mask);
+        const int q = p;
         const float mq = mm[q];
         const float m = unim ? L.p.m0f : mq;
         const float ri = unim ? mq : rinv_of(rr[q], P.r_soft_f);
@@ -657,13 +661,13 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
       int nrem = 0, nband = 0;
       uint32_t rmask = 0;                 // this thread's removals (bit k: position p0 + k)
       // no branch per member: a slot past the members or removed earlier
-      // adds nothing and is not tested (every slot of the run is within the
-      // arrays), so the loop's members can overlap
+      // adds nothing and is not tested (a run may reach a few words past its
+      // array, into the next one), so the loop's members can overlap
       if (p0 < nmem_loc) {
 #pragma unroll 4
         for (int k = 0; k < ipt; ++k) {
           const int p = p0 + k;
-          const int q = sw(p, mask);
+          const int q = p;
           const float mq = mm[q];
           const bool alive = p < nmem_loc && !signbit(mq);
           const float m = unim ? L.p.m0f : mq;
@@ -689,7 +693,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
       // the removed: exact m v from the stored velocity, and their record
       for (uint32_t b = rmask; b; b &= b - 1) {
         const int k = __ffs(b) - 1;
-        const int q = sw(p0 + k, mask);
+        const int q = p0 + k;
         const float m = unim ? L.p.m0f : -mm[q];
         const int j = (int)jj[q];
         const long long slot = H.offset + j;
@@ -747,8 +751,12 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
 
     if (tid == 0 && rank == 0) trace_mark(L.trace, H.index, 4);
     // ---- emit: bound list, phi, compacted (r, inclusive M) for the virial search ----
+    // (a uniform mass needs no masses: the bound list and phi are compacted
+    // there and go out coalesced, instead of 32 sectors per warp and store)
     float* rc = wx;                       // reuse: w is no longer needed
     long long* mc = (long long*)ex1;      // ex1 and ex2 are contiguous
+    float* pc = ex1;                      // uniform mass: phi, candidate position
+    uint32_t* jc = (uint32_t*)ex2;
     {
       long long tm = tm_own, tr = tr_own, tc = tc_own;
       if constexpr (CS == 1) {
@@ -773,7 +781,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
       for (int k = 0; k < ipt; ++k) {
         const int p = p0 + k;
         if (p < nmem_loc) {
-          const int q = sw(p, mask);
+          const int q = p;
           const float mq = mm[q];
           if (!signbit(mq)) {
             const float r = rr[q];
@@ -783,14 +791,17 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
             const float phi = phi_of(fix_to_float_fast(tm, s_m, sc_m), ri, fix_to_float_fast(T_tot - tr, s_r, sc_r),
                                      P.Gf);
             const int j = (int)jj[q];
-            const long long slot = H.offset + j;
-            const long long pi = L.out.member_idx ? L.out.member_idx[slot] : slot;
-            const long long dst = H.offset + C_pre + tl;
-            L.out.bound_idx[dst] = pi;
-            if (L.out.phi) ((float*)L.out.phi)[dst] = phi;
-            const int kq = sw((int)tl, mask);
-            rc[kq] = r;
-            mc[kq] = tm + mfix;
+            rc[tl] = r;
+            if (unim) {
+              pc[tl] = phi;
+              jc[tl] = (uint32_t)j;
+            } else {
+              const long long slot = H.offset + j;
+              const long long dst = H.offset + C_pre + tl;
+              L.out.bound_idx[dst] = L.out.member_idx ? L.out.member_idx[slot] : slot;
+              if (L.out.phi) ((float*)L.out.phi)[dst] = phi;
+              mc[tl] = tm + mfix;
+            }
             tm += mfix;
             tr += fix_from_float(m * ri, s_r);
             tl += 1;
@@ -799,11 +810,19 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
       }
       if (tid == 0) S.k_first = 0x7fffffff;
       __syncthreads();
+      if (unim) {
+        const long long d0 = H.offset + C_pre;
+        for (int i = tid; i < (int)C_loc; i += NT) {
+          const long long slot = H.offset + (long long)jc[i];
+          L.out.bound_idx[d0 + i] = L.out.member_idx ? L.out.member_idx[slot] : slot;
+          if (L.out.phi) ((float*)L.out.phi)[d0 + i] = pc[i];
+        }
+      }
       float r_after = __int_as_float(0x7f800000);   // +inf: radius of the next bound particle
       if constexpr (CS > 1) {
         if (tid == 0) {
           X.nb_loc = (int)C_loc;
-          X.first_r = C_loc > 0 ? rc[sw(0, mask)] : 0.0f;
+          X.first_r = C_loc > 0 ? rc[0] : 0.0f;
         }
         Cl<CS>::sync();
         for (int r2 = rank + 1; r2 < CS; ++r2) {
@@ -816,10 +835,10 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
       for (int k = 0; k < ipt; ++k) {
         const int kk = p0 + k;
         if (kk < C_loc) {
-          const float rn = kk + 1 < C_loc ? rc[sw(kk + 1, mask)] : r_after;
+          const float rn = kk + 1 < C_loc ? rc[kk + 1] : r_after;
           bool cross = true;
           if (!isinf(rn)) {
-            const long long mk = mc[sw(kk, mask)];
+            const long long mk = unim ? (C_pre + kk + 1) * m0fix : mc[kk];
             const float lhs = fix_to_float_fast(mk, s_m, sc_m);
             const float rhs = P.crit_f * rn * rn * rn;
             if (lhs < rhs * (1.0f - 1e-5f)) cross = true;
@@ -859,11 +878,11 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
           if (nb > 0) {
             const int kl = (int)(k - C_pre);
             // M_vir: (k+1) m0 in FP64 for a uniform mass, else the exact sum
-            const long long mkx = unim ? 0 : mc[sw(kl, mask)];
+            const long long mkx = unim ? 0 : mc[kl];
             const double mk = unim ? double_from_fix(k + 1, 0) * L.p.m0 : double_from_fix(mkx, s_m);
             const float mkf = unim ? (float)(k + 1) * L.p.m0f : float_from_fix(mkx, s_m);
             if (k == nb - 1) status |= AHF_HALO_RVIR_BEYOND_EDGE;
-            if (below_threshold(mk, mkf, rc[sw(kl, mask)], P.crit_f, P.crit)) {
+            if (below_threshold(mk, mkf, rc[kl], P.crit_f, P.crit)) {
               status |= AHF_HALO_RVIR_NONE;
             } else {
               kv = k;
@@ -881,7 +900,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
                       pre += nl;
                     }
                   }
-                  const int l = sw((int)(p - pre), mask);
+                  const int l = (int)(p - pre);
                   r = float_to_double(Cl<CS>::at(rc, q)[l]);
                   m = unim ? double_from_fix(p + 1, 0) * L.p.m0 : double_from_fix(Cl<CS>::at(mc, q)[l], s_m);
                 };
@@ -920,7 +939,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
           // takes the largest inclusive mass (the last particle inside)
           if (tid == 0) {
             if (!owner) X.has_rvir = 0;
-            X.last_r = C_loc > 0 ? rc[sw((int)C_loc - 1, mask)] : 0.0f;
+            X.last_r = C_loc > 0 ? rc[(int)C_loc - 1] : 0.0f;
           }
           Cl<CS>::sync();
           double r_vir = 0.0;
@@ -939,11 +958,11 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
             int lo = 0, hi = (int)C_loc;            // first local k with rc[k] > e_b
             while (lo < hi) {
               const int mid = (lo + hi) >> 1;
-              if (le_edge_band(rc[sw(mid, mask)], ef, r_out, fac)) lo = mid + 1;
+              if (le_edge_band(rc[mid], ef, r_out, fac)) lo = mid + 1;
               else hi = mid;
             }
             X.pc[b] = lo;
-            X.pm[b] = lo > 0 ? mc[sw(lo - 1, mask)] : 0;
+            X.pm[b] = lo > 0 && !unim ? mc[lo - 1] : 0;
           }
           Cl<CS>::sync();
           if (rank == 0) {
@@ -981,7 +1000,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
       if constexpr (CS == 1) {
         if (L.rows.prof) {
           __syncthreads();                        // S.rvir
-          profile_rows(L.rows, H.index, rc, mc, [&](long long kk) { return sw((int)kk, mask); }, nb, S.rvir, s_m,
+          profile_rows(L.rows, H.index, rc, mc, [](long long kk) { return (int)kk; }, nb, S.rvir, s_m,
                        P.G, P.Gf, unim ? &L.p.m0 : nullptr, tid, NT);
         }
       }

@@ -18,9 +18,8 @@ namespace {
 constexpr int WARP_CAP = 512;                 // candidate slots per warp
 constexpr int IPL = WARP_CAP / 32;            // items per lane
 constexpr int WPB = 8;                        // warps per CTA
+constexpr int SORT_CELLS = 128;               // cells of the radial sort
 constexpr size_t WARP_BYTES = (size_t)WARP_CAP * 24 + 256 * 2;
-
-__device__ __forceinline__ int sw(int p, int mask) { return p ^ ((p >> 5) & mask); }
 
 __device__ __forceinline__ long long warp_excl(long long x, int lane, long long& total) {
   const long long inc = warp_inclusive_scan(x, lane);
@@ -29,20 +28,20 @@ __device__ __forceinline__ long long warp_excl(long long x, int lane, long long&
 }
 
 // Stable LSD radix sort of n <= WARP_CAP (key, val) pairs by one warp, 8-bit
-// digits ranked by lane matching; the last pass writes element p at
-// sw(p, mask).  For one warp this is faster than the CTA classes' counting
-// sort (4 passes at most instead of 6); keys are read again for the scatter,
-// so only the ranks stay in registers.  Returns 0 if the result is in
+// digits ranked by lane matching, for what dist_sort leaves (dozens of equal
+// radii).  For one warp this is faster than the CTA classes' counting sort (4
+// passes at most instead of 6); keys are read again for the scatter, so only
+// the ranks stay in registers.  Returns 0 if the result is in
 // (kA, vA), 1 if in (kB, vB).
 __device__ int warp_radix_sort(uint32_t* kA, uint32_t* vA, uint32_t* kB, uint32_t* vB, uint16_t* hist, int n,
-                               uint32_t diff, int mask, int lane) {
+                               uint32_t diff, int lane) {
   int passes[4], np = 0;
   for (int d = 0; d < 4; ++d)
     if ((diff >> (8 * d)) & 0xffu) passes[np++] = d;
   if (np == 0) {
     for (int p = lane; p < n; p += 32) {
-      kB[sw(p, mask)] = kA[p];
-      vB[sw(p, mask)] = vA[p];
+      kB[p] = kA[p];
+      vB[p] = vA[p];
     }
     __syncwarp();
     return 1;
@@ -51,7 +50,6 @@ __device__ int warp_radix_sort(uint32_t* kA, uint32_t* vA, uint32_t* kB, uint32_
   const int nb = (n + 31) / 32;
   for (int ip = 0; ip < np; ++ip) {
     const int shift = 8 * passes[ip];
-    const bool last = (ip == np - 1);
 #pragma unroll
     for (int i = 0; i < 8; ++i) hist[lane * 8 + i] = 0;
     __syncwarp();
@@ -95,8 +93,7 @@ __device__ int warp_radix_sort(uint32_t* kA, uint32_t* vA, uint32_t* kB, uint32_
         if (e < n) {
           const uint32_t key = kin[e], val = vin[e];
           const uint32_t dg = (key >> shift) & 0xffu;
-          int dst = (int)hist[dg] + (int)rk[b];
-          if (last) dst = sw(dst, mask);
+          const int dst = (int)hist[dg] + (int)rk[b];
           kout[dst] = key;
           vout[dst] = val;
         }
@@ -137,12 +134,9 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
       continue;
     }
     prefetch_candidates<CT>(L.p, L.out.member_idx, H.offset, H.offset + n_cand, lane);
-    int ipt = 1;
-    while (ipt * 32 < n_cand) ipt <<= 1;
-    const int mask = ipt - 1;
-
     // ---- gather ----
     uint32_t orb = 0u, andb = 0xffffffffu, mxm = 0u, mxr = 0u, mxv = 0u;
+    uint32_t kmn = 0xffffffffu, kmx = 0u;        // extreme member keys
     int nmem = 0;
     for (int i = lane; i < n_cand; i += 32) {
       const long long slot = H.offset + i;
@@ -168,12 +162,13 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
           mxr = max(mxr, __float_as_uint(fabsf(m * rinv_of(r, P.r_soft_f))));
 #pragma unroll
           for (int k = 0; k < 3; ++k) mxv = max(mxv, __float_as_uint(fabsf(__fmul_rn(m, v[k]))));
+          kmn = min(kmn, key);
+          kmx = max(kmx, key);
           ++nmem;
         }
       }
       if (key == KEY_NONMEMBER && L.out.removed_iter) L.out.removed_iter[slot] = -1;
       kA[i] = key;
-      vA[i] = (uint32_t)i;
       orb |= key;
       andb &= key;
     }
@@ -182,6 +177,8 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
     mxm = __reduce_max_sync(FULL_MASK, mxm);
     mxr = __reduce_max_sync(FULL_MASK, mxr);
     mxv = __reduce_max_sync(FULL_MASK, mxv);
+    kmn = __reduce_min_sync(FULL_MASK, kmn);
+    kmx = __reduce_max_sync(FULL_MASK, kmx);
     const int n_mem = (int)__reduce_add_sync(FULL_MASK, (unsigned)nmem);
     __syncwarp();
     const int s_m = fix_scale(float_exponent_of_bits(mxm), n_mem);
@@ -195,7 +192,14 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
 
     if (lane == 0) trace_mark(L.trace, H.index, 1);
     // ---- radial sort (once) ----
-    const int which = warp_radix_sort(kA, vA, kB, vB, hist, n_cand, orb ^ andb, mask, lane);
+    // (counts in ex1, whose word past the last is ex2's first; cells in ex2)
+    int which = 0;
+    if (n_mem > 0 && !dist_sort<32, SORT_CELLS>(kA, vA, kB, vB, vA, (uint32_t*)ex1, (uint32_t*)ex2 + 8, nullptr,
+                                                nullptr, n_cand, n_mem, kmn, kmx, lane)) {
+      for (int i = lane; i < n_cand; i += 32) vA[i] = (uint32_t)i;
+      __syncwarp();
+      which = warp_radix_sort(kA, vA, kB, vB, hist, n_cand, orb ^ andb, lane);
+    }
     float* rr = (float*)(which ? kB : kA);
     uint32_t* jj = which ? vB : vA;
     float* mm = (float*)(which ? kA : kB);
@@ -207,7 +211,7 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
     // ---- fill ----
     long long mv[3] = {0, 0, 0};
     for (int p = lane; p < n_mem; p += 32) {
-      const int q = sw(p, mask);
+      const int q = p;
       const int j = (int)jj[q];
       float dfl[3], v[3], m;
       if (L.rec) {
@@ -233,12 +237,13 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
     for (int k = 0; k < 3; ++k) mv[k] = warp_sum(mv[k]);
     __syncwarp();
 
+    const int ipt = run_length(n_mem, 32);
     const int p0 = lane * ipt;
     long long tm_own = 0, tr_own = 0, tc_own = 0;
     for (int k = 0; k < ipt; ++k) {
       const int p = p0 + k;
       if (p < n_mem) {
-        const int q = sw(p, mask);
+        const int q = p;
         const float mq = mm[q];
         const float m = unim ? L.p.m0f : mq;
         const float ri = unim ? mq : rinv_of(rr[q], P.r_soft_f);
@@ -272,13 +277,13 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
       int nrem = 0, nband = 0;
       uint32_t rmask = 0;                 // this lane's removals (bit k: position p0 + k)
       // no branch per member: a slot past the members or removed earlier
-      // adds nothing and is not tested (every slot of the run is within the
-      // arrays), so the loop's members can overlap
+      // adds nothing and is not tested (a run may reach a few words past its
+      // array, into the next one), so the loop's members can overlap
       if (p0 < n_mem) {
 #pragma unroll 4
         for (int k = 0; k < ipt; ++k) {
           const int p = p0 + k;
-          const int q = sw(p, mask);
+          const int q = p;
           const float mq = mm[q];
           const bool alive = p < n_mem && !signbit(mq);
           const float m = unim ? L.p.m0f : mq;
@@ -305,7 +310,7 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
       // velocity, and their removal iteration
       for (uint32_t b = rmask; b; b &= b - 1) {
         const int k = __ffs(b) - 1;
-        const int q = sw(p0 + k, mask);
+        const int q = p0 + k;
         const float m = unim ? L.p.m0f : -mm[q];
         const long long slot = H.offset + (long long)jj[q];
         float v[3];
@@ -336,7 +341,11 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
     if (lane == 0) trace_mark(L.trace, H.index, 4);
     // ---- emit ----
     float* rc = wx;
+    // (a uniform mass needs no masses: phi and the candidate positions are
+    // compacted there and go out coalesced)
     long long* mc = (long long*)ex1;      // ex1 and ex2 are contiguous
+    float* pc = ex1;
+    uint32_t* jc = (uint32_t*)ex2;
     long long M_tot, T_tot, nb;
     long long tm = warp_excl(tm_own, lane, M_tot);
     long long tr = warp_excl(tr_own, lane, T_tot);
@@ -345,7 +354,7 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
     for (int k = 0; k < ipt; ++k) {
       const int p = p0 + k;
       if (p < n_mem) {
-        const int q = sw(p, mask);
+        const int q = p;
         const float mq = mm[q];
         if (!signbit(mq)) {
           const float r = rr[q];
@@ -355,14 +364,17 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
           const float phi = phi_of(fix_to_float_fast(tm, s_m, sc_m), ri, fix_to_float_fast(T_tot - tr, s_r, sc_r),
                                    P.Gf);
           const long long slot = H.offset + (long long)jj[q];
-          const long long pi = L.out.member_idx ? L.out.member_idx[slot] : slot;
-          const long long dst = H.offset + tl;
-          L.out.bound_idx[dst] = pi;
-          if (L.out.phi) ((float*)L.out.phi)[dst] = phi;
           if (L.out.removed_iter) L.out.removed_iter[slot] = 0;
-          const int kq = sw((int)tl, mask);
-          rc[kq] = r;
-          mc[kq] = tm + mfix;
+          rc[tl] = r;
+          if (unim) {
+            pc[tl] = phi;
+            jc[tl] = jj[q];
+          } else {
+            const long long dst = H.offset + tl;
+            L.out.bound_idx[dst] = L.out.member_idx ? L.out.member_idx[slot] : slot;
+            if (L.out.phi) ((float*)L.out.phi)[dst] = phi;
+            mc[tl] = tm + mfix;
+          }
           tm += mfix;
           tr += fix_from_float(m * ri, s_r);
           tl += 1;
@@ -370,6 +382,13 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
       }
     }
     __syncwarp();
+    if (unim) {
+      for (int i = lane; i < (int)nb; i += 32) {
+        const long long slot = H.offset + (long long)jc[i];
+        L.out.bound_idx[H.offset + i] = L.out.member_idx ? L.out.member_idx[slot] : slot;
+        if (L.out.phi) ((float*)L.out.phi)[H.offset + i] = pc[i];
+      }
+    }
     // virial: first k with M_k < delta_rho 4pi/3 r_{k+1}^3 (r_{N+1} = inf)
     int kf = 0x7fffffff;
     for (int k = 0; k < ipt; ++k) {
@@ -377,8 +396,8 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
       if (kk < nb) {
         bool cross = true;
         if (kk + 1 < nb) {
-          const float rn = rc[sw(kk + 1, mask)];
-          const long long mk = mc[sw(kk, mask)];
+          const float rn = rc[kk + 1];
+          const long long mk = unim ? (kk + 1) * m0fix : mc[kk];
           const float lhs = fix_to_float_fast(mk, s_m, sc_m);
           const float rhs = P.crit_f * rn * rn * rn;
           if (lhs < rhs * (1.0f - 1e-5f)) cross = true;
@@ -400,11 +419,11 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
       double mvir = 0.0;
       if (nb > 0) {
         // M_vir: (k+1) m0 in FP64 for a uniform mass, else the exact sum
-        const long long mkx = unim ? 0 : mc[sw(kf, mask)];
+        const long long mkx = unim ? 0 : mc[kf];
         const double mk = unim ? double_from_fix(kf + 1, 0) * L.p.m0 : double_from_fix(mkx, s_m);
         const float mkf = unim ? (float)(kf + 1) * L.p.m0f : float_from_fix(mkx, s_m);
         if (kf == nb - 1) status |= AHF_HALO_RVIR_BEYOND_EDGE;
-        if (below_threshold(mk, mkf, rc[sw(kf, mask)], P.crit_f, P.crit)) {
+        if (below_threshold(mk, mkf, rc[kf], P.crit_f, P.crit)) {
           status |= AHF_HALO_RVIR_NONE;
         } else {
           kv = kf;
@@ -412,8 +431,8 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
           r_vir_l = virial_radius(mk, P.inv_crit);
           if (P.rise_edge && kf == nb - 1) {
             auto at = [&](long long k, double& r, double& m) {
-              r = float_to_double(rc[sw((int)k, mask)]);
-              m = unim ? double_from_fix(k + 1, 0) * L.p.m0 : double_from_fix(mc[sw((int)k, mask)], s_m);
+              r = float_to_double(rc[(int)k]);
+              m = unim ? double_from_fix(k + 1, 0) * L.p.m0 : double_from_fix(mc[(int)k], s_m);
             };
             const long long ke = rise_edge_index(nb, at);
             if (ke >= 0) {
@@ -440,7 +459,7 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
     }
     if (L.rows.prof) {
       const double r_vir = __shfl_sync(FULL_MASK, r_vir_l, 0);
-      profile_rows(L.rows, H.index, rc, mc, [&](long long k) { return sw((int)k, mask); }, nb, r_vir, s_m, P.G, P.Gf,
+      profile_rows(L.rows, H.index, rc, mc, [](long long k) { return (int)k; }, nb, r_vir, s_m, P.G, P.Gf,
                    unim ? &L.p.m0 : nullptr, lane, 32);
     }
     if (lane == 0 && L.trace) {
