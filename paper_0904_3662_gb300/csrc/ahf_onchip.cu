@@ -5,12 +5,12 @@
 //   gather   candidates -> (radius key, candidate position), FP64-accurate
 //            recentring and sphere test, exponent maxima for the exact sums;
 //            each member's offset, mass and velocity to its 32-byte record
-//   sort     stable LSD radix sort of the keys, once: the centre is fixed and
+//   sort     by radius, stable, once: the centre is fixed and
 //            particles only leave, so the survivors of every later iteration
 //            stay in radial order.  One CTA distributes (dist_sort; count_sort
-//            for dozens of equal radii); a cluster ranks 8-bit digits by lane
-//            matching, each CTA holding a contiguous chunk of the order, the
-//            scatter writing into the owner CTA's shared memory.
+//            for dozens of equal radii); a cluster first hands every CTA its
+//            share of the order (cluster_dist_sort; cluster_radix_sort when a
+//            share would not fit).
 //   fill     sorted SoA from the records: radius, mass, w = v + H d; exact
 //            sum m v
 //   iterate  scan of the exact M(<r) and sum m/r prefixes ->
@@ -62,9 +62,10 @@ constexpr int FUSE_BINS = 128;
 // Values a CTA publishes to the other CTAs of its cluster.
 struct Xchg {
   int halo;
-  uint32_t g_or, g_and, g_mxm, g_mxr, g_mxv;
+  uint32_t g_or, g_and, g_mxm, g_mxr, g_mxv, g_kmx, g_kmn;
   int g_nmem;
-  uint32_t cnt[256];            // radix pass: digit counts of this CTA
+  uint32_t cnt[256];            // radix pass: digit counts of this CTA; dist sort: its
+                                // members bound for each CTA
   long long mv[3];              // fill: partial sum m v
   // iteration exchange, two alternating copies: scan totals of this CTA
   // (M, sum m/r, count) and its removals of the previous iteration (m,
@@ -91,7 +92,7 @@ struct Smem {
   long long scan_base[NW][3];
   long long tot[3];
   uint32_t or_bits, and_bits, max_m, max_mr, max_mv;
-  uint32_t max_key, min_key;    // extreme member keys (single-CTA sort)
+  uint32_t max_key, min_key;    // extreme member keys
   int n_member;
   long long acc[4];             // block accumulators (m v or removed m, m v)
   int acc_n, acc_band;
@@ -319,7 +320,166 @@ __device__ int cluster_radix_sort(uint32_t* kA, uint32_t* vA, uint32_t* kB, uint
   return pout == pA ? 0 : 1;
 }
 
-constexpr int SORT_CELLS = 512;     // cells of the single-CTA radial sort
+constexpr int SORT_CELLS = 512;     // cells of a CTA's radial sort
+constexpr int CLUSTER_CELLS = 1024; // cells a cluster divides its members by
+
+// The radial sort of a cluster by distribution: the members are counted in
+// cells over the whole halo; the cells' counts give every CTA an equal share of
+// the order (within the few members by which a cell is not linear); each member
+// goes to the CTA of its share, once; every CTA sorts what it got (dist_sort).
+// Four cluster barriers and one DSMEM store per member, where the radix sort
+// takes two barriers, a ranking by lane matching and a store per key byte:
+// 42 -> 20 us per halo in clusters of 2 and 4 CTAs, 46 -> 23 of 8, 55 -> 23 of 16.
+// CTA r's share is radially below CTA r + 1's; what it holds is its own (nrec;
+// not the chunk of the candidates), in order, in (kA, vA) or (kB, vB) (0 or 1
+// returned).  -1, with everything as it was, when a share would not fit.
+template <int NT, int IPT, int CS>
+__device__ int cluster_dist_sort(uint32_t* kA, uint32_t* vA, uint32_t* kB, uint32_t* vB, uint32_t* ex1, uint32_t* ex2,
+                                 uint32_t* hist, Smem<NT>& S, Xchg& X, int nloc, int n_mem, int rank, int& nrec) {
+  constexpr int NW = NT / 32, CAP = IPT * NT, SLICE = CLUSTER_CELLS / CS;
+  static_assert(SLICE <= NT && CLUSTER_CELLS % NT == 0 && NW * 16 <= NT, "slices and counters fit the threads");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t* mine = ex2;                  // this CTA's cells
+  uint32_t* cum = ex1;                   // all of them: counts, then members before each cell
+  uint32_t* wq = hist;                   // [NW][16] members of each warp per destination
+  uint32_t* wtot = reinterpret_cast<uint32_t*>(&S.red[0][0]);
+  const uint32_t kmin = S.min_key, range = S.max_key - kmin;
+  const int sh = max(1, 32 - __clz(range | 1u) - 10);    // CLUSTER_CELLS << sh > range
+  static_assert(CLUSTER_CELLS == 1 << 10, "");
+  for (int c = tid; c < CLUSTER_CELLS; c += NT) mine[c] = 0u;
+  if (tid < NW * 16) wq[tid] = 0u;
+  __syncthreads();
+#pragma unroll 4
+  for (int i = tid; i < nloc; i += NT) {
+    const uint32_t key = kA[i];
+    if (key != KEY_NONMEMBER) atomicAdd(&mine[(key - kmin) >> sh], 1u);
+  }
+  Cl<CS>::sync();
+  // each CTA adds up a slice of the cells and hands it to all
+  if (tid < SLICE) {
+    const int c = rank * SLICE + tid;
+    uint32_t t = 0u;
+#pragma unroll
+    for (int r = 0; r < CS; ++r) t += Cl<CS>::at(mine, r)[c];
+#pragma unroll
+    for (int r = 0; r < CS; ++r) Cl<CS>::at(cum, r)[c] = t;
+  }
+  Cl<CS>::sync();
+  {
+    constexpr int CPT = CLUSTER_CELLS / NT;
+    uint32_t v[CPT], s = 0u;
+#pragma unroll
+    for (int j = 0; j < CPT; ++j) {
+      v[j] = cum[tid * CPT + j];
+      s += v[j];
+    }
+    uint32_t run = group_excl<NT>(s, wtot, tid);
+#pragma unroll
+    for (int j = 0; j < CPT; ++j) {
+      cum[tid * CPT + j] = run;
+      run += v[j];
+    }
+    if (tid == 0) cum[CLUSTER_CELLS] = (uint32_t)n_mem;
+  }
+  __syncthreads();
+  // destinations, and the rank among the warp's members for each: a warp takes
+  // consecutive candidates, so that equal radii arrive in candidate order
+  const uint32_t share = (uint32_t)(n_mem + CS - 1) / CS;
+  const int wchunk = ((nloc + NW * 32 - 1) / (NW * 32)) * 32;
+  uint32_t* pk = ex2;                    // (the cells in it have been read)
+  for (int e = warp * wchunk + lane; e - lane < min(nloc, (warp + 1) * wchunk); e += 32) {
+    const uint32_t key = e < nloc ? kA[e] : KEY_NONMEMBER;
+    const bool valid = key != KEY_NONMEMBER;
+    uint32_t q = 0u;
+    if (valid) {
+      const uint32_t x = key - kmin, c = x >> sh, b = cum[c];
+      q = (b + __umulhi(cum[c + 1] - b, x << (32 - sh))) / share;
+    }
+    unsigned peers = __ballot_sync(FULL_MASK, valid);
+#pragma unroll
+    for (int bit = 1; bit < CS; bit <<= 1) {
+      const unsigned bb = __ballot_sync(FULL_MASK, (q & bit) != 0u);
+      peers &= (q & bit) ? bb : ~bb;
+    }
+    const uint32_t base = wq[warp * 16 + q];
+    __syncwarp();
+    if (valid) {
+      const unsigned below = peers & lanemask_lt();
+      pk[e] = (q << 16) | (base + __popc(below));
+      if (below == 0u) wq[warp * 16 + q] = base + __popc(peers);
+    }
+    __syncwarp();
+  }
+  __syncthreads();
+  if (tid < CS) {
+    uint32_t run = 0u;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+      const uint32_t c = wq[w * 16 + tid];
+      wq[w * 16 + tid] = run;
+      run += c;
+    }
+    X.cnt[tid] = run;
+  }
+  Cl<CS>::sync();
+  if (tid < CS) {
+    uint32_t pre = 0u, tot = 0u;
+#pragma unroll
+    for (int r = 0; r < CS; ++r) {
+      const uint32_t v = Cl<CS>::at(X.cnt, r)[tid];
+      if (r < rank) pre += v;
+      tot += v;
+    }
+    S.dpre[tid] = pre;
+    S.dtot[tid] = tot;
+  }
+  __syncthreads();
+  bool fits = true;                      // (the parts' counts take one word more than the members)
+  for (int q = 0; q < CS; ++q) fits = fits && S.dtot[q] < (uint32_t)CAP;
+  if (!fits) {                           // the same in every CTA
+    Cl<CS>::sync();                      // every CTA has read the counts
+    return -1;
+  }
+  for (int e = warp * wchunk + lane; e < min(nloc, (warp + 1) * wchunk); e += 32) {
+    const uint32_t key = kA[e];
+    if (key != KEY_NONMEMBER) {
+      const uint32_t x = pk[e], q = x >> 16;
+      Cl<CS>::at(reinterpret_cast<uint2*>(kB), (int)q)[S.dpre[q] + wq[warp * 16 + q] + (x & 0xffffu)] =
+          make_uint2(key, vA[e]);
+    }
+  }
+  if (tid == 0) {
+    S.max_key = 0u;
+    S.min_key = 0xffffffffu;
+  }
+  Cl<CS>::sync();
+  nrec = (int)S.dtot[rank];
+  uint32_t mx = 0u, mn = 0xffffffffu;
+  for (int i = tid; i < nrec; i += NT) {
+    const uint2 x = reinterpret_cast<const uint2*>(kB)[i];
+    kA[i] = x.x;
+    vA[i] = x.y;
+    mx = max(mx, x.x);
+    mn = min(mn, x.x);
+  }
+  mx = __reduce_max_sync(FULL_MASK, mx);
+  mn = __reduce_min_sync(FULL_MASK, mn);
+  if (lane == 0) {
+    atomicMax(&S.max_key, mx);
+    atomicMin(&S.min_key, mn);
+  }
+  __syncthreads();
+  if (nrec == 0) return 0;
+  if (dist_sort<NT, SORT_CELLS>(kA, vA, kB, vB, ex2, ex1, hist, wtot, vA, nrec, nrec, S.min_key, S.max_key, tid))
+    return 0;
+  // dozens of equal radii: the counting radix sort of this CTA's share (its
+  // counters in ex1)
+  static_assert(count_sort_words(NT) <= CAP, "counters fit");
+  const uint32_t differ = S.max_key ^ S.min_key;
+  const uint32_t diff = differ ? 0xffffffffu >> __clz(differ) : 0u;
+  return count_sort<NT, (run_length(CAP, NT) + 3) / 4 * 4>(kA, vA, kB, vB, ex1, wtot, nrec, run_length(nrec, NT), diff,
+                                                           0u, tid);
+}
 
 template <int NT, int CS>
 constexpr int min_blocks() { return CS > 1 ? 1 : (NT <= 128 ? 6 : (NT <= 256 ? 2 : 1)); }
@@ -412,6 +572,8 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
         if (CS > 1 || key != KEY_NONMEMBER) {
           orb |= key;
           andb &= key;
+        }
+        if (key != KEY_NONMEMBER) {
           kmx = max(kmx, key);
           kmn = min(kmn, key);
         }
@@ -422,15 +584,11 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
       mxr = __reduce_max_sync(FULL_MASK, mxr);
       mxv = __reduce_max_sync(FULL_MASK, mxv);
       nmem = __reduce_add_sync(FULL_MASK, nmem);
-      if constexpr (CS == 1) {
-        kmx = __reduce_max_sync(FULL_MASK, kmx);
-        kmn = __reduce_min_sync(FULL_MASK, kmn);
-      }
+      kmx = __reduce_max_sync(FULL_MASK, kmx);
+      kmn = __reduce_min_sync(FULL_MASK, kmn);
       if (lane == 0) {
-        if constexpr (CS == 1) {
-          atomicMax(&S.max_key, kmx);
-          atomicMin(&S.min_key, kmn);
-        }
+        atomicMax(&S.max_key, kmx);
+        atomicMin(&S.min_key, kmn);
         atomicOr(&S.or_bits, orb);
         atomicAnd(&S.and_bits, andb);
         atomicMax(&S.max_m, mxm);
@@ -444,23 +602,26 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
       if (tid == 0) {
         X.g_or = S.or_bits; X.g_and = S.and_bits; X.g_mxm = S.max_m; X.g_mxr = S.max_mr; X.g_mxv = S.max_mv;
         X.g_nmem = S.n_member;
+        X.g_kmx = S.max_key; X.g_kmn = S.min_key;
       }
       Cl<CS>::sync();
       if (tid == 0) {
-        uint32_t o = 0u, a = 0xffffffffu, m1 = 0u, m2 = 0u, m3 = 0u;
+        uint32_t o = 0u, a = 0xffffffffu, m1 = 0u, m2 = 0u, m3 = 0u, kx = 0u, kn = 0xffffffffu;
         int nm = 0;
         for (int r = 0; r < CS; ++r) {
           const Xchg* Y = Cl<CS>::at(&X, r);
           o |= Y->g_or; a &= Y->g_and;
           m1 = max(m1, Y->g_mxm); m2 = max(m2, Y->g_mxr); m3 = max(m3, Y->g_mxv);
           nm += Y->g_nmem;
+          kx = max(kx, Y->g_kmx); kn = min(kn, Y->g_kmn);
         }
+        S.max_key = kx; S.min_key = kn;
         S.or_bits = o; S.and_bits = a; S.max_m = m1; S.max_mr = m2; S.max_mv = m3; S.n_member = nm;
       }
       __syncthreads();
     }
     const int n_mem = S.n_member;                        // members of the halo
-    const int nmem_loc = max(0, min(n_mem - lo, nloc));  // held by this CTA after the sort
+    int nmem_loc = max(0, min(n_mem - lo, nloc));        // held by this CTA after the sort
     const int s_m = fix_scale(float_exponent_of_bits(S.max_m), n_mem);
     const int s_r = fix_scale(float_exponent_of_bits(S.max_mr), n_mem);
     const int s_v = fix_scale(float_exponent_of_bits(S.max_mv), n_mem);
@@ -491,8 +652,13 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
                                                                    run_length(nloc, NT), diff, sub, tid);
       }
     } else {
-      which = cluster_radix_sort<NT, IPT, CS>(kA, vA, kB, vB, hist, S, X, nloc, chunk, S.or_bits ^ S.and_bits,
-                                              rank);
+      which = -1;
+      if (n_mem > 0)
+        which = cluster_dist_sort<NT, IPT, CS>(kA, vA, kB, vB, reinterpret_cast<uint32_t*>(ex1),
+                                               reinterpret_cast<uint32_t*>(ex2), reinterpret_cast<uint32_t*>(hist), S, X,
+                                               nloc, n_mem, rank, nmem_loc);
+      if (which < 0)
+        which = cluster_radix_sort<NT, IPT, CS>(kA, vA, kB, vB, hist, S, X, nloc, chunk, S.or_bits ^ S.and_bits, rank);
     }
     if (tid == 0 && rank == 0) trace_mark(L.trace, H.index, 2);
     float* rr = (float*)(which ? kB : kA);         // radius, sorted
