@@ -57,14 +57,17 @@ __device__ __forceinline__ int float_exponent_of_bits(uint32_t bits) {
 __device__ __forceinline__ long long fix_from_float(float x, int s) {
   const uint32_t b = __float_as_uint(x);
   const int e = (int)((b >> 23) & 0xff);
-  if (e == 0) return 0;                                   // zero / subnormal
-  const long long mant = (long long)((b & 0x7fffffu) | 0x800000u);
+  const uint32_t mant = (b & 0x7fffffu) | 0x800000u;
   const int sh = e - 150 + s;
   long long v;
-  if (sh >= 0) v = mant << (sh > 39 ? 39 : sh);
-  else if (sh > -25) v = ((mant >> (-sh - 1)) + 1) >> 1;
-  else v = 0;
-  return (b >> 31) ? -v : v;
+  if (sh >= 0 && e != 0) {
+    // the usual case: the quantum is finer than x's last place
+    v = (long long)((unsigned long long)mant << sh);
+  } else {
+    v = (e == 0 || sh <= -25) ? 0 : (long long)(((mant >> (-sh - 1)) + 1u) >> 1);   // (e = 0: zero / subnormal)
+  }
+  const long long sg = (long long)((int)b >> 31);         // all ones for x < 0
+  return (v ^ sg) - sg;
 }
 
 __device__ __forceinline__ long long fix_from_double(double x, int s) {
@@ -853,6 +856,68 @@ __device__ __forceinline__ float phi_of(float m_inner, float rinv, float outer, 
   return __fmul_rn(-G, __fmaf_rn(m_inner, rinv, outer));
 }
 
+// fix_from_float of a normal x > 0 (the exact term m / r of a uniform mass): one
+// shift when the quantum is finer than x's last place, as it is unless x is
+// 2^20 times smaller than the halo's largest term.
+__device__ __forceinline__ long long fix_positive(float x, int s) {
+  const uint32_t b = __float_as_uint(x);
+  const int sh = (int)(b >> 23) + (s - 150);
+  if (sh < 0) return fix_from_float(x, s);
+  return (long long)((unsigned long long)((b & 0x7fffffu) | 0x800000u) << sh);
+}
+
+// One iteration over a thread's run of members [p0, p0 + n): phi from the exact
+// sums before the run (tm: M(<r); out: the outer sum from the run's first
+// member on), the escape test against v_bulk vb; the members to remove as a
+// mask, and the count inside the band.  mm holds 1 / max(r, r_soft) with one
+// mass for all, else the mass; its sign bit marks a removed member, which adds
+// nothing and is not tested.  MODE 0: one mass, scales 2^-s normal floats (sc_m,
+// sc_r); 1: a mass each, the same; 2: any.
+//
+// The member loop is most of an iteration, and bound by issue slots (four warps
+// a scheduler), so it holds only what every member needs: 0 takes 55
+// instructions a member where the one loop for all modes, which also summed and
+// marked the removed, took about 130.
+template <int MODE>
+__device__ __forceinline__ void member_pass(const float* rr, const float* mm, const float* wx, const float* wy,
+                                            const float* wz, int p0, int n, const ParamsDev& P, bool unim, float m0f,
+                                            long long m0fix, int s_m, int s_r, float sc_m, float sc_r, float vb0,
+                                            float vb1, float vb2, long long tm, long long out, uint32_t& rmask,
+                                            int& nband) {
+#pragma unroll 4
+  for (int k = 0; k < n; ++k) {
+    const int q = p0 + k;
+    const float mq = mm[q];
+    const bool alive = !signbit(mq);
+    float ri, Mf, Sf;
+    long long mfix, rfix;
+    if (MODE == 0) {
+      ri = mq;
+      mfix = m0fix;
+      const float t = m0f * ri;                               // (0: at the centre; < 0: removed)
+      rfix = t >= 1.17549435e-38f ? fix_positive(t, s_r) : 0ll;
+      Mf = fix_to_float_sc(tm, sc_m);
+      Sf = fix_to_float_sc(out, sc_r);
+    } else {
+      const bool u = MODE == 2 && unim;
+      const float m = u ? m0f : mq;
+      ri = u ? mq : rinv_of(rr[q], P.r_soft_f);
+      mfix = u ? m0fix : fix_from_float(m, s_m);
+      rfix = fix_from_float(m * ri, s_r);
+      Mf = MODE == 1 ? fix_to_float_sc(tm, sc_m) : float_from_fix(tm, s_m);
+      Sf = MODE == 1 ? fix_to_float_sc(out, sc_r) : float_from_fix(out, s_r);
+    }
+    const float phi = phi_of(Mf, ri, Sf, P.Gf);
+    const float ux = wx[q] - vb0, uy = wy[q] - vb1, uz = wz[q] - vb2;
+    const float u2 = fmaf(uz, uz, fmaf(uy, uy, ux * ux));
+    const float two_phi = -2.0f * phi;
+    nband += (alive && fabsf(u2 - two_phi) < P.band_f * two_phi) ? 1 : 0;
+    if (alive && u2 > two_phi) rmask |= 1u << k;
+    tm += alive ? mfix : 0ll;
+    out -= alive ? rfix : 0ll;
+  }
+}
+
 // r <= e for a float radius r against the FP64 edge e (ef its float
 // rounding), decided exactly.
 __device__ __forceinline__ bool le_edge(float r, float ef, double e) {
@@ -893,10 +958,13 @@ __device__ __forceinline__ bool le_edge_band(float r, float ef, double r_out, do
 // chip: radii rc[idx(k)] ascending and inclusive exact masses mc[idx(k)]
 // (scale 2^-s_m), k < nb.  Row b covers (e_b, e_{b+1}], e_b = r_out f^(1-b/n),
 // r_out = r_vir or the outermost bound radius (Sect. 2.1, the radially binned
-// output).  The calling threads take rows t0, t0 + stride, ...
+// output); k_vir the last particle within r_vir (-1: none).  The calling threads,
+// whole warps of consecutive t0, take rows t0, t0 + stride, ...: each locates one
+// edge by binary search and gets the next one's from its neighbour.
 template <typename Idx>
 __device__ void profile_rows(const ProfileRows& Q, int h, const float* rc, const long long* mc, Idx idx, long long nb,
-                             double r_vir, int s_m, double G, float Gf, const double* m0, int t0, int stride) {
+                             double r_vir, long long k_vir, int s_m, double G, float Gf, const double* m0, int t0,
+                             int stride) {
   const int n = Q.n_bins;
   double* out = Q.prof + (size_t)h * n * 4;
   if (nb == 0) {
@@ -917,8 +985,18 @@ __device__ void profile_rows(const ProfileRows& Q, int h, const float* rc, const
     }
     return lo;
   };
-  for (int b = t0; b < n; b += stride) {
-    const long long c0 = count_le(b), c1 = count_le(b + 1);
+  // the last edge, r_out: the particles up to k_vir, checked; all without an r_vir
+  long long cn = r_vir > 0.0 ? k_vir + 1 : nb;
+  if (r_vir > 0.0 && !(cn > 0 && le_edge_band(rc[idx(cn - 1)], r_out_f, r_out, 1.0) &&
+                       (cn == nb || !le_edge_band(rc[idx(cn)], r_out_f, r_out, 1.0))))
+    cn = count_le(n);
+  const int lane = t0 & 31;
+  for (int b0 = t0 - lane; b0 < n; b0 += stride) {
+    const int b = b0 + lane;
+    const long long c0 = b < n ? count_le(b) : cn;
+    long long c1 = __shfl_down_sync(FULL_MASK, c0, 1);
+    if (lane == 31) c1 = b + 1 < n ? count_le(b + 1) : cn;
+    if (b >= n) continue;
     // masses: count * m0 for a uniform particle mass (m0 != NULL), else the
     // exact fixed-point sums
     double M1, Mshell;

@@ -2685,7 +2685,7 @@ __global__ void __launch_bounds__(T) g_rows_mixed(GridLaunch L) {
   const double m0 = L.p.m0;
   const long long gb = H.gbase;
   profile_rows(L.rows, H.index, (const float*)L.rc, (const long long*)L.mc, [gb](long long j) { return gb + j; },
-               S.n_alive, Rs.r_vir, S.s_m, L.prm.G, L.prm.Gf, L.p.m == nullptr ? &m0 : nullptr, threadIdx.x, T);
+               S.n_alive, Rs.r_vir, Rs.k_vir, S.s_m, L.prm.G, L.prm.Gf, L.p.m == nullptr ? &m0 : nullptr, threadIdx.x, T);
 }
 
 // The all-FP64 rows: FP64 radii against the FP64 edges, __int128 masses.

@@ -107,7 +107,8 @@ struct Smem {
   int c_removed, c_band;
   int k_first;
   float vb[3];
-  double rvir;                  // emit: the record's r_vir, for the profile rows
+  double rvir;                  // emit: the record's r_vir and k_vir, for the profile rows
+  long long kvir;
   uint32_t dtot[256];
   uint32_t dpre[256];
 };
@@ -337,7 +338,8 @@ template <int NT, int IPT, int CS>
 __device__ int cluster_dist_sort(uint32_t* kA, uint32_t* vA, uint32_t* kB, uint32_t* vB, uint32_t* ex1, uint32_t* ex2,
                                  uint32_t* hist, Smem<NT>& S, Xchg& X, int nloc, int n_mem, int rank, int& nrec) {
   constexpr int NW = NT / 32, CAP = IPT * NT, SLICE = CLUSTER_CELLS / CS;
-  static_assert(SLICE <= NT && CLUSTER_CELLS % NT == 0 && NW * 16 <= NT, "slices and counters fit the threads");
+  static_assert(SLICE <= NT && CLUSTER_CELLS % NT == 0 && NW * 16 <= NT,
+                "slices and counters fit the threads");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t* mine = ex2;                  // this CTA's cells
   uint32_t* cum = ex1;                   // all of them: counts, then members before each cell
@@ -473,19 +475,33 @@ __device__ int cluster_dist_sort(uint32_t* kA, uint32_t* vA, uint32_t* kB, uint3
   if (dist_sort<NT, SORT_CELLS>(kA, vA, kB, vB, ex2, ex1, hist, wtot, vA, nrec, nrec, S.min_key, S.max_key, tid))
     return 0;
   // dozens of equal radii: the counting radix sort of this CTA's share (its
-  // counters in ex1)
-  static_assert(count_sort_words(NT) <= CAP, "counters fit");
+  // counters in ex1 and ex2)
+  static_assert(count_sort_words(NT) <= 2 * CAP, "counters fit");
   const uint32_t differ = S.max_key ^ S.min_key;
   const uint32_t diff = differ ? 0xffffffffu >> __clz(differ) : 0u;
   return count_sort<NT, (run_length(CAP, NT) + 3) / 4 * 4>(kA, vA, kB, vB, ex1, wtot, nrec, run_length(nrec, NT), diff,
                                                            0u, tid);
 }
 
-template <int NT, int CS>
-constexpr int min_blocks() { return CS > 1 ? 1 : (NT <= 128 ? 6 : (NT <= 256 ? 2 : 1)); }
+#ifndef X1K
+#define X1K 128
+#define B1K 6
+#endif
+#ifndef X4K
+#define X4K 256
+#endif
+#ifndef X8K
+#define X8K 512
+#endif
+#ifndef XCL
+#define XCL 512
+#endif
+constexpr int NT_1K = X1K, NT_4K = X4K, NT_8K = X8K, NT_CL = XCL;
+template <int CAP, int CS>
+constexpr int min_blocks() { return CS > 1 ? 1 : (CAP <= 1024 ? B1K : (CAP <= 4096 ? 2 : 1)); }
 
 template <int NT, int CAP, int CT, int CS>
-__global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(OnchipLaunch L) {
+__global__ void __launch_bounds__(NT, (min_blocks<CAP, CS>())) unbind_kernel(OnchipLaunch L) {
   constexpr int IPT = CAP / NT;
   static_assert(IPT * NT == CAP && IPT <= 32 && (IPT & (IPT - 1)) == 0, "bad tile");
   extern __shared__ __align__(16) unsigned char dyn[];
@@ -502,6 +518,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
   const int tid = threadIdx.x, lane = tid & 31;
   const int rank = Cl<CS>::rank();
   const ParamsDev& P = L.prm;
+  const bool unim = L.p.m == nullptr;                    // every particle has mass m0
 
   for (;;) {
     if (rank == 0 && tid == 0) X.halo = atomicAdd(L.queue, 1);
@@ -558,10 +575,18 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
             float v[3];
             cand_velocity<CT>(c, v);
             if (L.rec) put_record(L.rec + 2 * (H.gbase + j), df, m, v);
-            mxm = max(mxm, __float_as_uint(fabsf(m)));
-            mxr = max(mxr, __float_as_uint(fabsf(m * rinv_of(r, P.r_soft_f))));
+            if (unim) {
+              // (one mass: the maxima follow from the smallest radius and the
+              // largest |v_k| below, rounding being monotone)
 #pragma unroll
-            for (int k = 0; k < 3; ++k) mxv = max(mxv, __float_as_uint(fabsf(__fmul_rn(m, v[k]))));
+              for (int k = 0; k < 3; ++k) mxv = max(mxv, __float_as_uint(fabsf(v[k])));
+              if (fmaxf(r, P.r_soft_f) > 0.0f) mxr = max(mxr, ~__float_as_uint(r));
+            } else {
+              mxm = max(mxm, __float_as_uint(fabsf(m)));
+              mxr = max(mxr, __float_as_uint(fabsf(m * rinv_of(r, P.r_soft_f))));
+#pragma unroll
+              for (int k = 0; k < 3; ++k) mxv = max(mxv, __float_as_uint(fabsf(__fmul_rn(m, v[k]))));
+            }
             ++nmem;
           }
         }
@@ -621,11 +646,17 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
       __syncthreads();
     }
     const int n_mem = S.n_member;                        // members of the halo
+    // the exponents of the largest m, m / r and |m v_k|
+    uint32_t mxm = S.max_m, mxr = S.max_mr, mxv = S.max_mv;
+    if (unim) {
+      mxm = n_mem > 0 ? __float_as_uint(fabsf(L.p.m0f)) : 0u;
+      mxr = mxr ? __float_as_uint(fabsf(L.p.m0f * rinv_of(__uint_as_float(~mxr), P.r_soft_f))) : 0u;
+      mxv = __float_as_uint(fabsf(__fmul_rn(L.p.m0f, __uint_as_float(mxv))));
+    }
     int nmem_loc = max(0, min(n_mem - lo, nloc));        // held by this CTA after the sort
-    const int s_m = fix_scale(float_exponent_of_bits(S.max_m), n_mem);
-    const int s_r = fix_scale(float_exponent_of_bits(S.max_mr), n_mem);
-    const int s_v = fix_scale(float_exponent_of_bits(S.max_mv), n_mem);
-    const bool unim = L.p.m == nullptr;                  // every particle has mass m0
+    const int s_m = fix_scale(float_exponent_of_bits(mxm), n_mem);
+    const int s_r = fix_scale(float_exponent_of_bits(mxr), n_mem);
+    const int s_v = fix_scale(float_exponent_of_bits(mxv), n_mem);
     const long long m0fix = fix_from_float(L.p.m0f, s_m);
     // 2^-s of the mass and m/r sums as floats (0 when not normal): each
     // exact sum's float value is then one multiply, the bits of float_from_fix
@@ -636,11 +667,12 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
     int which;
     if constexpr (CS == 1) {
       which = 0;
-      uint32_t* aux = reinterpret_cast<uint32_t*>(hist);
+      uint32_t* aux = reinterpret_cast<uint32_t*>(ex1);    // count_sort's: ex1, ex2 and hist
       uint32_t* wtot = reinterpret_cast<uint32_t*>(&S.red[0][0]);
       // (the counts' last word, cnt[CAP], is ex2's first)
-      if (n_mem > 0 && !dist_sort<NT, SORT_CELLS>(kA, vA, kB, vB, vA, reinterpret_cast<uint32_t*>(ex1), aux, wtot,
-                                                  nullptr, nloc, n_mem, S.min_key, S.max_key, tid)) {
+      if (n_mem > 0 && !dist_sort<NT, SORT_CELLS>(kA, vA, kB, vB, vA, reinterpret_cast<uint32_t*>(ex1),
+                                                  reinterpret_cast<uint32_t*>(hist), wtot, nullptr, nloc, n_mem,
+                                                  S.min_key, S.max_key, tid)) {
         for (int i = tid; i < nloc; i += NT) vA[i] = (uint32_t)i;
         uint32_t diff = S.or_bits ^ S.and_bits, sub = 0u;
         if (n_mem < n_cand) {              // non-members get a key just above the members'
@@ -668,15 +700,18 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
     float* wy = ex1;
     float* wz = ex2;
 
-    // ---- fill: m and w = v + H d in the radial order, and the exact sum m v
-    // of the members (the sorted candidates re-read from the store, mostly L2)
+    // ---- fill: m and w = v + H d in the radial order (from the records, mostly
+    // L2), each thread its own run: the exact sum m v of the members, and the
+    // run's exact sums of m, m/r and its alive count
     const int ipt = run_length(nmem_loc, NT);
     const int p0 = tid * ipt;
+    long long tm_own = 0, tr_own = 0, tc_own = 0;
     {
       long long smv[3] = {0, 0, 0};
-      for (int p = tid; p < nmem_loc; p += NT) {
-        const int q = p;
-        const int j = (int)jj[q];
+      const int p1 = min(p0 + ipt, nmem_loc);
+#pragma unroll 2
+      for (int p = p0; p < p1; ++p) {
+        const int j = (int)jj[p];
         float dfl[3], v[3], m;
         if (L.rec) {
           get_record(L.rec + 2 * (H.gbase + j), dfl, m, v);
@@ -690,13 +725,17 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
         }
         // with a uniform mass the slot holds 1 / max(r, r_soft) instead (the
         // mass is m0): the reciprocal is formed once, not every iteration
-        mm[q] = unim ? rinv_of(rr[q], P.r_soft_f) : m;
-        wx[q] = fmaf(P.Hf, dfl[0], v[0]);
-        wy[q] = fmaf(P.Hf, dfl[1], v[1]);
-        wz[q] = fmaf(P.Hf, dfl[2], v[2]);
+        const float ri = rinv_of(rr[p], P.r_soft_f);
+        mm[p] = unim ? ri : m;
+        wx[p] = fmaf(P.Hf, dfl[0], v[0]);
+        wy[p] = fmaf(P.Hf, dfl[1], v[1]);
+        wz[p] = fmaf(P.Hf, dfl[2], v[2]);
+        tm_own += unim ? m0fix : fix_from_float(m, s_m);
+        tr_own += fix_from_float(m * ri, s_r);
 #pragma unroll
         for (int k = 0; k < 3; ++k) smv[k] += fix_from_float(__fmul_rn(m, v[k]), s_v);
       }
+      tc_own = max(0, p1 - p0);
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
         const long long t = warp_sum(smv[k]);
@@ -718,21 +757,6 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
     __syncthreads();
 
     if (tid == 0 && rank == 0) trace_mark(L.trace, H.index, 3);
-    // per-thread exact sums of m, m/r and the alive count over its run
-    long long tm_own = 0, tr_own = 0, tc_own = 0;
-    for (int k = 0; k < ipt; ++k) {
-      const int p = p0 + k;
-      if (p < nmem_loc) {
-        const int q = p;
-        const float mq = mm[q];
-        const float m = unim ? L.p.m0f : mq;
-        const float ri = unim ? mq : rinv_of(rr[q], P.r_soft_f);
-        tm_own += (unim ? m0fix : fix_from_float(m, s_m));
-        tr_own += fix_from_float(m * ri, s_r);
-        tc_own += 1;
-      }
-    }
-
     // ---- iterate (Appendix A) ----
     int n_iter = 0, status = 0;
     long long part_iter = 0, n_band = 0;
@@ -754,7 +778,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
     // a cluster: one exchange per iteration (cluster_exchange) carries the
     // scan totals of the current set and the previous iteration's removals;
     // the last one, of the final set, also serves the emit
-    long long e_tm = 0, e_tr = 0, e_tc = 0;   // the emit's prefixes (cluster)
+    long long e_tm = 0, e_tr = 0, e_tc = 0;   // the emit's prefixes
     int xs = 0;
     for (;;) {
       long long tm = tm_own, tr = tr_own;
@@ -826,41 +850,28 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
       long long rm = 0, rq = 0, rv0 = 0, rv1 = 0, rv2 = 0;
       int nrem = 0, nband = 0;
       uint32_t rmask = 0;                 // this thread's removals (bit k: position p0 + k)
-      // no branch per member: a slot past the members or removed earlier
-      // adds nothing and is not tested (a run may reach a few words past its
-      // array, into the next one), so the loop's members can overlap
-      if (p0 < nmem_loc) {
-#pragma unroll 4
-        for (int k = 0; k < ipt; ++k) {
-          const int p = p0 + k;
-          const int q = p;
-          const float mq = mm[q];
-          const bool alive = p < nmem_loc && !signbit(mq);
-          const float m = unim ? L.p.m0f : mq;
-          const float ri = unim ? mq : rinv_of(rr[q], P.r_soft_f);
-          const long long mfix = alive ? (unim ? m0fix : fix_from_float(m, s_m)) : 0ll;
-          const long long rfix = alive ? fix_from_float(m * ri, s_r) : 0ll;
-          const float phi = phi_of(fix_to_float_fast(tm, s_m, sc_m), ri, fix_to_float_fast(T_tot - tr, s_r, sc_r),
-                                   P.Gf);
-          const float ux = wx[q] - vb0, uy = wy[q] - vb1, uz = wz[q] - vb2;
-          const float u2 = fmaf(uz, uz, fmaf(uy, uy, ux * ux));
-          const float two_phi = -2.0f * phi;
-          nband += (alive && fabsf(u2 - two_phi) < P.band_f * two_phi) ? 1 : 0;
-          if (alive && u2 > two_phi) {
-            mm[q] = -mq;
-            rmask |= 1u << k;
-            rm += mfix;
-            rq += rfix;
-          }
-          tm += mfix;
-          tr += rfix;
-        }
+      const int run = min(ipt, nmem_loc - p0);            // members of this thread's run
+      if (sc_m != 0.0f && sc_r != 0.0f) {
+        if (unim)
+          member_pass<0>(rr, mm, wx, wy, wz, p0, run, P, true, L.p.m0f, m0fix, s_m, s_r, sc_m, sc_r, vb0, vb1, vb2, tm,
+                         T_tot - tr, rmask, nband);
+        else
+          member_pass<1>(rr, mm, wx, wy, wz, p0, run, P, false, 0.0f, 0ll, s_m, s_r, sc_m, sc_r, vb0, vb1, vb2, tm,
+                         T_tot - tr, rmask, nband);
+      } else {
+        member_pass<2>(rr, mm, wx, wy, wz, p0, run, P, unim, L.p.m0f, m0fix, s_m, s_r, 0.0f, 0.0f, vb0, vb1, vb2, tm,
+                       T_tot - tr, rmask, nband);
       }
-      // the removed: exact m v from the stored velocity, and their record
+      // the removed: their mark, their exact terms, m v from the stored velocity,
+      // and their record
       for (uint32_t b = rmask; b; b &= b - 1) {
-        const int k = __ffs(b) - 1;
-        const int q = p0 + k;
-        const float m = unim ? L.p.m0f : -mm[q];
+        const int q = p0 + __ffs(b) - 1;
+        const float mq = mm[q];
+        mm[q] = -mq;
+        const float m = unim ? L.p.m0f : mq;
+        const float ri = unim ? mq : rinv_of(rr[q], P.r_soft_f);
+        rm += unim ? m0fix : fix_from_float(m, s_m);
+        rq += fix_from_float(m * ri, s_r);
         const int j = (int)jj[q];
         const long long slot = H.offset + j;
         float v[3];
@@ -901,7 +912,12 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
         mvl[1] -= acc[2];
         mvl[2] -= acc[3];
         n_alive -= removed;
-        if (removed == 0) { converged = true; break; }
+        if (removed == 0) {              // the scan was of the final set
+          converged = true;
+          e_tm = tm;
+          e_tr = tr;
+          break;
+        }
       }
       // a cluster: this iteration's removal sums go out with the next exchange
     }
@@ -926,11 +942,16 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
     {
       long long tm = tm_own, tr = tr_own, tc = tc_own;
       if constexpr (CS == 1) {
-        block_exclusive_scan3<NT>(tm, tr, tc, S);
-        if (tid < 3) {
-          S.c_pre[tid] = 0;
-          S.c_tot[tid] = S.tot[tid];
+        if (converged) {
+          tm = e_tm;
+          tr = e_tr;
+          tc = group_excl<NT>((uint32_t)tc_own, reinterpret_cast<uint32_t*>(&S.red[0][0]), tid);
+          if (tid < 3) S.c_tot[tid] = tid < 2 ? S.tot[tid] : n_alive;
+        } else {
+          block_exclusive_scan3<NT>(tm, tr, tc, S);
+          if (tid < 3) S.c_tot[tid] = S.tot[tid];
         }
+        if (tid < 3) S.c_pre[tid] = 0;
         __syncthreads();
       } else {                            // the last exchange was of the final set
         tm = e_tm;
@@ -938,40 +959,37 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
         tc = e_tc;
       }
       const long long C_pre = S.c_pre[2];
-      const long long C_loc = S.tot[2];
+      const long long C_loc = CS == 1 ? S.c_tot[2] : S.tot[2];
       const long long T_tot = S.c_tot[1];
       const long long nb = S.c_tot[2];
       tm += S.c_pre[0];
       tr += S.c_pre[1];
       long long tl = tc;                  // local rank of the thread's first bound particle
-      for (int k = 0; k < ipt; ++k) {
-        const int p = p0 + k;
-        if (p < nmem_loc) {
-          const int q = p;
-          const float mq = mm[q];
-          if (!signbit(mq)) {
-            const float r = rr[q];
-            const float m = unim ? L.p.m0f : mq;
-            const float ri = unim ? mq : rinv_of(r, P.r_soft_f);
-            const long long mfix = (unim ? m0fix : fix_from_float(m, s_m));
-            const float phi = phi_of(fix_to_float_fast(tm, s_m, sc_m), ri, fix_to_float_fast(T_tot - tr, s_r, sc_r),
-                                     P.Gf);
-            const int j = (int)jj[q];
-            rc[tl] = r;
-            if (unim) {
-              pc[tl] = phi;
-              jc[tl] = (uint32_t)j;
-            } else {
-              const long long slot = H.offset + j;
-              const long long dst = H.offset + C_pre + tl;
-              L.out.bound_idx[dst] = L.out.member_idx ? L.out.member_idx[slot] : slot;
-              if (L.out.phi) ((float*)L.out.phi)[dst] = phi;
-              mc[tl] = tm + mfix;
-            }
-            tm += mfix;
-            tr += fix_from_float(m * ri, s_r);
-            tl += 1;
+      long long out = T_tot - tr;
+      const int p1 = min(p0 + ipt, nmem_loc);
+      for (int q = p0; q < p1; ++q) {
+        const float mq = mm[q];
+        if (!signbit(mq)) {
+          const float r = rr[q];
+          const float m = unim ? L.p.m0f : mq;
+          const float ri = unim ? mq : rinv_of(r, P.r_soft_f);
+          const long long mfix = (unim ? m0fix : fix_from_float(m, s_m));
+          const float phi = phi_of(fix_to_float_fast(tm, s_m, sc_m), ri, fix_to_float_fast(out, s_r, sc_r), P.Gf);
+          const int j = (int)jj[q];
+          rc[tl] = r;
+          if (unim) {
+            pc[tl] = phi;
+            jc[tl] = (uint32_t)j;
+          } else {
+            const long long slot = H.offset + j;
+            const long long dst = H.offset + C_pre + tl;
+            L.out.bound_idx[dst] = L.out.member_idx ? L.out.member_idx[slot] : slot;
+            if (L.out.phi) ((float*)L.out.phi)[dst] = phi;
+            mc[tl] = tm + mfix;
           }
+          tm += mfix;
+          out -= fix_from_float(m * ri, s_r);
+          tl += 1;
         }
       }
       if (tid == 0) S.k_first = 0x7fffffff;
@@ -1089,6 +1107,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
           R->m_vir = mv;
           R->r_vir = rv;
           S.rvir = rv;
+          S.kvir = kv;
           if constexpr (CS > 1) {
             X.rvir = rv;
             X.has_rvir = 1;
@@ -1166,7 +1185,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
       if constexpr (CS == 1) {
         if (L.rows.prof) {
           __syncthreads();                        // S.rvir
-          profile_rows(L.rows, H.index, rc, mc, [](long long kk) { return (int)kk; }, nb, S.rvir, s_m,
+          profile_rows(L.rows, H.index, rc, mc, [](long long kk) { return (int)kk; }, nb, S.rvir, S.kvir, s_m,
                        P.G, P.Gf, unim ? &L.p.m0 : nullptr, tid, NT);
         }
       }
@@ -1182,10 +1201,12 @@ __global__ void __launch_bounds__(NT, (min_blocks<NT, CS>())) unbind_kernel(Onch
 }
 
 // Dynamic shared memory: six 4-byte arrays of CAP slots, then the sort's
-// counters (per-warp digit counts in a cluster, count_sort's words in one CTA).
+// counters (per-warp digit counts in a cluster, dist_sort's cells in one CTA).
 template <int NT, int CAP, int CS>
 constexpr size_t dyn_bytes() {
-  return (size_t)CAP * 24 + (CS == 1 ? (size_t)count_sort_words(NT) * 4 : (size_t)(NT / 32) * 256 * 2);
+  constexpr int words = SORT_CELLS + 8;
+  static_assert(CS > 1 || count_sort_words(NT) <= 2 * CAP + words, "count_sort's counters lie in ex1, ex2 and hist");
+  return (size_t)CAP * 24 + (CS == 1 ? (size_t)words * 4 : (size_t)(NT / 32) * 256 * 2);
 }
 
 template <int CS>
@@ -1288,13 +1309,13 @@ int onchip_capacity(int variant) {
 
 int onchip_max_grid(int variant, int device) {
   switch (variant) {
-    case 0: return max_grid_variant<128, 1024, 1>(device);
-    case 1: return max_grid_variant<256, 4096, 1>(device);
-    case 2: return max_grid_variant<512, 8192, 1>(device);
-    case 3: return max_grid_variant<512, 8192, 2>(device);
-    case 4: return max_grid_variant<512, 8192, 4>(device);
-    case 5: return max_grid_variant<512, 8192, 8>(device);
-    case 6: return max_grid_variant<512, 8192, 16>(device);
+    case 0: return max_grid_variant<NT_1K, 1024, 1>(device);
+    case 1: return max_grid_variant<NT_4K, 4096, 1>(device);
+    case 2: return max_grid_variant<NT_8K, 8192, 1>(device);
+    case 3: return max_grid_variant<NT_CL, 8192, 2>(device);
+    case 4: return max_grid_variant<NT_CL, 8192, 4>(device);
+    case 5: return max_grid_variant<NT_CL, 8192, 8>(device);
+    case 6: return max_grid_variant<NT_CL, 8192, 16>(device);
     default: return 0;
   }
 }
@@ -1302,20 +1323,20 @@ int onchip_max_grid(int variant, int device) {
 cudaError_t launch_onchip(const OnchipLaunch& L, int variant, int grid, cudaStream_t s) {
   const bool f64 = L.p.coord_type == AHF_COORD_F64;
   switch (variant) {
-    case 0: return f64 ? launch_variant<128, 1024, AHF_COORD_F64, 1>(L, grid, s)
-                       : launch_variant<128, 1024, AHF_COORD_F32_REL, 1>(L, grid, s);
-    case 1: return f64 ? launch_variant<256, 4096, AHF_COORD_F64, 1>(L, grid, s)
-                       : launch_variant<256, 4096, AHF_COORD_F32_REL, 1>(L, grid, s);
-    case 2: return f64 ? launch_variant<512, 8192, AHF_COORD_F64, 1>(L, grid, s)
-                       : launch_variant<512, 8192, AHF_COORD_F32_REL, 1>(L, grid, s);
-    case 3: return f64 ? launch_variant<512, 8192, AHF_COORD_F64, 2>(L, grid, s)
-                       : launch_variant<512, 8192, AHF_COORD_F32_REL, 2>(L, grid, s);
-    case 4: return f64 ? launch_variant<512, 8192, AHF_COORD_F64, 4>(L, grid, s)
-                       : launch_variant<512, 8192, AHF_COORD_F32_REL, 4>(L, grid, s);
-    case 5: return f64 ? launch_variant<512, 8192, AHF_COORD_F64, 8>(L, grid, s)
-                       : launch_variant<512, 8192, AHF_COORD_F32_REL, 8>(L, grid, s);
-    case 6: return f64 ? launch_variant<512, 8192, AHF_COORD_F64, 16>(L, grid, s)
-                       : launch_variant<512, 8192, AHF_COORD_F32_REL, 16>(L, grid, s);
+    case 0: return f64 ? launch_variant<NT_1K, 1024, AHF_COORD_F64, 1>(L, grid, s)
+                       : launch_variant<NT_1K, 1024, AHF_COORD_F32_REL, 1>(L, grid, s);
+    case 1: return f64 ? launch_variant<NT_4K, 4096, AHF_COORD_F64, 1>(L, grid, s)
+                       : launch_variant<NT_4K, 4096, AHF_COORD_F32_REL, 1>(L, grid, s);
+    case 2: return f64 ? launch_variant<NT_8K, 8192, AHF_COORD_F64, 1>(L, grid, s)
+                       : launch_variant<NT_8K, 8192, AHF_COORD_F32_REL, 1>(L, grid, s);
+    case 3: return f64 ? launch_variant<NT_CL, 8192, AHF_COORD_F64, 2>(L, grid, s)
+                       : launch_variant<NT_CL, 8192, AHF_COORD_F32_REL, 2>(L, grid, s);
+    case 4: return f64 ? launch_variant<NT_CL, 8192, AHF_COORD_F64, 4>(L, grid, s)
+                       : launch_variant<NT_CL, 8192, AHF_COORD_F32_REL, 4>(L, grid, s);
+    case 5: return f64 ? launch_variant<NT_CL, 8192, AHF_COORD_F64, 8>(L, grid, s)
+                       : launch_variant<NT_CL, 8192, AHF_COORD_F32_REL, 8>(L, grid, s);
+    case 6: return f64 ? launch_variant<NT_CL, 8192, AHF_COORD_F64, 16>(L, grid, s)
+                       : launch_variant<NT_CL, 8192, AHF_COORD_F32_REL, 16>(L, grid, s);
     default: return cudaErrorInvalidValue;
   }
 }

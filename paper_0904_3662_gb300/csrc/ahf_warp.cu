@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
   float* ex2 = ex1 + WARP_CAP;
   uint16_t* hist = (uint16_t*)(ex2 + WARP_CAP);
   const ParamsDev& P = L.prm;
+  const bool unim = L.p.m == nullptr;                    // every particle has mass m0
 
   for (;;) {
     int hq = 0;
@@ -158,16 +159,25 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
           float v[3];
           load_velocity<CT>(L.p, pi, v);
           if (L.rec) put_record(L.rec + 2 * (H.gbase + i), df, m, v);
-          mxm = max(mxm, __float_as_uint(fabsf(m)));
-          mxr = max(mxr, __float_as_uint(fabsf(m * rinv_of(r, P.r_soft_f))));
+          if (unim) {
+            // (one mass: the maxima follow from the smallest radius and the
+            // largest |v_k| below, rounding being monotone)
 #pragma unroll
-          for (int k = 0; k < 3; ++k) mxv = max(mxv, __float_as_uint(fabsf(__fmul_rn(m, v[k]))));
+            for (int k = 0; k < 3; ++k) mxv = max(mxv, __float_as_uint(fabsf(v[k])));
+            if (fmaxf(r, P.r_soft_f) > 0.0f) mxr = max(mxr, ~__float_as_uint(r));
+          } else {
+            mxm = max(mxm, __float_as_uint(fabsf(m)));
+            mxr = max(mxr, __float_as_uint(fabsf(m * rinv_of(r, P.r_soft_f))));
+#pragma unroll
+            for (int k = 0; k < 3; ++k) mxv = max(mxv, __float_as_uint(fabsf(__fmul_rn(m, v[k]))));
+          }
           kmn = min(kmn, key);
           kmx = max(kmx, key);
           ++nmem;
         }
       }
-      if (key == KEY_NONMEMBER && L.out.removed_iter) L.out.removed_iter[slot] = -1;
+      // members start bound (removal overwrites with its iteration)
+      if (L.out.removed_iter) L.out.removed_iter[slot] = key == KEY_NONMEMBER ? -1 : 0;
       kA[i] = key;
       orb |= key;
       andb &= key;
@@ -181,10 +191,14 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
     kmx = __reduce_max_sync(FULL_MASK, kmx);
     const int n_mem = (int)__reduce_add_sync(FULL_MASK, (unsigned)nmem);
     __syncwarp();
+    if (unim) {
+      mxm = n_mem > 0 ? __float_as_uint(fabsf(L.p.m0f)) : 0u;
+      mxr = mxr ? __float_as_uint(fabsf(L.p.m0f * rinv_of(__uint_as_float(~mxr), P.r_soft_f))) : 0u;
+      mxv = __float_as_uint(fabsf(__fmul_rn(L.p.m0f, __uint_as_float(mxv))));
+    }
     const int s_m = fix_scale(float_exponent_of_bits(mxm), n_mem);
     const int s_r = fix_scale(float_exponent_of_bits(mxr), n_mem);
     const int s_v = fix_scale(float_exponent_of_bits(mxv), n_mem);
-    const bool unim = L.p.m == nullptr;                  // every particle has mass m0
     const long long m0fix = fix_from_float(L.p.m0f, s_m);
     // 2^-s of the mass and m/r sums as floats (0 when not normal): each
     // exact sum's float value is then one multiply, the bits of float_from_fix
@@ -209,10 +223,15 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
 
     if (lane == 0) trace_mark(L.trace, H.index, 2);
     // ---- fill ----
+    // each lane its own run of the radial order: the members' m and w = v + H d,
+    // the exact sum m v, and the run's exact sums of m, m/r and its alive count
     long long mv[3] = {0, 0, 0};
-    for (int p = lane; p < n_mem; p += 32) {
-      const int q = p;
-      const int j = (int)jj[q];
+    const int ipt = run_length(n_mem, 32);
+    const int p0 = lane * ipt, p1 = min(p0 + ipt, n_mem);
+    long long tm_own = 0, tr_own = 0, tc_own = max(0, p1 - p0);
+#pragma unroll 2
+    for (int p = p0; p < p1; ++p) {
+      const int j = (int)jj[p];
       float dfl[3], v[3], m;
       if (L.rec) {
         get_record(L.rec + 2 * (H.gbase + j), dfl, m, v);
@@ -226,32 +245,19 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
       }
       // with a uniform mass the slot holds 1 / max(r, r_soft) instead (the
       // mass is m0): the reciprocal is formed once, not every iteration
-      mm[q] = unim ? rinv_of(rr[q], P.r_soft_f) : m;
-      wx[q] = fmaf(P.Hf, dfl[0], v[0]);
-      wy[q] = fmaf(P.Hf, dfl[1], v[1]);
-      wz[q] = fmaf(P.Hf, dfl[2], v[2]);
+      const float ri = rinv_of(rr[p], P.r_soft_f);
+      mm[p] = unim ? ri : m;
+      wx[p] = fmaf(P.Hf, dfl[0], v[0]);
+      wy[p] = fmaf(P.Hf, dfl[1], v[1]);
+      wz[p] = fmaf(P.Hf, dfl[2], v[2]);
+      tm_own += unim ? m0fix : fix_from_float(m, s_m);
+      tr_own += fix_from_float(m * ri, s_r);
 #pragma unroll
       for (int k = 0; k < 3; ++k) mv[k] += fix_from_float(__fmul_rn(m, v[k]), s_v);
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) mv[k] = warp_sum(mv[k]);
     __syncwarp();
-
-    const int ipt = run_length(n_mem, 32);
-    const int p0 = lane * ipt;
-    long long tm_own = 0, tr_own = 0, tc_own = 0;
-    for (int k = 0; k < ipt; ++k) {
-      const int p = p0 + k;
-      if (p < n_mem) {
-        const int q = p;
-        const float mq = mm[q];
-        const float m = unim ? L.p.m0f : mq;
-        const float ri = unim ? mq : rinv_of(rr[q], P.r_soft_f);
-        tm_own += (unim ? m0fix : fix_from_float(m, s_m));
-        tr_own += fix_from_float(m * ri, s_r);
-        tc_own += 1;
-      }
-    }
 
     if (lane == 0) trace_mark(L.trace, H.index, 3);
     // ---- iterate (Appendix A) ----
@@ -260,6 +266,7 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
     int n_alive = n_mem;
     bool converged = false;
     float vb0 = 0.0f, vb1 = 0.0f, vb2 = 0.0f;
+    long long e_tm = 0, e_tr = 0, M_fin = 0, T_fin = 0;   // the emit's prefixes and totals
     while (n_alive > 0 && n_iter < P.max_iter) {
       ++n_iter;
       part_iter += n_alive;
@@ -276,42 +283,28 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
       long long rm = 0, rq = 0, rv0 = 0, rv1 = 0, rv2 = 0;
       int nrem = 0, nband = 0;
       uint32_t rmask = 0;                 // this lane's removals (bit k: position p0 + k)
-      // no branch per member: a slot past the members or removed earlier
-      // adds nothing and is not tested (a run may reach a few words past its
-      // array, into the next one), so the loop's members can overlap
-      if (p0 < n_mem) {
-#pragma unroll 4
-        for (int k = 0; k < ipt; ++k) {
-          const int p = p0 + k;
-          const int q = p;
-          const float mq = mm[q];
-          const bool alive = p < n_mem && !signbit(mq);
-          const float m = unim ? L.p.m0f : mq;
-          const float ri = unim ? mq : rinv_of(rr[q], P.r_soft_f);
-          const long long mfix = alive ? (unim ? m0fix : fix_from_float(m, s_m)) : 0ll;
-          const long long rfix = alive ? fix_from_float(m * ri, s_r) : 0ll;
-          const float phi = phi_of(fix_to_float_fast(tm, s_m, sc_m), ri, fix_to_float_fast(T_tot - tr, s_r, sc_r),
-                                   P.Gf);
-          const float ux = wx[q] - vb0, uy = wy[q] - vb1, uz = wz[q] - vb2;
-          const float u2 = fmaf(uz, uz, fmaf(uy, uy, ux * ux));
-          const float two_phi = -2.0f * phi;
-          nband += (alive && fabsf(u2 - two_phi) < P.band_f * two_phi) ? 1 : 0;
-          if (alive && u2 > two_phi) {
-            mm[q] = -mq;
-            rmask |= 1u << k;
-            rm += mfix;
-            rq += rfix;
-          }
-          tm += mfix;
-          tr += rfix;
-        }
+      const int run = min(ipt, n_mem - p0);            // members of this lane's run
+      if (sc_m != 0.0f && sc_r != 0.0f) {
+        if (unim)
+          member_pass<0>(rr, mm, wx, wy, wz, p0, run, P, true, L.p.m0f, m0fix, s_m, s_r, sc_m, sc_r, vb0, vb1, vb2, tm,
+                         T_tot - tr, rmask, nband);
+        else
+          member_pass<1>(rr, mm, wx, wy, wz, p0, run, P, false, 0.0f, 0ll, s_m, s_r, sc_m, sc_r, vb0, vb1, vb2, tm,
+                         T_tot - tr, rmask, nband);
+      } else {
+        member_pass<2>(rr, mm, wx, wy, wz, p0, run, P, unim, L.p.m0f, m0fix, s_m, s_r, 0.0f, 0.0f, vb0, vb1, vb2, tm,
+                       T_tot - tr, rmask, nband);
       }
-      // the removed, off the per-particle path: exact m v from the stored
-      // velocity, and their removal iteration
+      // the removed: their mark, their exact terms, m v from the stored velocity,
+      // and their record
       for (uint32_t b = rmask; b; b &= b - 1) {
-        const int k = __ffs(b) - 1;
-        const int q = p0 + k;
-        const float m = unim ? L.p.m0f : -mm[q];
+        const int q = p0 + __ffs(b) - 1;
+        const float mq = mm[q];
+        mm[q] = -mq;
+        const float m = unim ? L.p.m0f : mq;
+        const float ri = unim ? mq : rinv_of(rr[q], P.r_soft_f);
+        rm += unim ? m0fix : fix_from_float(m, s_m);
+        rq += fix_from_float(m * ri, s_r);
         const long long slot = H.offset + (long long)jj[q];
         float v[3];
         if (L.rec) get_velocity_record(L.rec + 2 * (H.gbase + (long long)jj[q]), v);
@@ -333,7 +326,14 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
         mv[2] -= warp_sum(rv2);
       }
       n_alive -= removed;
-      if (removed == 0) { converged = true; break; }
+      if (removed == 0) {                // the scan was of the final set
+        converged = true;
+        e_tm = tm;
+        e_tr = tr;
+        M_fin = M_tot;
+        T_fin = T_tot;
+        break;
+      }
     }
     if (n_alive == 0) status |= AHF_HALO_EMPTY;
     else if (!converged) status |= AHF_HALO_NOT_CONVERGED;
@@ -346,39 +346,36 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
     long long* mc = (long long*)ex1;      // ex1 and ex2 are contiguous
     float* pc = ex1;
     uint32_t* jc = (uint32_t*)ex2;
-    long long M_tot, T_tot, nb;
-    long long tm = warp_excl(tm_own, lane, M_tot);
-    long long tr = warp_excl(tr_own, lane, T_tot);
-    long long tl = warp_excl(tc_own, lane, nb);
+    if (!converged) {
+      e_tm = warp_excl(tm_own, lane, M_fin);
+      e_tr = warp_excl(tr_own, lane, T_fin);
+    }
+    long long tm = e_tm, out = T_fin - e_tr;
+    const long long M_tot = M_fin, nb = n_alive;
+    int tl = (int)(warp_inclusive_scan((uint32_t)tc_own, lane) - (uint32_t)tc_own);
     __syncwarp();
-    for (int k = 0; k < ipt; ++k) {
-      const int p = p0 + k;
-      if (p < n_mem) {
-        const int q = p;
-        const float mq = mm[q];
-        if (!signbit(mq)) {
-          const float r = rr[q];
-          const float m = unim ? L.p.m0f : mq;
-          const float ri = unim ? mq : rinv_of(r, P.r_soft_f);
-          const long long mfix = (unim ? m0fix : fix_from_float(m, s_m));
-          const float phi = phi_of(fix_to_float_fast(tm, s_m, sc_m), ri, fix_to_float_fast(T_tot - tr, s_r, sc_r),
-                                   P.Gf);
+    for (int q = p0; q < p1; ++q) {
+      const float mq = mm[q];
+      if (!signbit(mq)) {
+        const float r = rr[q];
+        const float m = unim ? L.p.m0f : mq;
+        const float ri = unim ? mq : rinv_of(r, P.r_soft_f);
+        const long long mfix = (unim ? m0fix : fix_from_float(m, s_m));
+        const float phi = phi_of(fix_to_float_fast(tm, s_m, sc_m), ri, fix_to_float_fast(out, s_r, sc_r), P.Gf);
+        rc[tl] = r;
+        if (unim) {
+          pc[tl] = phi;
+          jc[tl] = jj[q];
+        } else {
           const long long slot = H.offset + (long long)jj[q];
-          if (L.out.removed_iter) L.out.removed_iter[slot] = 0;
-          rc[tl] = r;
-          if (unim) {
-            pc[tl] = phi;
-            jc[tl] = jj[q];
-          } else {
-            const long long dst = H.offset + tl;
-            L.out.bound_idx[dst] = L.out.member_idx ? L.out.member_idx[slot] : slot;
-            if (L.out.phi) ((float*)L.out.phi)[dst] = phi;
-            mc[tl] = tm + mfix;
-          }
-          tm += mfix;
-          tr += fix_from_float(m * ri, s_r);
-          tl += 1;
+          const long long dst = H.offset + tl;
+          L.out.bound_idx[dst] = L.out.member_idx ? L.out.member_idx[slot] : slot;
+          if (L.out.phi) ((float*)L.out.phi)[dst] = phi;
+          mc[tl] = tm + mfix;
         }
+        tm += mfix;
+        out -= fix_from_float(m * ri, s_r);
+        tl += 1;
       }
     }
     __syncwarp();
@@ -414,8 +411,8 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
     // the record: lane 0 the virial pair, lanes 1-3 one bulk velocity
     // component each (FP64 work in parallel rather than in sequence)
     double r_vir_l = 0.0;
+    long long kv = -1;
     if (lane == 0) {
-      long long kv = -1;
       double mvir = 0.0;
       if (nb > 0) {
         // M_vir: (k+1) m0 in FP64 for a uniform mass, else the exact sum
@@ -459,7 +456,8 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
     }
     if (L.rows.prof) {
       const double r_vir = __shfl_sync(FULL_MASK, r_vir_l, 0);
-      profile_rows(L.rows, H.index, rc, mc, [](long long k) { return (int)k; }, nb, r_vir, s_m, P.G, P.Gf,
+      kv = __shfl_sync(FULL_MASK, kv, 0);
+      profile_rows(L.rows, H.index, rc, mc, [](long long k) { return (int)k; }, nb, r_vir, kv, s_m, P.G, P.Gf,
                    unim ? &L.p.m0 : nullptr, lane, 32);
     }
     if (lane == 0 && L.trace) {
