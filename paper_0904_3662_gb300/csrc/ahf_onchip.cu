@@ -76,10 +76,10 @@ struct Xchg {
   float first_r;                // emit: first compacted radius of this CTA
   int nb_loc;                   // emit: bound particles held by this CTA
   int kf;                       // emit: first local virial crossing (global index)
-  // fused profile rows: r_vir from the owner CTA, last radius, and this CTA's
-  // bound count and inclusive mass at every bin edge
+  // fused profile rows: r_vir and the outermost radius, from the CTAs that hold
+  // them; the bound count at every bin edge (all CTAs', in rank 0) and this CTA's
+  // inclusive mass there
   double rvir;
-  int has_rvir;
   float last_r;
   int pc[FUSE_BINS + 1];
   long long pm[FUSE_BINS + 1];
@@ -1063,7 +1063,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<CAP, CS>())) unbind_kernel(Onc
             const int kl = (int)(k - C_pre);
             // M_vir: (k+1) m0 in FP64 for a uniform mass, else the exact sum
             const long long mkx = unim ? 0 : mc[kl];
-            const double mk = unim ? double_from_fix(k + 1, 0) * L.p.m0 : double_from_fix(mkx, s_m);
+            const double mk = unim ? (double)(k + 1) * L.p.m0 : double_from_fix(mkx, s_m);
             const float mkf = unim ? (float)(k + 1) * L.p.m0f : float_from_fix(mkx, s_m);
             if (k == nb - 1) status |= AHF_HALO_RVIR_BEYOND_EDGE;
             if (below_threshold(mk, mkf, rc[kl], P.crit_f, P.crit)) {
@@ -1086,7 +1086,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<CAP, CS>())) unbind_kernel(Onc
                   }
                   const int l = (int)(p - pre);
                   r = float_to_double(Cl<CS>::at(rc, q)[l]);
-                  m = unim ? double_from_fix(p + 1, 0) * L.p.m0 : double_from_fix(Cl<CS>::at(mc, q)[l], s_m);
+                  m = unim ? (double)(p + 1) * L.p.m0 : double_from_fix(Cl<CS>::at(mc, q)[l], s_m);
                 };
                 const long long ke = rise_edge_index(nb, at);
                 if (ke >= 0) {
@@ -1109,8 +1109,8 @@ __global__ void __launch_bounds__(NT, (min_blocks<CAP, CS>())) unbind_kernel(Onc
           S.rvir = rv;
           S.kvir = kv;
           if constexpr (CS > 1) {
-            X.rvir = rv;
-            X.has_rvir = 1;
+#pragma unroll
+            for (int r2 = 0; r2 < CS; ++r2) Cl<CS>::at(&X, r2)->rvir = rv;
           }
         } else if (tid == 32 || tid == 64 || tid == 96) {
           const int c = tid / 32 - 1;
@@ -1119,48 +1119,38 @@ __global__ void __launch_bounds__(NT, (min_blocks<CAP, CS>())) unbind_kernel(Onc
       }
       if constexpr (CS > 1) {
         if (L.rows.prof && L.rows.n_bins <= FUSE_BINS) {
-          // rows of a halo spread over the cluster: each CTA counts its chunk
-          // of the radial order at every edge; rank 0 adds the counts and
-          // takes the largest inclusive mass (the last particle inside)
-          if (tid == 0) {
-            if (!owner) X.has_rvir = 0;
-            X.last_r = C_loc > 0 ? rc[(int)C_loc - 1] : 0.0f;
-          }
+          // rows of a halo spread over the cluster: each CTA counts its share of
+          // the radial order at every edge and adds that to rank 0's counts; the
+          // inclusive mass is the largest CTA's (the last particle's inside)
+          if (rank == 0)
+            for (int b = tid; b <= L.rows.n_bins; b += NT) X.pc[b] = 0;
+          if (tid < CS && C_loc > 0 && C_pre + C_loc == nb) Cl<CS>::at(&X, tid)->last_r = rc[(int)C_loc - 1];
           Cl<CS>::sync();
-          double r_vir = 0.0;
-          float r_last = 0.0f;
-          for (int r2 = 0; r2 < CS; ++r2) {
-            const Xchg* Y = Cl<CS>::at(&X, r2);
-            if (Y->has_rvir) r_vir = Y->rvir;
-            if (Y->nb_loc > 0) r_last = Y->last_r;
-          }
-          const double r_out = r_vir > 0.0 ? r_vir : float_to_double(r_last);
-          const float r_out_f = double_to_float(r_out);
+          const double r_vir = X.rvir;
+          const double r_out = r_vir > 0.0 ? r_vir : (nb > 0 ? (double)X.last_r : 0.0);
+          const float r_out_f = (float)r_out;
           const int n = L.rows.n_bins;
           for (int b = tid; b <= n; b += NT) {
-            const float ef = b == n ? r_out_f : r_out_f * L.rows.factor_f[b];
-            const double fac = b == n ? 1.0 : L.rows.factor[b];
-            int lo = 0, hi = (int)C_loc;            // first local k with rc[k] > e_b
-            while (lo < hi) {
-              const int mid = (lo + hi) >> 1;
-              if (le_edge_band(rc[mid], ef, r_out, fac)) lo = mid + 1;
-              else hi = mid;
-            }
-            X.pc[b] = lo;
-            X.pm[b] = lo > 0 && !unim ? mc[lo - 1] : 0;
+            const int lo = count_inside(rc, [](int k) { return k; }, (int)C_loc,
+                                        b == n ? r_out_f : r_out_f * L.rows.factor_f[b], r_out,
+                                        b == n ? 1.0 : L.rows.factor[b]);
+            if (lo > 0) atomicAdd(&Cl<CS>::at(&X, 0)->pc[b], lo);
+            if (!unim) X.pm[b] = lo > 0 ? mc[lo - 1] : 0;
           }
           Cl<CS>::sync();
           if (rank == 0) {
             double* out = L.rows.prof + (size_t)H.index * n * 4;
             const float inv_r = 1.0f / r_out_f;
             for (int b = tid; b < n; b += NT) {
-              long long c0 = 0, c1 = 0, f0 = 0, f1 = 0;
-              for (int r2 = 0; r2 < CS; ++r2) {
-                const Xchg* Y = Cl<CS>::at(&X, r2);
-                c0 += Y->pc[b];
-                c1 += Y->pc[b + 1];
-                f0 = max(f0, Y->pm[b]);
-                f1 = max(f1, Y->pm[b + 1]);
+              const long long c0 = X.pc[b], c1 = X.pc[b + 1];
+              long long f0 = 0, f1 = 0;
+              if (!unim) {
+#pragma unroll
+                for (int r2 = 0; r2 < CS; ++r2) {
+                  const Xchg* Y = Cl<CS>::at(&X, r2);
+                  f0 = max(f0, Y->pm[b]);
+                  f1 = max(f1, Y->pm[b + 1]);
+                }
               }
               if (nb == 0) {
                 out[4 * b + 0] = out[4 * b + 1] = out[4 * b + 2] = out[4 * b + 3] = 0.0;
@@ -1168,13 +1158,13 @@ __global__ void __launch_bounds__(NT, (min_blocks<CAP, CS>())) unbind_kernel(Onc
               }
               double M1, Ms;
               if (unim) {
-                M1 = double_from_fix(c1, 0) * L.p.m0;
-                Ms = double_from_fix(c1 - c0, 0) * L.p.m0;
+                M1 = (double)c1 * L.p.m0;
+                Ms = (double)(c1 - c0) * L.p.m0;
               } else {
                 M1 = double_from_fix(f1, s_m);
                 Ms = double_from_fix(f1 - f0, s_m);
               }
-              out[4 * b + 0] = double_from_fix(c1 - c0, 0);
+              out[4 * b + 0] = (double)(c1 - c0);
               out[4 * b + 1] = M1;
               out[4 * b + 2] = shell_density(Ms, r_out, inv_r, L.rows.factor, L.rows.factor_f, n, b);
               out[4 * b + 3] = circular_velocity(P.G, P.Gf, M1, r_out, inv_r, L.rows.factor, L.rows.factor_f, n, b);

@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
       if (nb > 0) {
         // M_vir: (k+1) m0 in FP64 for a uniform mass, else the exact sum
         const long long mkx = unim ? 0 : mc[kf];
-        const double mk = unim ? double_from_fix(kf + 1, 0) * L.p.m0 : double_from_fix(mkx, s_m);
+        const double mk = unim ? (double)(kf + 1) * L.p.m0 : double_from_fix(mkx, s_m);
         const float mkf = unim ? (float)(kf + 1) * L.p.m0f : float_from_fix(mkx, s_m);
         if (kf == nb - 1) status |= AHF_HALO_RVIR_BEYOND_EDGE;
         if (below_threshold(mk, mkf, rc[kf], P.crit_f, P.crit)) {
@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
           if (P.rise_edge && kf == nb - 1) {
             auto at = [&](long long k, double& r, double& m) {
               r = float_to_double(rc[(int)k]);
-              m = unim ? double_from_fix(k + 1, 0) * L.p.m0 : double_from_fix(mc[(int)k], s_m);
+              m = unim ? (double)(k + 1) * L.p.m0 : double_from_fix(mc[(int)k], s_m);
             };
             const long long ke = rise_edge_index(nb, at);
             if (ke >= 0) {
