@@ -285,7 +285,7 @@ int ahf_unbind_profile_batch(ahf_ctx *ctx, const ahf_particles *p, const ahf_hal
  *   AHF_OPT_SERIAL       1 = the on-chip size classes run one after another on
  *                        the caller's stream, so that each phase's events time
  *                        its kernel alone (as a profiler's launch list does);
- *                        0 (default) = concurrently on side streams.  Results
+ *                        0 (default) = concurrently.  Results
  *                        are the same bits either way.
  *   AHF_OPT_PROMOTE      1 (default) = a batch that would leave SMs idle runs its
  *                        haloes in larger size classes (up to two classes up,

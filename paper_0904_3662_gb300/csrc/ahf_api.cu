@@ -928,14 +928,24 @@ int unbind_pass(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64
     AHF_CUDA(cudaMemsetAsync(c->trace_dev, 0, sizeof(long long) * AHF_TRACE_FIELDS * (size_t)n_halos, s));
     c->trace_n = n_halos;
   }
-  // the on-chip variants run on side streams, largest first, concurrently
-  // with the multi-CTA class on the caller's stream
+  // The on-chip variants run as a chain on one stream, largest haloes first: each
+  // launch may start once every CTA of the one before it has started, so the
+  // classes take the SMs in launch order, as a list schedule.  On a stream per
+  // class they took them in the order in which the hardware came to the streams
+  // (a process has 8 queues by default, and the classes that share one waited):
+  // the clusters, which need whole SMs, then ran after the small haloes, 43 us
+  // into the 2,000-halo batch (318 us; 284 as a chain; 11,000 particles in one
+  // halo 70, now 65, without the fork and join; 20,000 haloes even).  With the
+  // multi-CTA class the chain runs on a side stream beside it.  Phase times
+  // (AHF_OPT_TIMING) and outputs pushed to host buffers, which record events or
+  // launch copies between the classes, keep a stream per class.
   struct VLaunch {
     int v, grid, n;
     long long cands;
     OnchipLaunch L;
   };
   std::vector<VLaunch> vl;
+  const bool chain = !c->serial && !c->timing && !push;
   int first_of[NV];
   for (int v = 0, f = 0; v < NV; ++v) { first_of[v] = f; f += P.n_class[v]; }
   // launch order (the block scheduler serves earlier launches first): the
@@ -961,6 +971,8 @@ int unbind_pass(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64
     L.trace = c->trace ? c->trace_dev : nullptr;
     L.variant = v;
     L.rec = drec;
+    L.done = chain ? queues + NV + v : nullptr;
+    L.follow = chain && !vl.empty();
     for (int k = 0; k < n; ++k) x.cands += P.hd[(size_t)first_of[v] + k].count;
     x.grid = (int)std::min<long long>(variant_grid_for(v, n), c->variant_grid[v]);
     vl.push_back(x);
@@ -974,6 +986,18 @@ int unbind_pass(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64
         if ((prc = phase_end(c, x.v, o))) return prc;
         if (push) AHF_CUDA(launch_push(*push, x.L.halos, x.n, P.hd[(size_t)first_of[x.v]].count, o));
       }
+      return AHF_OK;
+    }
+    if (vl.empty()) return AHF_OK;
+    if (chain) {
+      cudaStream_t st = o;
+      if (n_grid) {
+        st = c->side[0];
+        AHF_CUDA(cudaEventRecord(c->fork, o));
+        AHF_CUDA(cudaStreamWaitEvent(st, c->fork, 0));
+      }
+      for (const VLaunch& x : vl) AHF_CUDA(launch_variant(x.L, x.v, x.grid, st));
+      if (n_grid) AHF_CUDA(cudaEventRecord(c->join[0], st));
       return AHF_OK;
     }
     AHF_CUDA(cudaEventRecord(c->fork, o));
@@ -1050,8 +1074,11 @@ int unbind_pass(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64
         c->stats.launches += 1;
       }
     }
-    if (!c->serial)
+    if (chain) {
+      if (n_grid && !vl.empty()) AHF_CUDA(cudaStreamWaitEvent(s, c->join[0], 0));
+    } else if (!c->serial) {
       for (const VLaunch& x : vl) AHF_CUDA(cudaStreamWaitEvent(s, c->join[x.v], 0));
+    }
   }
   if ((rc = end_call(c, s))) return rc;
   if (prof) {

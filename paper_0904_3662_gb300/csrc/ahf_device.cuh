@@ -1045,6 +1045,18 @@ __device__ __forceinline__ int sm_id() {
 }
 
 // Record trace field f of halo h (no-op when tracing is off).
+// Chained launches (OnchipLaunch::done): let the next launch of the stream start
+// beside this one (no effect unless it asks for that) ...
+__device__ __forceinline__ void chain_open() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// ... and keep this one from ending before the launch it follows has, so that the
+// end of a chain is the end of all its launches: the last of the `n` workers to run
+// out of haloes waits, where every other SM is already free for the next class (one
+// thread of each worker calls this; the launch it waits for has all its CTAs on
+// SMs, so the wait ends).
+__device__ __forceinline__ void chain_close(int* done, int n) {
+  if (done && atomicAdd(done, 1) == n - 1) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 __device__ __forceinline__ void trace_mark(long long* trace, int h, int f) {
   if (trace) trace[(size_t)h * AHF_TRACE_FIELDS + f] = global_ns();
 }

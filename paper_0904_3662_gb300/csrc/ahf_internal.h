@@ -167,7 +167,21 @@ struct OnchipLaunch {
   // loads in place of seven scattered 4-byte ones).  NULL: both read the
   // particle store again.
   float4 *rec;
+  // Chained launches: the kernel may start once every CTA of the launch before
+  // it on the stream has started, and ends after that one has ended.  `done`
+  // counts the CTAs (warps of the warp class) that ran out of haloes (zeroed by
+  // the launcher; NULL: no chain).
+  int *done;
+  bool follow;
 };
+
+// add the attribute of a chained launch to cfg's attributes
+inline void follow_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr) {
+  attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs += 1;
+}
 
 // Warp class: one warp per halo of at most warp_capacity() candidates.
 int warp_capacity();

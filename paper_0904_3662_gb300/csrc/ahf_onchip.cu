@@ -520,6 +520,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<CAP, CS>())) unbind_kernel(Onc
   const ParamsDev& P = L.prm;
   const bool unim = L.p.m == nullptr;                    // every particle has mass m0
 
+  chain_open();
   for (;;) {
     if (rank == 0 && tid == 0) X.halo = atomicAdd(L.queue, 1);
     Cl<CS>::sync();
@@ -1188,6 +1189,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<CAP, CS>())) unbind_kernel(Onc
     }
     Cl<CS>::sync();
   }
+  if (tid == 0 && rank == 0) chain_close(L.done, (int)gridDim.x / CS);
 }
 
 // Dynamic shared memory: six 4-byte arrays of CAP slots, then the sort's
@@ -1201,11 +1203,13 @@ constexpr size_t dyn_bytes() {
 
 template <int CS>
 void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr) {
+  cfg.attrs = attr;
+  cfg.numAttrs = 0;
+  if (CS == 1) return;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = CS;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
   cfg.numAttrs = 1;
 }
 
@@ -1223,19 +1227,15 @@ cudaError_t launch_variant(const OnchipLaunch& L, int grid, cudaStream_t s) {
     }
     mark_used_on_device(attrs_set);
   }
-  if constexpr (CS == 1) {
-    k<<<grid, NT, smem, s>>>(L);
-    return cudaGetLastError();
-  } else {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid, 1, 1);
-    cfg.blockDim = dim3(NT, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    cluster_config<CS>(cfg, attr);
-    return cudaLaunchKernelEx(&cfg, k, L);
-  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3(NT, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  cluster_config<CS>(cfg, attr);
+  if (L.follow) follow_config(cfg, attr);
+  return cudaLaunchKernelEx(&cfg, k, L);
 }
 
 // CTAs of the variant that can be resident at once (whole clusters only).

@@ -175,6 +175,7 @@ extern "C" int ahf_unbind_batch_static(const ahf_particles* p, const ahf_halo* h
   }
 
   OnchipLaunch L;
+  L.done = nullptr; L.follow = false;
   L.p.x = p->x; L.p.y = p->y; L.p.z = p->z; L.p.vx = p->vx; L.p.vy = p->vy; L.p.vz = p->vz; L.p.m = p->m;
   L.p.m0 = p->m0; L.p.m0f = (float)p->m0; L.p.coord_type = p->coord_type; L.p.n = p->n;
   L.frame.box = prm->box;

@@ -122,6 +122,7 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
   const ParamsDev& P = L.prm;
   const bool unim = L.p.m == nullptr;                    // every particle has mass m0
 
+  chain_open();
   for (;;) {
     int hq = 0;
     if (lane == 0) hq = atomicAdd(L.queue, 1);
@@ -468,6 +469,7 @@ __global__ void __launch_bounds__(WPB * 32) warp_kernel(OnchipLaunch L) {
     }
     __syncwarp();
   }
+  if (lane == 0) chain_close(L.done, (int)gridDim.x * WPB);
 }
 
 template <int CT>
@@ -480,8 +482,14 @@ cudaError_t launch_ct(const OnchipLaunch& L, int grid, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     mark_used_on_device(attrs_set);
   }
-  k<<<grid, WPB * 32, smem, s>>>(L);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3(WPB * 32, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  if (L.follow) follow_config(cfg, attr);
+  return cudaLaunchKernelEx(&cfg, k, L);
 }
 
 }  // namespace
