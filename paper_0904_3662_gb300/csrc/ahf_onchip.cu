@@ -483,22 +483,9 @@ __device__ int cluster_dist_sort(uint32_t* kA, uint32_t* vA, uint32_t* kB, uint3
                                                            0u, tid);
 }
 
-#ifndef X1K
-#define X1K 128
-#define B1K 6
-#endif
-#ifndef X4K
-#define X4K 256
-#endif
-#ifndef X8K
-#define X8K 512
-#endif
-#ifndef XCL
-#define XCL 512
-#endif
-constexpr int NT_1K = X1K, NT_4K = X4K, NT_8K = X8K, NT_CL = XCL;
+constexpr int NT_1K = 128, NT_4K = 256, NT_8K = 512, NT_CL = 512;
 template <int CAP, int CS>
-constexpr int min_blocks() { return CS > 1 ? 1 : (CAP <= 1024 ? B1K : (CAP <= 4096 ? 2 : 1)); }
+constexpr int min_blocks() { return CS > 1 ? 1 : (CAP <= 1024 ? 6 : (CAP <= 4096 ? 2 : 1)); }
 
 template <int NT, int CAP, int CT, int CS>
 __global__ void __launch_bounds__(NT, (min_blocks<CAP, CS>())) unbind_kernel(OnchipLaunch L) {
