@@ -149,18 +149,37 @@ __device__ __forceinline__ double double_from_fix128(__int128 v, int s) {
 }
 
 __device__ __forceinline__ long long fixr(float x, int s) { return fix_from_float(x, s); }
-// round(x 2^s) for x >= 0 (the terms m and m/r): fix_from_float's value, with
-// the round half up done as one add before the shift
+// round(x 2^s) for x >= 0 (the terms m and m/r): fix_from_float's value, as one
+// 32 x 32 -> 64-bit product where the quantum is finer than x's last place by 2^30
+// at most, else with the round half up done as one add before the shift
 __device__ __forceinline__ long long fixp(float x, int s) {
   const uint32_t b = __float_as_uint(x);
   const int e = (int)(b >> 23);
-  if (e == 0) return 0;
   const int sh = e - 150 + s;
   const uint32_t mant = (b & 0x7fffffu) | 0x800000u;
+  if ((unsigned)sh <= 30u && e != 0) return (long long)((unsigned long long)mant * (unsigned long long)(1u << sh));
+  if (e == 0) return 0;
   if (sh >= 0) return (long long)((unsigned long long)mant << (sh > 39 ? 39 : sh));
   const int rs = -sh;
   return rs > 24 ? 0ll : (long long)((mant + (1u << (rs - 1))) >> rs);
 }
+// acc += fix_from_float(x, s): with the quantum finer than x's last place by 2^30
+// at most (as it is unless x is 2^20 times smaller than the halo's largest term)
+// one 32 x 32 -> 64-bit multiply-add of the signed mantissa, 10 instructions for
+// 18 (21 with the general case's branches)
+__device__ __forceinline__ void add_fix(long long& acc, float x, int s) {
+  const uint32_t b = __float_as_uint(x);
+  const int e = (int)((b >> 23) & 0xff);
+  const int sh = e - 150 + s;
+  if ((unsigned)sh <= 30u && e != 0) {
+    const int mant = (int)((b & 0x7fffffu) | 0x800000u), sg = (int)b >> 31;
+    acc += (long long)((mant ^ sg) - sg) * (long long)(int)(1u << sh);
+  } else {
+    acc += fix_from_float(x, s);
+  }
+}
+__device__ __forceinline__ void add_fix(__int128& acc, double x, int s) { acc += fix128_from_double(x, s); }
+
 __device__ __forceinline__ __int128 fixp(double x, int s) { return fix128_from_double(x, s); }
 __device__ __forceinline__ __int128 fixr(double x, int s) { return fix128_from_double(x, s); }
 __device__ __forceinline__ float from_fix(long long v, int s, float) { return float_from_fix(v, s); }
@@ -717,10 +736,63 @@ __device__ __forceinline__ void store_ranks(const GridLaunch& L, int2 tr, const 
   if (over) L.ctl->overflow = 1;
 }
 
+// Recentring in FP32.  The offset of a float coordinate x is RN(x - c'), c' the
+// centre rounded to the halo's fixed-point grid (at most 62 bits: the sum of
+// three floats).  x - hi and (x - hi) - mid split into sum and rounding error
+// (Knuth's TwoSum, exact); what is left, t, is known to 2^-22 of its terms, and
+// where both ends of that interval round the sum to the same float that is the
+// result (Ziv's test).  Elsewhere (a tie, or about one candidate in 10^5), for x
+// off the grid, and for candidates half a box away, the exact fixed-point route
+// decides.  About 25 instructions an axis for 60 of the exact route.
+struct Recentre {
+  float hi[3], mid[3], lo[3];
+  float near;                            // |x - hi| up to which no box wrap can occur
+  uint32_t x0, xn;                       // |x| bits x0 .. x0 + xn are on the grid (xn = 0: never)
+};
+// Axis a of halo H's (one thread each).
+__device__ __forceinline__ void recentre_axis(Recentre& C, const HaloDev& H, int a) {
+  const long long c = H.cfix[a];
+  const float h = f32_from_i64_rn(c);
+  const long long r = c - (long long)h;
+  const float m = f32_from_i64_rn(r);
+  const float l = f32_from_i64_rn(r - (long long)m);
+  const bool ok = !H.fast && H.frac >= -60 && H.frac <= 100;
+  const float q = ok ? __int_as_float((127 - H.frac) << 23) : 0.0f;
+  C.hi[a] = h * q;
+  C.mid[a] = m * q;
+  C.lo[a] = l * q;
+  if (a == 0) {
+    // half the box less 2^-18 of it and of the frame (the centre is within it)
+    const float half = f32_from_i64_rn(H.boxfix >> 1) * q;
+    C.near = H.boxfix > 0 ? half - 0x1p-18f * half - 0x1p-18f * (0x1p60f * q) : INFINITY;
+    C.x0 = (uint32_t)(150 - H.frac) << 23;
+    C.xn = ok ? 37u << 23 : 0u;
+  }
+}
+// One axis; false: the exact route must decide.
+__device__ __forceinline__ bool recentre(const Recentre& C, int a, float x, float& d) {
+  const float h = C.hi[a], m = C.mid[a], l = C.lo[a];
+  const float s = __fsub_rn(x, h), sb = __fsub_rn(s, x);
+  const float e = __fsub_rn(__fsub_rn(x, __fsub_rn(s, sb)), __fadd_rn(h, sb));
+  const float u = __fsub_rn(s, m), ub = __fsub_rn(u, s);
+  const float w = __fsub_rn(__fsub_rn(s, __fsub_rn(u, ub)), __fadd_rn(m, ub));
+  const float t = __fsub_rn(__fadd_rn(e, w), l);
+  const float q = __fadd_rn(__fadd_rn(fabsf(e), fabsf(w)), fabsf(l));
+  d = __fadd_rn(u, __fmaf_rn(q, 0x1p-21f, t));
+  const float d2 = __fadd_rn(u, __fmaf_rn(q, -0x1p-21f, t));
+  return d == d2 && fabsf(s) <= C.near && (__float_as_uint(x) & 0x7fffffffu) - C.x0 < C.xn;
+}
+
 // Mixed precision: the on-chip classes' float offsets (exact recentring),
 // membership and radius; the record holds w = v + H d and r, then v and m.
 // BINS: each member is counted in its radial bin and its rank of arrival kept;
 // otherwise the keys and the first digit's histogram of the radix sort.
+//
+// Bound by issue slots and latency, not by memory (a third of the DRAM rate): a
+// member took 474 instructions, in one chain a candidate.  The FP32 recentring
+// and GROUP candidates in step (their chains overlap) took 144e6 candidates from
+// 3.55 to 2.98 ms; 2 and 8 in step, 3, 5 and 6 CTAs an SM were slower.
+constexpr int GROUP = 4;
 template <int CT, bool BINS>
 __global__ void __launch_bounds__(T, 4) g_prepare_mixed(GridLaunch L) {
   const int t = blockIdx.x;
@@ -732,7 +804,9 @@ __global__ void __launch_bounds__(T, 4) g_prepare_mixed(GridLaunch L) {
   float4* rec = (float4*)L.rec;
   __shared__ uint32_t h0[CELLS + 1];
   __shared__ uint32_t scnt[BINS ? AGG_BINS : 1];
+  __shared__ Recentre C;
   const int t0 = L.halo_tile0[k], th = L.halo_tile0[k + 1] - t0;
+  if (CT != AHF_COORD_F64 && threadIdx.x < 3) recentre_axis(C, L.halos[k], threadIdx.x);
   BinMap BM;
   if (BINS) {
     BM = load_bin_map(L, k, t0, H.count, th, h0);
@@ -740,66 +814,93 @@ __global__ void __launch_bounds__(T, 4) g_prepare_mixed(GridLaunch L) {
     if (halo_bins(th) <= AGG_BINS)
       for (int c = threadIdx.x; c < halo_bins(th); c += T) scnt[c] = 0u;
   } else h0[threadIdx.x] = 0u;
-  Cand<CT> c[IPT];
-  bool ok[IPT];
-#pragma unroll
-  for (int q = 0; q < IPT; ++q) {
-    const int e = q * T + threadIdx.x;
-    ok[q] = e < tr.y;
-    if (ok[q]) {
-      const long long slot = H.offset + ((long long)tr.x + e - H.gbase);
-      long long pi = slot;
-      if (L.out.member_idx) {
-        pi = L.out.member_idx[slot];
-        if (pi < 0 || pi >= L.p.n) {
-          ok[q] = false;
-          atomicOr(L.out.err, ERR_BAD_INDEX);
-        }
-      }
-      if (ok[q]) load_cand<CT>(L.p, pi, c[q]);
-    }
-  }
   uint32_t orb = 0, andb = 0xffffffffu;
   Maxima<float> mx;
   int nmem = 0;
   uint32_t* cnt = L.bin_n + (size_t)t0 * 2 * BIN_PAD;
   const int nb = halo_bins(th);
-  __syncthreads();                       // h0 is ready
+  bool ok[IPT];
   uint32_t bin[IPT], rk[IPT];
+  // GROUP candidates at a time, each step of the way for all of them
 #pragma unroll
-  for (int q = 0; q < IPT; ++q) {
-    const int e = q * T + threadIdx.x;
-    bin[q] = 0u;
-    if (e >= tr.y) continue;
-    const long long g = (long long)tr.x + e;
-    uint32_t key = KEY_NONMEMBER;
-    if (ok[q]) {
-      float d[3];
-      long long f[3];
-      cand_offset<CT>(c[q], H, d, f);
-      ok[q] = cand_member<CT>(c[q], H, d, f);
-      if (ok[q]) {
-        const float r = radius_of(d);
-        const float m = cand_mass<CT>(L.p, c[q]);
-        float v[3];
-        cand_velocity<CT>(c[q], v);
-        rec[2 * g] = make_float4(fmaf(P.Hf, d[0], v[0]), fmaf(P.Hf, d[1], v[1]), fmaf(P.Hf, d[2], v[2]), r);
-        rec[2 * g + 1] = make_float4(v[0], v[1], v[2], m);
-        key = key_of(r);
-        if (BINS && th > 1) {
-          bin[q] = part_of(bin_key(r), BM, h0) / PARTS;
-          rk[q] = bin_rank_now(cnt, nb, bin[q]);
+  for (int q0 = 0; q0 < IPT; q0 += GROUP) {
+    Cand<CT> c[GROUP];
+#pragma unroll
+    for (int i = 0; i < GROUP; ++i) {
+      const int e = (q0 + i) * T + threadIdx.x;
+      ok[q0 + i] = e < tr.y;
+      long long pi = 0;
+      if (ok[q0 + i]) {
+        const long long slot = H.offset + ((long long)tr.x + e - H.gbase);
+        pi = slot;
+        if (L.out.member_idx) {
+          pi = L.out.member_idx[slot];
+          if (pi < 0 || pi >= L.p.n) {
+            ok[q0 + i] = false;
+            atomicOr(L.out.err, ERR_BAD_INDEX);
+          }
         }
-        mx.add(P, L.p.m != nullptr, m, r, v);
-        ++nmem;
+      }
+      if (ok[q0 + i]) load_cand<CT>(L.p, pi, c[i]);
+      else c[i] = Cand<CT>{};
+    }
+    if (q0 == 0) __syncthreads();        // the map, the counters and C are ready
+    float d[GROUP][3], r[GROUP];
+    bool sure[GROUP];
+#pragma unroll
+    for (int i = 0; i < GROUP; ++i) {
+      sure[i] = false;
+      d[i][0] = d[i][1] = d[i][2] = 0.0f;
+      if (CT != AHF_COORD_F64 && !H.fast)
+        sure[i] = recentre(C, 0, (float)c[i].x, d[i][0]) & recentre(C, 1, (float)c[i].y, d[i][1]) &
+                  recentre(C, 2, (float)c[i].z, d[i][2]);
+    }
+#pragma unroll
+    for (int i = 0; i < GROUP; ++i) {
+      const float r2 = fmaf(d[i][2], d[i][2], fmaf(d[i][1], d[i][1], d[i][0] * d[i][0]));
+      const bool in = r2 < H.R2lo;
+      if (ok[q0 + i] && !(sure[i] && (in || r2 > H.R2hi))) {
+        long long f[3];
+        cand_offset<CT>(c[i], H, d[i], f);
+        ok[q0 + i] = cand_member<CT>(c[i], H, d[i], f);
+      } else {
+        ok[q0 + i] = ok[q0 + i] && in;
       }
     }
-    if (L.out.removed_iter) L.out.removed_iter[H.offset + (g - H.gbase)] = key == KEY_NONMEMBER ? -1 : 0;
-    if (!BINS) {
-      key_a[g] = key;
-      atomicAdd(&h0[key & 0xffu], 1u);
-      orb |= key;
-      andb &= key;
+#pragma unroll
+    for (int i = 0; i < GROUP; ++i) r[i] = radius_of(d[i]);
+    if (BINS && th > 1) {
+#pragma unroll
+      for (int i = 0; i < GROUP; ++i) bin[q0 + i] = part_of(ok[q0 + i] ? bin_key(r[i]) : 0u, BM, h0) / PARTS;
+#pragma unroll
+      for (int i = 0; i < GROUP; ++i)
+        if (ok[q0 + i]) rk[q0 + i] = bin_rank_now(cnt, nb, bin[q0 + i]);
+    }
+#pragma unroll
+    for (int i = 0; i < GROUP; ++i) {
+      const int q = q0 + i;
+      const int e = q * T + threadIdx.x;
+      if (!BINS || th == 1) bin[q] = 0u;
+      if (e >= tr.y) continue;
+      const long long g = (long long)tr.x + e;
+      uint32_t key = KEY_NONMEMBER;
+      if (ok[q]) {
+        const float m = cand_mass<CT>(L.p, c[i]);
+        float v[3];
+        cand_velocity<CT>(c[i], v);
+        rec[2 * g] = make_float4(fmaf(P.Hf, d[i][0], v[0]), fmaf(P.Hf, d[i][1], v[1]), fmaf(P.Hf, d[i][2], v[2]), r[i]);
+        rec[2 * g + 1] = make_float4(v[0], v[1], v[2], m);
+        key = key_of(r[i]);
+        mx.add(P, L.p.m != nullptr, m, r[i], v);
+        ++nmem;
+      }
+      if (L.out.removed_iter) L.out.removed_iter[H.offset + (g - H.gbase)] = key == KEY_NONMEMBER ? -1 : 0;
+      if (!BINS) {
+        key_a[g] = key;
+        atomicAdd(&h0[key & 0xffu], 1u);
+        orb |= key;
+        andb &= key;
+      }
     }
   }
   if (BINS) {
@@ -1887,7 +1988,7 @@ __global__ void __launch_bounds__(HT) g_halo(GridLaunch L, int pass) {
 // radial order, the streams (w, r), (v, m), the position (and mass, thermal
 // energy), the exact sum m v, and the sub-tiles' sums of the initial set.
 template <typename R>
-__global__ void __launch_bounds__(T, 3) g_bin_sort(GridLaunch L) {
+__global__ void __launch_bounds__(T, sizeof(R) == 4 ? 4 : 3) g_bin_sort(GridLaunch L) {
   using V4 = typename Prec<R>::V4;
   using Key = typename Prec<R>::Key;
   using Acc = typename Prec<R>::Acc;
@@ -1992,10 +2093,15 @@ __global__ void __launch_bounds__(T, 3) g_bin_sort(GridLaunch L) {
   // rows aligned to 32 positions of the halo, so that none straddles two sub-tiles
   const int lead = (int)(at & 31u);
   const int rows = (n + lead + 31) >> 5;
-  for (int row = warp; row < rows; row += NWARP) {
+  // each warp a run of rows: its lanes keep the sums of a sub-tile (8 rows) and
+  // reduce them where it ends (144e6 members: 3.27 -> 3.17 ms with add_fix)
+  const int share = (rows + NWARP - 1) / NWARP;
+  const int row1 = min(rows, (warp + 1) * share);
+  Acc a = 0, b = 0;
+  int c = 0;
+  for (int row = warp * share; row < row1; ++row) {
     const int e = row * 32 - lead + lane;
     const bool in = e >= 0 && e < n;
-    Acc a = 0, b = 0;
     if (in) {
       const int i = sout[e];
       const V4 x = rb[2 * i];
@@ -2014,21 +2120,24 @@ __global__ void __launch_bounds__(T, 3) g_bin_sort(GridLaunch L) {
         ((R*)L.uth)[dst] = (R)(L.p.coord_type == AHF_COORD_F64 ? __ldg((const double*)L.p.u_th + pi)
                                                                : (double)__ldg((const float*)L.p.u_th + pi));
       }
-      a = L.ms ? (Acc)fixp(m, s_m) : mfix0;
-      b = fixp(m * rinv_real(x.w, L.prm), s_r);
-      smv[0] += fixr(mul_rn(m, y.x), s_v);
-      smv[1] += fixr(mul_rn(m, y.y), s_v);
-      smv[2] += fixr(mul_rn(m, y.z), s_v);
+      if (L.ms) add_fix(a, m, s_m);
+      add_fix(b, m * rinv_real(x.w, L.prm), s_r);
+      add_fix(smv[0], mul_rn(m, y.x), s_v);
+      add_fix(smv[1], mul_rn(m, y.y), s_v);
+      add_fix(smv[2], mul_rn(m, y.z), s_v);
     }
-    const int c = __popc(__ballot_sync(FULL_MASK, in));
-    if (L.ms) a = wsum(a);
-    else a = mfix0 * (Acc)c;
-    b = wsum(b);
-    if (lane == 0 && c) {
-      const size_t u = sub0 + ((at + (uint32_t)max(row * 32 - lead, 0)) / SUB);
-      atomic_add_acc((Acc*)L.agg_m + u, a);
-      atomic_add_acc((Acc*)L.agg_r + u, b);
-      atomicAdd(&L.agg_c[u], c);
+    c += __popc(__ballot_sync(FULL_MASK, in));
+    const uint32_t u = (at - (uint32_t)lead + (uint32_t)row * 32u) / SUB;
+    if (row + 1 == row1 || (at - (uint32_t)lead + (uint32_t)row * 32u + 32u) / SUB != u) {
+      const Acc am = L.ms ? wsum(a) : mfix0 * (Acc)c, br = wsum(b);
+      if (lane == 0 && c) {
+        atomic_add_acc((Acc*)L.agg_m + sub0 + u, am);
+        atomic_add_acc((Acc*)L.agg_r + sub0 + u, br);
+        atomicAdd(&L.agg_c[sub0 + u], c);
+      }
+      a = 0;
+      b = 0;
+      c = 0;
     }
   }
 #pragma unroll
@@ -2292,9 +2401,9 @@ __global__ void __launch_bounds__(T) g_removed(GridLaunch L, int pass) {
         else atomicOr((unsigned long long*)&wr[g].w, 0x8000000000000000ull);
         if (L.out.removed_iter) L.out.removed_iter[H.offset + pos[e]] = pass;
         const R m = UNIF ? m0 : ((const R*)L.ms)[g];
-        mv0 += fixr(mul_rn(m, vm[e].x), s_v);
-        mv1 += fixr(mul_rn(m, vm[e].y), s_v);
-        mv2 += fixr(mul_rn(m, vm[e].z), s_v);
+        add_fix(mv0, mul_rn(m, vm[e].x), s_v);
+        add_fix(mv1, mul_rn(m, vm[e].y), s_v);
+        add_fix(mv2, mul_rn(m, vm[e].z), s_v);
       }
     }
     mv0 = wsum(mv0);
