@@ -120,9 +120,25 @@ __device__ __forceinline__ __int128 fix128_from_double(double x, int s) {
   return (b >> 63) ? -v : v;
 }
 
-// v 2^-s as the nearest double (ties to even).
+// v 2^-s as the nearest double (ties to even): the top 64 bits with every bit below
+// ORed into the last, rounded to 53 by an add whose carry runs into the exponent.
+// Integer instructions only: the FP64 pipe (two lanes a clock and SM) bounds the
+// all-FP64 kernels.
 __device__ __forceinline__ double double_from_fix128(__int128 v, int s) {
-  if (v == 0) return 0.0;
+  const unsigned long long vh = (unsigned long long)((unsigned __int128)v >> 64), vl = (unsigned long long)v;
+  if (v >= 0) {
+    if (v == 0) return 0.0;
+    const int z = vh ? __clzll((long long)vh) : 64 + __clzll((long long)vl);
+    const int ex = 127 - z + 1022 - s;                  // the exponent field less one
+    if (ex >= 0 && ex < 2045) {
+      const unsigned __int128 n = (unsigned __int128)v << z;
+      unsigned long long t = (unsigned long long)(n >> 64);
+      if ((unsigned long long)n) t |= 1ull;
+      const unsigned long long m = t >> 11;
+      const unsigned up = ((unsigned)t & 0x7ffu) + ((unsigned)m & 1u) > 0x400u ? 1u : 0u;
+      return __longlong_as_double((long long)(((unsigned long long)ex << 52) + m + up));
+    }
+  }
   const bool negv = v < 0;
   const unsigned __int128 a = negv ? (unsigned __int128)0 - (unsigned __int128)v : (unsigned __int128)v;
   const unsigned long long hi = (unsigned long long)(a >> 64), lo = (unsigned long long)a;
@@ -279,13 +295,25 @@ __device__ __forceinline__ unsigned long long abs_bits(double x) {
   return (unsigned long long)__double_as_longlong(fabs(x));
 }
 __device__ __forceinline__ float rinv_real(float r, const ParamsDev& P) { return rinv_of(r, P.r_soft_f); }
+// Comparisons of doubles on the integer pipe (same truth values, NaN included).
+constexpr unsigned long long INF_BITS = 0x7ff0000000000000ull;
+// a <= b, b >= 0 and a >= 0 or NaN
+__device__ __forceinline__ bool le_positive(double a, double b) {
+  const unsigned long long x = (unsigned long long)__double_as_longlong(a), y = (unsigned long long)__double_as_longlong(b);
+  return x <= y && y <= INF_BITS;
+}
+__device__ __forceinline__ bool positive(double a) {
+  return (unsigned long long)__double_as_longlong(a) - 1ull < INF_BITS;
+}
 __device__ __forceinline__ double rinv_real(double r, const ParamsDev& P) {
-  const double rr = fmax(r, P.r_soft);
-  return rr > 0.0 ? 1.0 / rr : 0.0;
+  // fmax(r, r_soft) for r_soft >= 0 (r: not NaN), on the integer pipe
+  const long long a = __double_as_longlong(r), b = __double_as_longlong(P.r_soft);
+  const double rr = __longlong_as_double(a > b ? a : b);
+  return positive(rr) ? 1.0 / rr : 0.0;
 }
 // rinv_real(r, P) > 0, without the division
 __device__ __forceinline__ bool rinv_positive(float r, const ParamsDev& P) { return fmaxf(r, P.r_soft_f) > 0.0f; }
-__device__ __forceinline__ bool rinv_positive(double r, const ParamsDev& P) { return fmax(r, P.r_soft) > 0.0; }
+__device__ __forceinline__ bool rinv_positive(double r, const ParamsDev& P) { return positive(r) || positive(P.r_soft); }
 __device__ __forceinline__ unsigned long long bits_of(float x) { return __float_as_uint(x); }
 __device__ __forceinline__ unsigned long long bits_of(double x) { return (unsigned long long)__double_as_longlong(x); }
 __device__ __forceinline__ float real_of_bits(unsigned long long b, float) { return __uint_as_float((uint32_t)b); }
@@ -322,8 +350,11 @@ __device__ __forceinline__ void offset_f64(const ParticlesDev& p, long long i, c
     double v = __dsub_rn(x[a], H.c[a]);
     if (box > 0.0) {
       const double half = 0.5 * box;
-      if (v > half) v = __dsub_rn(v, box);
-      if (v < -half) v = __dadd_rn(v, box);
+      // (|v| > half, or NaN, on the integer pipe; rarely taken)
+      if (((unsigned long long)__double_as_longlong(v) & ~(1ull << 63)) > (unsigned long long)__double_as_longlong(half)) {
+        if (v > half) v = __dsub_rn(v, box);
+        if (v < -half) v = __dadd_rn(v, box);
+      }
     }
     d[a] = v;
   }
@@ -496,10 +527,13 @@ __host__ __device__ __forceinline__ int halo_bins(int th) { return th > 1 ? 2 * 
 
 __device__ __forceinline__ bool bins_overflowed(const GridLaunch& L) { return __ldcg(&L.ctl->overflow) != 0; }
 
-// The key a bin is found from: the bits of r as a float (rounding a double
-// radius is monotone).
+// The key a bin is found from: the bits of r as a float (cutting a double
+// radius is monotone, and needs no conversion on the FP64 pipe).
 __device__ __forceinline__ uint32_t bin_key(float r) { return __float_as_uint(r); }
-__device__ __forceinline__ uint32_t bin_key(double r) { return __float_as_uint(__double2float_rn(r)); }
+__device__ __forceinline__ uint32_t bin_key(double r) {
+  const unsigned long long x = (unsigned long long)__double_as_longlong(r) >> 29, base = 896ull << 23;
+  return x > base ? (uint32_t)min(x - base, 0x7f7fffffull) : 0u;
+}
 
 // Candidates sampled of n: an eighth, 512 to SAMPLE_MAX of them.
 __device__ __forceinline__ int sample_size(long long n) {
@@ -597,7 +631,7 @@ __global__ void __launch_bounds__(T) g_sample(GridLaunch L) {
         double d[3];
         offset_f64<CT>(L.p, pi, H, L.frame.box, d);
         const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])), __dmul_rn(d[2], d[2]));
-        if (r2 <= H.R2) key = bin_key(sqrt(r2));
+        if (le_positive(r2, H.R2)) key = bin_key(sqrt(r2));
       }
     }
     ((uint32_t*)L.rec_b)[H.gbase + j] = key;
@@ -973,7 +1007,7 @@ __global__ void __launch_bounds__(T) g_prepare_f64(GridLaunch L) {
       double d[3];
       offset_f64<CT>(L.p, pi, H, L.frame.box, d);
       const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])), __dmul_rn(d[2], d[2]));
-      if (r2 <= H.R2) {
+      if (le_positive(r2, H.R2)) {
         const double r = sqrt(r2);
         const double m = load_mass_f64<CT>(L.p, pi);
         double v[3];
@@ -2109,7 +2143,8 @@ __global__ void __launch_bounds__(T, sizeof(R) == 4 ? 4 : 3) g_bin_sort(GridLaun
       const uint32_t p = binned_pos(y.w);
       const long long dst = g0 + e;
       const R m = L.ms ? ((const R*)L.ms_b)[g0 + i] : m0;
-      y.w = m;
+      const R ri = rinv_real(x.w, L.prm);
+      y.w = ri;                          // (the mass is in ms, or uniform)
       ((V4*)L.wr)[dst] = x;
       vr[dst] = y;
       L.val_x[dst] = p;
@@ -2121,7 +2156,7 @@ __global__ void __launch_bounds__(T, sizeof(R) == 4 ? 4 : 3) g_bin_sort(GridLaun
                                                                : (double)__ldg((const float*)L.p.u_th + pi));
       }
       if (L.ms) add_fix(a, m, s_m);
-      add_fix(b, m * rinv_real(x.w, L.prm), s_r);
+      add_fix(b, m * ri, s_r);
       add_fix(smv[0], mul_rn(m, y.x), s_v);
       add_fix(smv[1], mul_rn(m, y.y), s_v);
       add_fix(smv[2], mul_rn(m, y.z), s_v);
@@ -2177,27 +2212,93 @@ __device__ __forceinline__ void sub_prefix(const GridLaunch& L, int u, int t, in
 template <typename R>
 __device__ __forceinline__ void write_skip(const GridLaunch& L, int u, const GridHaloState& S, R mg, R uu, R r0,
                                            const R vb[3]) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    mg = fmin(mg, __shfl_xor_sync(FULL_MASK, mg, o));
-    uu = fmax(uu, __shfl_xor_sync(FULL_MASK, uu, o));
+  // floats in order as integers (no NaN among them, |u|^2 not negative)
+  int m, w;
+  if (sizeof(R) == 4) {
+    m = __float_as_int((float)mg);
+    w = __float_as_int((float)uu);
+  } else {
+    m = __float_as_int(__double2float_rd((double)mg));
+    w = __float_as_int(__double2float_ru((double)uu));
   }
+  m = __reduce_min_sync(FULL_MASK, m ^ ((m >> 31) & 0x7fffffff));
+  w = __reduce_max_sync(FULL_MASK, w);
   if ((threadIdx.x & 31) != 0) return;
   SkipRec rc;
-  if (sizeof(R) == 4) {
-    rc.margin = (float)mg;
-    rc.umax = __fsqrt_ru((float)uu);
-    rc.rin = fabsf((float)r0);
-  } else {
-    rc.margin = __double2float_rd((double)mg);
-    rc.umax = __double2float_ru(sqrt((double)uu));
-    rc.rin = __double2float_rd(fabs((double)r0));
-  }
+  rc.margin = __int_as_float(m ^ ((m >> 31) & 0x7fffffff));
+  rc.umax = __fsqrt_ru(__int_as_float(w));
+  rc.rin = sizeof(R) == 4 ? fabsf((float)r0) : __double2float_rd(fabs((double)r0));
 #pragma unroll
   for (int a = 0; a < 3; ++a) rc.vb[a] = (float)vb[a];
   rc.mrem = S.mrem;
   L.skip[u] = rc;
 }
+
+// 2 |phi|: -2 phi_real, the doubling (exact) in the factor.
+__device__ __forceinline__ float two_phi_real(float M, float ri, float S, const ParamsDev& P) {
+  return -2.0f * phi_real(M, ri, S, P);
+}
+__device__ __forceinline__ double two_phi_real(double M, double ri, double S, const ParamsDev& P) {
+  return __dmul_rn(2.0 * P.G, __fma_rn(M, ri, S));
+}
+
+// The escape and band tests of a member and the skip record's extremes (the
+// smallest margin and the largest |u|^2 of the members kept; NaN left out).
+template <typename R>
+struct BandTest {
+  R band, mg = (R)INFINITY, uu = (R)0;
+  __device__ __forceinline__ explicit BandTest(R b) : band(b) {}
+  __device__ __forceinline__ bool in_band(R u2, R two_phi) const { return fabs(u2 - two_phi) < band * two_phi; }
+  __device__ __forceinline__ bool escapes(R u2, R two_phi) const { return u2 > two_phi; }
+  __device__ __forceinline__ void keep(R margin, R uk) {
+    mg = fmin(mg, margin);
+    uu = fmax(uu, uk);
+  }
+  __device__ __forceinline__ void extremes(R& m, R& u) const {
+    m = mg;
+    u = uu;
+  }
+};
+// In FP64 on the integer pipe: the bit patterns of positive doubles compare as
+// they do, two within band (< 1/4) of each other differ by less than band 2^54
+// in them, and the extremes are kept as upper words (rounded down and up at
+// the end: the skip test is one-sided).  A member takes 10 FP64 instructions (44
+// with the division, the comparisons and the conversions).
+template <>
+struct BandTest<double> {
+  double band;
+  unsigned long long near;               // differences of the bits that may be in the band
+  int mg = 0x7ff00000, uu = -1;
+  __device__ __forceinline__ explicit BandTest(double b) : band(b) {
+    near = b >= 0.0 && b < 0.25 ? (unsigned long long)(b * 0x1p54) + 2ull : ~0ull;
+  }
+  static __device__ __forceinline__ bool plain(unsigned long long a, unsigned long long b) {
+    return a <= INF_BITS && b <= INF_BITS;
+  }
+  __device__ __forceinline__ bool in_band(double u2, double two_phi) const {
+    const unsigned long long a = (unsigned long long)__double_as_longlong(u2);
+    const unsigned long long b = (unsigned long long)__double_as_longlong(two_phi);
+    if (plain(a, b) && (a > b ? a - b : b - a) > near) return false;
+    return fabs(u2 - two_phi) < band * two_phi;
+  }
+  __device__ __forceinline__ bool escapes(double u2, double two_phi) const {
+    const unsigned long long a = (unsigned long long)__double_as_longlong(u2);
+    const unsigned long long b = (unsigned long long)__double_as_longlong(two_phi);
+    return plain(a, b) ? a > b : u2 > two_phi;
+  }
+  __device__ __forceinline__ void keep(double margin, double uk) {
+    const int h = __double2hiint(margin), w = __double2hiint(uk);
+    mg = min(mg, (h & 0x7fffffff) > 0x7ff00000 ? 0x7ff00000 : h ^ ((h >> 31) & 0x7fffffff));
+    uu = max(uu, w > 0x7ff00000 ? -1 : w);
+  }
+  __device__ __forceinline__ void extremes(double& m, double& u) const {
+    // (upper words in order, the lower ones dropped: one down for negative
+    // margins, one up for |u|^2)
+    const int o = mg < 0 ? mg - 1 : mg;
+    m = __hiloint2double(o ^ ((o >> 31) & 0x7fffffff), 0);
+    u = uu < 0 ? 0.0 : __hiloint2double(min(uu + 1, 0x7ff00000), 0);
+  }
+};
 
 // Phi and the escape test over sub-tile w.x (halo w.y) in pass `pass`, by
 // one warp: lane l holds elements [8 l, 8 l + 8) of the sub-tile; one warp
@@ -2223,12 +2324,17 @@ __device__ __forceinline__ void pass_sub(const GridLaunch& L, const int4 w, int 
   const R m0 = sizeof(R) == 4 ? (R)L.p.m0f : (R)L.p.m0;
   // the lane's elements, all in flight at once
   V4 q[EPL];
-  R mq[EPL], uq[EPL];
+  R mq[EPL], uq[EPL], ri[EPL];
+  // FP64: 1/r as the bins' sort left it beside v (a division is a third of the
+  // FP64 instructions of a member)
+  const bool has_ri = sizeof(R) == 8 && L.vr != nullptr;
 #pragma unroll
   for (int i = 0; i < EPL; ++i) {
     const long long g = gl + i;
+    ri[i] = (R)0;
     if (i < nl) {
       q[i] = wr[g];
+      if (has_ri) ri[i] = ((const V4*)L.vr)[g].w;
       mq[i] = UNIF ? m0 : ((const R*)L.ms)[g];
       uq[i] = GAS ? ((const R*)L.uth)[g] : (R)0;
     } else {
@@ -2248,13 +2354,12 @@ __device__ __forceinline__ void pass_sub(const GridLaunch& L, const int4 w, int 
   const float sc_m = FAST ? pow2_neg(s_m) : 0.0f, sc_r = FAST ? pow2_neg(s_r) : 0.0f;
   const Acc mfix0 = fixp(m0, s_m);
   // per element: 1/r and the exact terms; the lane's sums
-  R ri[EPL];
   Acc rf[EPL];
   Acc a = 0, b = 0;
 #pragma unroll
   for (int i = 0; i < EPL; ++i) {
     const bool alive = !signbit(q[i].w);
-    ri[i] = rinv_real(q[i].w, P);
+    if (!has_ri) ri[i] = rinv_real(q[i].w, P);
     rf[i] = alive ? fixp(mq[i] * ri[i], s_r) : (Acc)0;
     if (alive) a += UNIF ? mfix0 : fixp(mq[i], s_m);
     b += rf[i];
@@ -2272,6 +2377,7 @@ __device__ __forceinline__ void pass_sub(const GridLaunch& L, const int4 w, int 
   Acc rm = 0, rr = 0;
   const R keep_frac = (R)1 - band - (R)0x1p-16;
   R mg = (R)INFINITY, uu = (R)0;
+  BandTest<R> test(band);
 #pragma unroll
   for (int i = 0; i < EPL; ++i) {
     const R r = q[i].w;
@@ -2280,25 +2386,24 @@ __device__ __forceinline__ void pass_sub(const GridLaunch& L, const int4 w, int 
       const R Mf = (FAST && sizeof(R) == 4) ? (R)fix_to_float_sc((long long)M, sc_m) : from_fix(M, s_m, R());
       const R Sf = (FAST && sizeof(R) == 4) ? (R)fix_to_float_sc((long long)(Ttot - Pp), sc_r)
                                             : from_fix(Ttot - Pp, s_r, R());
-      const R phi = phi_real(Mf, ri[i], Sf, P);
+      const R two_phi = two_phi_real(Mf, ri[i], Sf, P);
       const R ux = q[i].x - vb[0], uy = q[i].y - vb[1], uz = q[i].z - vb[2];
       const R uk = fma_x(uz, uz, fma_x(uy, uy, ux * ux));
       R u2 = uk;
       if (GAS) u2 += (R)2 * uq[i];                 // gas: |u|^2 + 2 u_th (Sect. 2.1)
-      const R two_phi = (R)-2 * phi;
-      if (fabs(u2 - two_phi) < band * two_phi) ++nband;
-      if (u2 > two_phi) {
+      if (test.in_band(u2, two_phi)) ++nband;
+      if (test.escapes(u2, two_phi)) {
         rem |= 1u << i;
         rm += mfix;
         rr += rf[i];
       } else {
-        mg = fmin(mg, two_phi * keep_frac - u2);
-        uu = fmax(uu, uk);
+        test.keep(fma_x(two_phi, keep_frac, -u2), uk);
       }
       M += mfix;
       Pp += rf[i];
     }
   }
+  test.extremes(mg, uu);
   write_skip<R>(L, u, S, mg, uu, q[0].w, vb);
   // the sub-tile's sums after the removals (next copy) and its removal flags
   const int nrem = __reduce_add_sync(FULL_MASK, __popc(rem));
@@ -2618,14 +2723,16 @@ __global__ void __launch_bounds__(T, sizeof(R) == 4 ? 4 : 2) g_final(GridLaunch 
   const int e0 = (u % SPT) * SUB;
   // rows of 32 consecutive elements (coalesced), read before the halo's
   // state arrives; elements past the last member count as removed
-  R rq[ROWS], mq[ROWS];
+  R rq[ROWS], mq[ROWS], ri_q[ROWS];
   uint32_t vq[ROWS];
+  const bool has_ri = sizeof(R) == 8 && L.vr != nullptr;   // as in a pass
 #pragma unroll
   for (int i = 0; i < ROWS; ++i) {
     const int e = e0 + 32 * i + lane;
     const long long g = (long long)tr.x + e;
     rq[i] = e < tr.y ? wr[g].w : neg0(R());
     mq[i] = (!UNIF && e < tr.y) ? ((const R*)L.ms)[g] : m0;
+    ri_q[i] = has_ri && e < tr.y ? ((const V4*)L.vr)[g].w : (R)0;
     vq[i] = e < tr.y ? L.val_x[g] : 0u;
   }
   const int k = L.tile_halo[t];
@@ -2644,7 +2751,7 @@ __global__ void __launch_bounds__(T, sizeof(R) == 4 ? 4 : 2) g_final(GridLaunch 
   for (int i = 0; i < ROWS; ++i) {
     const R r = rq[i];
     const bool alive = !signbit(r) && (long long)tr.x + e0 + 32 * i + lane < lim;
-    const R ri = rinv_real(r, P);
+    const R ri = has_ri ? ri_q[i] : rinv_real(r, P);
     const Acc a = alive ? (Acc)fixp(mq[i], s_m) : (Acc)0;
     const Acc b = alive ? (Acc)fixp(mq[i] * ri, s_r) : (Acc)0;
     const unsigned bal = __ballot_sync(FULL_MASK, alive);
