@@ -595,7 +595,6 @@ void grid_take(Bump& B, GridLaunch* G, const GridSizes& z) {
   char* prr = B.take<char>((size_t)z.n_tiles * as);
   long long* prc = B.take<long long>((size_t)z.n_tiles);
   int4* work = B.take<int4>(2 * n_sub);
-  uint8_t* rmask = B.take<uint8_t>(32 * n_sub);
   AccSlot* tmv = B.take<AccSlot>(3 * (size_t)z.n_tiles);
   SkipRec* skip = B.take<SkipRec>(n_sub);
   if (!G) return;
@@ -605,7 +604,6 @@ void grid_take(Bump& B, GridLaunch* G, const GridSizes& z) {
   G->n_big = z.n_big; G->tile_hist = hist; G->digit_base = dbase;
   G->agg_m = agm; G->agg_r = agr; G->agg_c = agc; G->pre_m = prm_; G->pre_r = prr; G->pre_c = prc;
   G->work = work;
-  G->rem_mask = rmask;
   G->wr_radix = wr;
   // the block has 2 es + 8 + v4 + as bytes per candidate: 40 (72 in FP64),
   // the records 2 v4 and the masses es of them: 36 (72)
@@ -665,7 +663,7 @@ int run_grid(ahf_ctx* c, GridLaunch& G, const ahf_params* prm, cudaStream_t s, i
     const int n = std::min(chunk, prm->max_iter - pass + 1);
     for (int i = 0; i < n; ++i) {
       AHF_CUDA(grid_iterate(G, pass++, s));
-      c->stats.launches += 3;
+      c->stats.launches += 2;
       c->stats.grid_iterations += 1;
     }
     // work_n and the bins' overflow word

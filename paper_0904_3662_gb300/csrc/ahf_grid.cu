@@ -2234,6 +2234,47 @@ __device__ __forceinline__ void write_skip(const GridLaunch& L, int u, const Gri
   L.skip[u] = rc;
 }
 
+// The particles a pass removed from sub-tile w.x (flags `rem` of the lane's
+// elements, nrem > 0 in the warp): the sign bit of r, their removal iteration, and
+// the exact sum m v of what the halo lost.  They are listed in shared memory first
+// (256 bytes a warp) and taken one per lane: a few of a sub-tile's 256 are removed,
+// mostly by a few lanes.
+template <typename R, bool UNIF>
+__device__ __forceinline__ void removed(const GridLaunch& L, const int4 w, int pass, unsigned rem, int nrem, uint8_t* list) {
+  using V4 = typename Prec<R>::V4;
+  using Acc = typename Prec<R>::Acc;
+  const int lane = threadIdx.x & 31;
+  GridHaloState& S = L.state[w.y];
+  const HaloDev& H = L.halos[w.y];
+  V4* wr = (V4*)L.wr;
+  const uint32_t n = (uint32_t)__popc(rem);
+  uint32_t at = wscan(n, lane) - n;
+  for (; rem; rem &= rem - 1) list[at++] = (uint8_t)(lane * EPL + __ffs(rem) - 1);
+  __syncwarp();
+  const R m0 = sizeof(R) == 4 ? (R)L.p.m0f : (R)L.p.m0;
+  const int s_v = S.s_mv;
+  Acc mv[3] = {0, 0, 0};
+  for (int j = lane; j < nrem; j += 32) {
+    const long long g = (long long)w.z + list[j];
+    const uint32_t pos = L.val_x[g];
+    const R m = UNIF ? m0 : ((const R*)L.ms)[g];
+    // radial order, or (radix sort) the candidate's record
+    const V4 v = L.vr ? ((const V4*)L.vr)[g] : ((const V4*)L.rec)[2 * (H.gbase + pos) + 1];
+    if (sizeof(R) == 4) atomicOr((unsigned*)&wr[g].w, 0x80000000u);
+    else atomicOr((unsigned long long*)&wr[g].w, 0x8000000000000000ull);
+    if (L.out.removed_iter) L.out.removed_iter[H.offset + pos] = pass;
+    add_fix(mv[0], mul_rn(m, v.x), s_v);
+    add_fix(mv[1], mul_rn(m, v.y), s_v);
+    add_fix(mv[2], mul_rn(m, v.z), s_v);
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    mv[a] = wsum(mv[a]);
+    if (lane == 0) atomic_acc(S.rem_mv[a], mv[a]);
+  }
+  __syncwarp();                          // the list is reused
+}
+
 // 2 |phi|: -2 phi_real, the doubling (exact) in the factor.
 __device__ __forceinline__ float two_phi_real(float M, float ri, float S, const ParamsDev& P) {
   return -2.0f * phi_real(M, ri, S, P);
@@ -2302,13 +2343,13 @@ struct BandTest<double> {
 
 // Phi and the escape test over sub-tile w.x (halo w.y) in pass `pass`, by
 // one warp: lane l holds elements [8 l, 8 l + 8) of the sub-tile; one warp
-// scan of the lanes' sums places every element's prefix.  The pass only
-// decides: it leaves the sub-tile's sums after the removals for the next
-// pass and one byte of removal flags per lane; g_removed does the rest.
+// scan of the lanes' sums places every element's prefix.  It leaves the
+// sub-tile's sums after the removals for the next pass and marks the removed
+// (a kernel of its own for that cost 6 to 60 us a pass).
 // FAST: the scales 2^-s of the halo are normal floats (the conversions of
 // the exact sums to float are then a multiply; same bits).
 template <typename R, bool UNIF, bool GAS, bool FAST>
-__device__ __forceinline__ void pass_sub(const GridLaunch& L, const int4 w, int pass) {
+__device__ __forceinline__ void pass_sub(const GridLaunch& L, const int4 w, int pass, uint8_t* list) {
   using V4 = typename Prec<R>::V4;
   using Acc = typename Prec<R>::Acc;
   const int u = w.x, k = w.y, t = u / SPT;
@@ -2408,10 +2449,10 @@ __device__ __forceinline__ void pass_sub(const GridLaunch& L, const int4 w, int 
   // the sub-tile's sums after the removals (next copy) and its removal flags
   const int nrem = __reduce_add_sync(FULL_MASK, __popc(rem));
   nband = __reduce_add_sync(FULL_MASK, nband);
-  L.rem_mask[(size_t)u * 32 + lane] = (uint8_t)rem;
   if (nrem) {                                      // uniform over the warp
     rm = wsum(rm);
     rr = wsum(rr);
+    removed<R, UNIF>(L, w, pass, rem, nrem, list);
   }
   if (lane == 0) {
     const size_t j = (size_t)(cp ^ 1) * n_sub + u;
@@ -2426,6 +2467,7 @@ __device__ __forceinline__ void pass_sub(const GridLaunch& L, const int4 w, int 
 // round robin, and clear the count of the next pass's list.
 template <typename R, bool UNIF, bool GAS>
 __global__ void __launch_bounds__(T, sizeof(R) == 4 ? 2 : 1) g_pass(GridLaunch L, int pass) {
+  __shared__ uint8_t removed_list[NWARP][SUB];
   if (blockIdx.x == 0 && threadIdx.x == 0) L.ctl->work_n[(pass + 1) & 1] = 0;
   if (gave_up(L)) return;
   const int n = __ldcg(&L.ctl->work_n[pass & 1]);
@@ -2434,92 +2476,9 @@ __global__ void __launch_bounds__(T, sizeof(R) == 4 ? 2 : 1) g_pass(GridLaunch L
     const int4 w = list[i];
     const GridHaloState& S = L.state[w.y];
     if (sizeof(R) == 4 && pow2_neg(S.s_m) != 0.0f && pow2_neg(S.s_mr) != 0.0f)
-      pass_sub<R, UNIF, GAS, true>(L, w, pass);
+      pass_sub<R, UNIF, GAS, true>(L, w, pass, removed_list[threadIdx.x >> 5]);
     else
-      pass_sub<R, UNIF, GAS, false>(L, w, pass);
-  }
-}
-
-// After a pass, the particles it removed (the flags of the listed sub-tiles):
-// the sign bit of r, their removal iteration, and the exact sum m v of what
-// each halo lost (v from the candidate's record), one warp per sub-tile.
-template <typename R, bool UNIF>
-__global__ void __launch_bounds__(T) g_removed(GridLaunch L, int pass) {
-  if (gave_up(L)) return;
-  using V4 = typename Prec<R>::V4;
-  using Acc = typename Prec<R>::Acc;
-  const int lane = threadIdx.x & 31;
-  const int n = __ldcg(&L.ctl->work_n[pass & 1]);
-  const int4* list = L.work + (size_t)(pass & 1) * L.n_tiles * SPT;
-  V4* wr = (V4*)L.wr;
-  const V4* rec = (const V4*)L.rec;
-  const V4* vr = (const V4*)L.vr;        // radial order, or NULL (radix sort): by candidate
-  const R m0 = sizeof(R) == 4 ? (R)L.p.m0f : (R)L.p.m0;
-  // `share` listed sub-tiles per step (32, fewer when the list would leave
-  // warps without any: 43 sub-tiles of one halo were two warps' work, 27 us in
-  // FP64): lane j checks entry i0 + j's flags (32 bytes), then the warp takes the
-  // flagged ones one after another
-  const int nwarps = (gridDim.x * T) >> 5;
-  const int share = min(32, (n + nwarps - 1) / nwarps);
-  for (int i0 = ((blockIdx.x * T + threadIdx.x) >> 5) * share; i0 < n; i0 += nwarps * share) {
-    const int ij = i0 + lane;
-    int4 wj = make_int4(0, 0, 0, 0);
-    bool any = false;
-    if (ij < n && lane < share) {
-      wj = list[ij];
-      const uint4* mk = (const uint4*)(L.rem_mask + (size_t)wj.x * 32);
-      const uint4 m0 = mk[0], m1 = mk[1];
-      any = (m0.x | m0.y | m0.z | m0.w | m1.x | m1.y | m1.z | m1.w) != 0u;
-    }
-    unsigned todo = __ballot_sync(FULL_MASK, any);
-    while (todo) {
-    const int jj = __ffs(todo) - 1;
-    todo &= todo - 1;
-    int4 w;
-    w.x = __shfl_sync(FULL_MASK, wj.x, jj);
-    w.y = __shfl_sync(FULL_MASK, wj.y, jj);
-    w.z = __shfl_sync(FULL_MASK, wj.z, jj);
-    w.w = __shfl_sync(FULL_MASK, wj.w, jj);
-    unsigned rem = L.rem_mask[(size_t)w.x * 32 + lane];
-    GridHaloState& S = L.state[w.y];
-    const HaloDev& H = L.halos[w.y];
-    const int s_v = S.s_mv;
-    Acc mv0 = 0, mv1 = 0, mv2 = 0;
-    if (rem) {
-      // the lane's removed elements: their candidate positions, then their
-      // records, each round's loads issued together
-      const long long g0 = (long long)w.z + lane * EPL;
-      uint32_t pos[EPL];
-#pragma unroll
-      for (int e = 0; e < EPL; ++e)
-        if ((rem >> e) & 1u) pos[e] = L.val_x[g0 + e];
-      V4 vm[EPL];
-#pragma unroll
-      for (int e = 0; e < EPL; ++e)
-        if ((rem >> e) & 1u) vm[e] = vr ? vr[g0 + e] : rec[2 * (H.gbase + pos[e]) + 1];  // (v, m)
-#pragma unroll
-      for (int e = 0; e < EPL; ++e) {
-        if (!((rem >> e) & 1u)) continue;
-        const long long g = g0 + e;
-        // removed: the sign bit of r, set without reading r
-        if (sizeof(R) == 4) atomicOr((unsigned*)&wr[g].w, 0x80000000u);
-        else atomicOr((unsigned long long*)&wr[g].w, 0x8000000000000000ull);
-        if (L.out.removed_iter) L.out.removed_iter[H.offset + pos[e]] = pass;
-        const R m = UNIF ? m0 : ((const R*)L.ms)[g];
-        add_fix(mv0, mul_rn(m, vm[e].x), s_v);
-        add_fix(mv1, mul_rn(m, vm[e].y), s_v);
-        add_fix(mv2, mul_rn(m, vm[e].z), s_v);
-      }
-    }
-    mv0 = wsum(mv0);
-    mv1 = wsum(mv1);
-    mv2 = wsum(mv2);
-    if (lane == 0) {
-      atomic_acc(S.rem_mv[0], mv0);
-      atomic_acc(S.rem_mv[1], mv1);
-      atomic_acc(S.rem_mv[2], mv2);
-    }
-    }
+      pass_sub<R, UNIF, GAS, false>(L, w, pass, removed_list[threadIdx.x >> 5]);
   }
 }
 
@@ -2563,7 +2522,7 @@ __device__ __forceinline__ float4 box_at(const float4* box, int lane, int i) { r
 // One sub-tile from its box in shared memory (the mixed mode, a uniform
 // particle mass, no gas): the arithmetic of pass_sub.
 template <bool FAST>
-__device__ __forceinline__ void pass_box(const GridLaunch& L, const int4 w, int pass, const float4* box) {
+__device__ __forceinline__ void pass_box(const GridLaunch& L, const int4 w, int pass, const float4* box, uint8_t* list) {
   using Acc = long long;
   const int u = w.x, k = w.y, t = u / SPT;
   GridHaloState& S = L.state[k];
@@ -2634,8 +2593,10 @@ __device__ __forceinline__ void pass_box(const GridLaunch& L, const int4 w, int 
   }
   const int nrem = __reduce_add_sync(FULL_MASK, __popc(rem));
   nband = __reduce_add_sync(FULL_MASK, nband);
-  L.rem_mask[(size_t)u * 32 + lane] = (uint8_t)rem;
-  if (nrem) rr = wsum(rr);
+  if (nrem) {
+    rr = wsum(rr);
+    removed<float, true>(L, w, pass, rem, nrem, list);
+  }
   if (lane == 0) {
     const size_t j = (size_t)(cp ^ 1) * n_sub + u;
     ((Acc*)L.agg_m)[j] = n_m - (Acc)nrem * mfix0;
@@ -2652,6 +2613,7 @@ __device__ __forceinline__ void pass_box(const GridLaunch& L, const int4 w, int 
 constexpr int TMA_SMEM = NWARP * 2 * 4096 + NWARP * 2 * 8;
 __global__ void __launch_bounds__(T, 3) g_pass_tma(const __grid_constant__ GridLaunch L, int pass) {
   extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ uint8_t removed_list[NWARP][SUB];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float4* box0 = (float4*)(smem + warp * 8192);
   uint64_t* bar = (uint64_t*)(smem + NWARP * 8192) + 2 * warp;
@@ -2693,8 +2655,8 @@ __global__ void __launch_bounds__(T, 3) g_pass_tma(const __grid_constant__ GridL
     if (b) phase1 ^= 1;
     else phase0 ^= 1;
     const GridHaloState& S = L.state[w.y];
-    if (pow2_neg(S.s_m) != 0.0f && pow2_neg(S.s_mr) != 0.0f) pass_box<true>(L, w, pass, box0 + b * 256);
-    else pass_box<false>(L, w, pass, box0 + b * 256);
+    if (pow2_neg(S.s_m) != 0.0f && pow2_neg(S.s_mr) != 0.0f) pass_box<true>(L, w, pass, box0 + b * 256, removed_list[warp]);
+    else pass_box<false>(L, w, pass, box0 + b * 256, removed_list[warp]);
     w = wn;
   }
 }
@@ -3079,8 +3041,6 @@ cudaError_t iterate_t(const GridLaunch& L, int pass, cudaStream_t s) {
   else if (!unif && !gas) g_pass<R, false, false><<<L.iter_grid, T, 0, s>>>(L, pass);
   else if (unif) g_pass<R, true, true><<<L.iter_grid, T, 0, s>>>(L, pass);
   else g_pass<R, false, true><<<L.iter_grid, T, 0, s>>>(L, pass);
-  if (unif) g_removed<R, true><<<L.iter_grid, T, 0, s>>>(L, pass);
-  else g_removed<R, false><<<L.iter_grid, T, 0, s>>>(L, pass);
   if (L.max_halo_tiles > 64) g_halo<R, false, HT_BIG><<<halo_ctas(L, HT_BIG), HT_BIG, 0, s>>>(L, pass);
   else g_halo<R, false, HT_SMALL><<<halo_ctas(L, HT_SMALL), HT_SMALL, 0, s>>>(L, pass);
   return cudaGetLastError();

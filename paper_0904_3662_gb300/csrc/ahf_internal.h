@@ -257,8 +257,6 @@ struct GridLaunch {
   long long* pre_c;
   AccSlot* tile_mv;        // [n_tiles][3]: sum m v of each tile's members (initial set)
   SkipRec* skip;           // [n_tiles * GRID_TILE / GRID_SUB]: the last test of each sub-tile
-  uint8_t* rem_mask;       // [n_tiles * GRID_TILE / GRID_SUB][32]: removal flags of the last
-                           // pass, one byte per lane (bit i: the lane's element i)
   int4* work;              // [2][n_tiles * GRID_TILE / GRID_SUB]: the sub-tiles of the active
                            // haloes for the passes of each parity: (sub-tile, halo, first
                            // flat element, members in it)
