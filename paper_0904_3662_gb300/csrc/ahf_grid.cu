@@ -2465,8 +2465,11 @@ __device__ __forceinline__ void pass_sub(const GridLaunch& L, const int4 w, int 
 
 // One pass: warps take the listed sub-tiles (those of the active haloes)
 // round robin, and clear the count of the next pass's list.
-template <typename R, bool UNIF, bool GAS>
-__global__ void __launch_bounds__(T, sizeof(R) == 4 ? 2 : 1) g_pass(GridLaunch L, int pass) {
+// PER: CTAs an SM.  In FP64 one (211 registers, nothing spilt) while that gives
+// every sub-tile its warp, else two (128 registers): 3,000 haloes 1268 -> 1214 us
+// with two, one halo of 43 sub-tiles 266 us with one and 274 with two.
+template <typename R, bool UNIF, bool GAS, int PER>
+__global__ void __launch_bounds__(T, PER) g_pass(GridLaunch L, int pass) {
   __shared__ uint8_t removed_list[NWARP][SUB];
   if (blockIdx.x == 0 && threadIdx.x == 0) L.ctl->work_n[(pass + 1) & 1] = 0;
   if (gave_up(L)) return;
@@ -3027,6 +3030,15 @@ cudaError_t sort_t(GridLaunch& L, cudaStream_t s, unsigned long long or_bits, un
 
 std::atomic<unsigned long long> g_tma_attr{0};
 
+template <typename R, int PER>
+void launch_pass(const GridLaunch& L, int pass, int grid, cudaStream_t s) {
+  const bool unif = L.ms == nullptr, gas = L.uth != nullptr;
+  if (unif && !gas) g_pass<R, true, false, PER><<<grid, T, 0, s>>>(L, pass);
+  else if (!unif && !gas) g_pass<R, false, false, PER><<<grid, T, 0, s>>>(L, pass);
+  else if (unif) g_pass<R, true, true, PER><<<grid, T, 0, s>>>(L, pass);
+  else g_pass<R, false, true, PER><<<grid, T, 0, s>>>(L, pass);
+}
+
 template <typename R>
 cudaError_t iterate_t(const GridLaunch& L, int pass, cudaStream_t s) {
   const bool unif = L.ms == nullptr, gas = L.uth != nullptr;
@@ -3037,10 +3049,13 @@ cudaError_t iterate_t(const GridLaunch& L, int pass, cudaStream_t s) {
       mark_used_on_device(g_tma_attr);
     }
     g_pass_tma<<<L.tma_grid, T, TMA_SMEM, s>>>(L, pass);
-  } else if (unif && !gas) g_pass<R, true, false><<<L.iter_grid, T, 0, s>>>(L, pass);
-  else if (!unif && !gas) g_pass<R, false, false><<<L.iter_grid, T, 0, s>>>(L, pass);
-  else if (unif) g_pass<R, true, true><<<L.iter_grid, T, 0, s>>>(L, pass);
-  else g_pass<R, false, true><<<L.iter_grid, T, 0, s>>>(L, pass);
+  } else if constexpr (sizeof(R) == 4) {
+    launch_pass<R, 2>(L, pass, L.iter_grid, s);
+  } else if ((long long)L.n_tiles * SPT > (long long)L.iter_grid * NWARP) {
+    launch_pass<R, 2>(L, pass, 2 * L.iter_grid, s);
+  } else {
+    launch_pass<R, 1>(L, pass, L.iter_grid, s);
+  }
   if (L.max_halo_tiles > 64) g_halo<R, false, HT_BIG><<<halo_ctas(L, HT_BIG), HT_BIG, 0, s>>>(L, pass);
   else g_halo<R, false, HT_SMALL><<<halo_ctas(L, HT_SMALL), HT_SMALL, 0, s>>>(L, pass);
   return cudaGetLastError();
@@ -3066,7 +3081,7 @@ template <typename R>
 int iter_grid_t(int device) {
   int sms = 0, per = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, g_pass<R, true, false>, T, 0) != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, g_pass<R, true, false, (sizeof(R) == 4 ? 2 : 1)>, T, 0) != cudaSuccess) return 0;
   return sms * (per > 0 ? per : 1);
 }
 
