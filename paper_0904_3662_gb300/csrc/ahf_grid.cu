@@ -2187,9 +2187,11 @@ __global__ void __launch_bounds__(T, sizeof(R) == 4 ? 4 : 3) g_bin_sort(GridLaun
 constexpr int EPL = SUB / 32;            // 8 consecutive elements per lane
 
 // Prefix sums of a sub-tile's start: the tile's prefix plus the sums of the
-// tile's sub-tiles before it in copy `cp` (lanes < u % SPT read one each).
-template <typename Acc>
-__device__ __forceinline__ void sub_prefix(const GridLaunch& L, int u, int t, int cp, Acc& M, Acc& P, long long* C) {
+// tile's sub-tiles before it in copy `cp` (lanes < u % SPT read one each).  With
+// one mass for all (UNIF) M is the count times its fixed-point value mfix0.
+template <bool UNIF, typename Acc>
+__device__ __forceinline__ void sub_prefix(const GridLaunch& L, int u, int t, int cp, Acc mfix0, Acc& M, Acc& P,
+                                           long long* C) {
   const int lane = threadIdx.x & 31;
   const int n_sub = L.n_tiles * SPT;
   const int ui = u % SPT;
@@ -2197,13 +2199,16 @@ __device__ __forceinline__ void sub_prefix(const GridLaunch& L, int u, int t, in
   int c = 0;
   if (lane < ui) {
     const size_t j = (size_t)cp * n_sub + (u - ui) + lane;
-    m = ((const Acc*)L.agg_m)[j];
+    if (!UNIF) m = ((const Acc*)L.agg_m)[j];
     r = ((const Acc*)L.agg_r)[j];
-    if (C) c = L.agg_c[j];
+    if (UNIF || C) c = L.agg_c[j];
   }
-  M = ((const Acc*)L.pre_m)[t] + wsum(m);
   P = ((const Acc*)L.pre_r)[t] + wsum(r);
-  if (C) *C = L.pre_c[t] + __reduce_add_sync(FULL_MASK, c);
+  long long n = 0;
+  if (UNIF || C) n = L.pre_c[t] + __reduce_add_sync(FULL_MASK, c);
+  if (UNIF) M = (Acc)n * mfix0;
+  else M = ((const Acc*)L.pre_m)[t] + wsum(m);
+  if (C) *C = n;
 }
 
 // The skip record of sub-tile u from the lanes' margins and |u|^2 maxima
@@ -2385,29 +2390,31 @@ __device__ __forceinline__ void pass_sub(const GridLaunch& L, const int4 w, int 
       uq[i] = (R)0;
     }
   }
+  const Acc mfix0 = fixp(m0, s_m);
   Acc M, Pp;
-  sub_prefix<Acc>(L, u, t, cp, M, Pp, nullptr);
+  sub_prefix<UNIF>(L, u, t, cp, mfix0, M, Pp, nullptr);
   R vb[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) vb[a] = sizeof(R) == 4 ? (R)S.vbulk[a] : (R)S.vbulk_d[a];
   const R band = sizeof(R) == 4 ? (R)P.band_f : (R)P.band;
   const Acc Ttot = Ald<Acc>(S.t_tot);
   const float sc_m = FAST ? pow2_neg(s_m) : 0.0f, sc_r = FAST ? pow2_neg(s_r) : 0.0f;
-  const Acc mfix0 = fixp(m0, s_m);
   // per element: 1/r and the exact terms; the lane's sums
   Acc rf[EPL];
   Acc a = 0, b = 0;
+  uint32_t na = 0;
 #pragma unroll
   for (int i = 0; i < EPL; ++i) {
     const bool alive = !signbit(q[i].w);
     if (!has_ri) ri[i] = rinv_real(q[i].w, P);
     rf[i] = alive ? fixp(mq[i] * ri[i], s_r) : (Acc)0;
-    if (alive) a += UNIF ? mfix0 : fixp(mq[i], s_m);
+    if (UNIF) na += alive ? 1u : 0u;
+    else if (alive) a += fixp(mq[i], s_m);
     b += rf[i];
   }
-  const Acc ia = wscan(a, lane), ib = wscan(b, lane);
-  M += ia - a;
-  Pp += ib - b;
+  if (UNIF) M += (Acc)(wscan(na, lane) - na) * mfix0;
+  else M += wscan(a, lane) - a;
+  Pp += wscan(b, lane) - b;
   const size_t jc = (size_t)cp * n_sub + u;
   const Acc n_m = ((const Acc*)L.agg_m)[jc], n_r = ((const Acc*)L.agg_r)[jc];
   const int n_c = L.agg_c[jc];
@@ -2535,17 +2542,17 @@ __device__ __forceinline__ void pass_box(const GridLaunch& L, const int4 w, int 
   const int n_sub = L.n_tiles * SPT;
   const int cp = pass & 1;
   const int nl = w.w - lane * EPL;                    // the lane's members (<= 0: none)
+  const float m0 = L.p.m0f;
+  const Acc mfix0 = fixp(m0, s_m);
   Acc M, Pp;
-  sub_prefix<Acc>(L, u, t, cp, M, Pp, nullptr);
+  sub_prefix<true>(L, u, t, cp, mfix0, M, Pp, nullptr);
   const float vb0 = S.vbulk[0], vb1 = S.vbulk[1], vb2 = S.vbulk[2];
   const float band = P.band_f;
   const Acc Ttot = Ald<Acc>(S.t_tot);
   const float sc_m = FAST ? pow2_neg(s_m) : 0.0f, sc_r = FAST ? pow2_neg(s_r) : 0.0f;
-  const float m0 = L.p.m0f;
-  const Acc mfix0 = fixp(m0, s_m);
   float ri[EPL];
   Acc rf[EPL];
-  Acc a = 0, b = 0;
+  Acc b = 0;
   unsigned alive = 0;
 #pragma unroll
   for (int i = 0; i < EPL; ++i) {
@@ -2554,12 +2561,11 @@ __device__ __forceinline__ void pass_box(const GridLaunch& L, const int4 w, int 
     alive |= (al ? 1u : 0u) << i;
     ri[i] = rinv_real(r, P);
     rf[i] = al ? fixp(m0 * ri[i], s_r) : 0ll;
-    a += al ? mfix0 : 0ll;
     b += rf[i];
   }
-  const Acc ia = wscan(a, lane), ib = wscan(b, lane);
-  M += ia - a;
-  Pp += ib - b;
+  const uint32_t na = (uint32_t)__popc(alive);
+  M += (Acc)(wscan(na, lane) - na) * mfix0;
+  Pp += wscan(b, lane) - b;
   const size_t jc = (size_t)cp * n_sub + u;
   const Acc n_m = ((const Acc*)L.agg_m)[jc], n_r = ((const Acc*)L.agg_r)[jc];
   const int n_c = L.agg_c[jc];
@@ -2709,7 +2715,8 @@ __global__ void __launch_bounds__(T, sizeof(R) == 4 ? 4 : 2) g_final(GridLaunch 
   const Acc Ttot = Ald<Acc>(S.t_tot);
   Acc M, Pp;
   long long C;
-  sub_prefix<Acc>(L, u, t, (S.n_iter + 1) & 1, M, Pp, &C);
+  const Acc mfix0 = fixp(m0, s_m);
+  sub_prefix<UNIF>(L, u, t, (S.n_iter + 1) & 1, mfix0, M, Pp, &C);
   const float sc_m = pow2_neg(s_m), sc_r = pow2_neg(s_r);
   const unsigned below = lanemask_lt();
 #pragma unroll
@@ -2717,14 +2724,15 @@ __global__ void __launch_bounds__(T, sizeof(R) == 4 ? 4 : 2) g_final(GridLaunch 
     const R r = rq[i];
     const bool alive = !signbit(r) && (long long)tr.x + e0 + 32 * i + lane < lim;
     const R ri = has_ri ? ri_q[i] : rinv_real(r, P);
-    const Acc a = alive ? (Acc)fixp(mq[i], s_m) : (Acc)0;
+    const Acc a = UNIF || !alive ? (Acc)0 : (Acc)fixp(mq[i], s_m);
     const Acc b = alive ? (Acc)fixp(mq[i] * ri, s_r) : (Acc)0;
     const unsigned bal = __ballot_sync(FULL_MASK, alive);
     if (bal == 0u) continue;
-    const Acc ia = wscan(a, lane), ib = wscan(b, lane);
+    const Acc ia = UNIF ? (Acc)0 : wscan(a, lane), ib = wscan(b, lane);
     if (alive) {
       // M(<r) before the particle, and the outer sum from the particle out
-      const R phi = phi_real(fix_to_real(M + ia - a, s_m, sc_m, R()), ri,
+      const Acc Mi = UNIF ? M + (Acc)__popc(bal & below) * mfix0 : M + ia - a;
+      const R phi = phi_real(fix_to_real(Mi, s_m, sc_m, R()), ri,
                              fix_to_real(Ttot - (Pp + ib - b), s_r, sc_r, R()), P);
       const long long slot = H.offset + vq[i];
       const long long pi = L.out.member_idx ? L.out.member_idx[slot] : slot;
@@ -2732,9 +2740,10 @@ __global__ void __launch_bounds__(T, sizeof(R) == 4 ? 4 : 2) g_final(GridLaunch 
       L.out.bound_idx[H.offset + c] = pi;
       if (L.out.phi) ((R*)L.out.phi)[H.offset + c] = phi;
       rc[H.gbase + c] = r;
-      mc[H.gbase + c] = M + ia;
+      if (!UNIF) mc[H.gbase + c] = M + ia;     // (uniform: the rank times the mass)
     }
-    M += shfl_idx_x(ia, 31);
+    if (UNIF) M += (Acc)__popc(bal) * mfix0;
+    else M += shfl_idx_x(ia, 31);
     Pp += shfl_idx_x(ib, 31);
     C += __popc(bal);
   }
@@ -2754,6 +2763,8 @@ __global__ void __launch_bounds__(T) g_virial(GridLaunch L) {
   const long long gb = L.halos[k].gbase;
   const long long nb = S.n_alive;
   const ParamsDev& P = L.prm;
+  const bool unif = L.ms == nullptr;
+  const Acc mfix0 = fixp(sizeof(R) == 4 ? (R)L.p.m0f : (R)L.p.m0, S.s_m);
   long long kf = 0x7fffffffffffffffll;
   for (int e = threadIdx.x; e < tr.y; e += T) {
     const long long g = (long long)tr.x + e;
@@ -2761,7 +2772,7 @@ __global__ void __launch_bounds__(T) g_virial(GridLaunch L) {
     if (kk >= nb) break;
     bool cross = true;
     if (kk + 1 < nb) {
-      const Acc mk = mc[g];
+      const Acc mk = unif ? (Acc)(kk + 1) * mfix0 : mc[g];
       if (sizeof(R) == 4) {
         const float rn = (float)rc[g + 1];
         const float lhs = from_fix(mk, S.s_m, R());
