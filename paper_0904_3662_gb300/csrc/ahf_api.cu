@@ -932,7 +932,7 @@ int unbind_pass(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64
   // class they took them in the order in which the hardware came to the streams
   // (a process has 8 queues by default, and the classes that share one waited):
   // the clusters, which need whole SMs, then ran after the small haloes, 43 us
-  // into the 2,000-halo batch (318 us; 284 as a chain; 11,000 particles in one
+  // into the 2,000-halo batch (318 us; 284 as a chain in the same order; 11,000 particles in one
   // halo 70, now 65, without the fork and join; 20,000 haloes even).  With the
   // multi-CTA class the chain runs on a side stream beside it.  Phase times
   // (AHF_OPT_TIMING) and outputs pushed to host buffers, which record events or
@@ -946,11 +946,11 @@ int unbind_pass(ahf_ctx* c, const ahf_particles* p, const ahf_halo* halos, int64
   const bool chain = !c->serial && !c->timing && !push;
   int first_of[NV];
   for (int v = 0, f = 0; v < NV; ++v) { first_of[v] = f; f += P.n_class[v]; }
-  // launch order (the block scheduler serves earlier launches first): the
-  // clusters (largest haloes) first, then the single-CTA variants of 8k and
-  // 4k slots, then the warp variant, whose haloes run longer than the 1k
-  // variant's, then that one
-  constexpr int kOrder[NV] = {7, 6, 5, 4, 3, 2, 0, 1};
+  // launch order, largest haloes first: a class's haloes take about as long as
+  // each other, 140 us with 128k slots down to 45 (1k) and 40 (warps), and the
+  // short ones fill what the long ones leave.  2,000 haloes: 279 us; the warps
+  // before the 1k class 288, the 16-CTA clusters after the smaller ones 314.
+  constexpr int kOrder[NV] = {7, 6, 5, 4, 3, 2, 1, 0};
   for (int oi = 0; oi < NV; ++oi) {
     const int v = kOrder[oi];
     const int n = P.n_class[v];
