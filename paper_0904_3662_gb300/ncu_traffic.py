@@ -20,9 +20,9 @@ and then, anywhere:
 
 Phases: each on-chip size class is one kernel launch per call (the figure is
 the mean over its launches); each multi-CTA phase is several kernels per call
-(prepare + radix passes; the passes of the iteration; the final pass, virial
+(sample, prepare and radial bins, or radix passes; the passes of the iteration; the final pass, virial
 search, records and profile rows), whose figure is their sum per call, the
-calls counted by the one g_scales launch each call makes (a list that a launch
+calls counted by the one g_result launch each call makes (a list that a launch
 count cut off inside a call is read up to its last complete call).
 """
 from __future__ import annotations
@@ -50,8 +50,8 @@ GRID_PHASES = (8, 9, 10)
 _ONCHIP_CLASS = {(128, 1024, 1): 1, (256, 4096, 1): 2, (512, 8192, 1): 3, (512, 8192, 2): 4,
                  (512, 8192, 4): 5, (512, 8192, 8): 6, (512, 8192, 16): 7}
 _GRID_KERNELS = [
-    (8, r"g_prepare_|g_scales|g_hist|g_digit_scan|g_digit_base|g_scatter|g_fill_identity|g_sums|g_halo<[^,]+, (true|1),"),
-    (9, r"g_pass|g_removed|g_halo<[^,]+, (false|0),"),
+    (8, r"g_sample|g_bin_|g_place|g_prepare_|g_scales|g_hist|g_digit_scan|g_digit_base|g_scatter|g_fill_identity|g_sums|g_halo<[^,]+, (true|1),"),
+    (9, r"g_pass|g_halo<[^,]+, (false|0),"),
     (10, r"g_final|g_virial|g_result|g_rows_"),
 ]
 # values in bytes, nanoseconds and instructions whatever unit a row names
@@ -119,10 +119,8 @@ def summarize(launches):
         while last + 1 < len(launches) and phase_of(launches[last + 1][1]) == 10:
             last += 1                      # the profile rows after the record
         launches = launches[:last + 1]
-    calls = 0
+    calls = len(ends) or sum("g_scales" in name for _, name, _ in launches)
     for _, name, m in launches:
-        if "g_scales" in name:
-            calls += 1
         ph = phase_of(name)
         if ph is None:
             continue
