@@ -2077,7 +2077,11 @@ __global__ void __launch_bounds__(T, sizeof(R) == 4 ? 4 : 3) g_bin_sort(GridLaun
     }
     __syncthreads();
     const uint32_t v0 = pcnt[2 * threadIdx.x], v1 = pcnt[2 * threadIdx.x + 1];
-    if (max(v0, v1) > PART_MAX) L.ctl->overflow = 1;
+    // (one decision for the CTA: no member of it has a place yet, and nothing
+    // below may read one)
+    const bool many = max(v0, v1) > PART_MAX;
+    if (many) L.ctl->overflow = 1;
+    if (__syncthreads_or(many)) return;
     const uint32_t ex = block_excl(v0 + v1, red);
     __syncthreads();
     pcnt[2 * threadIdx.x] = ex;
@@ -2101,7 +2105,6 @@ __global__ void __launch_bounds__(T, sizeof(R) == 4 ? 4 : 3) g_bin_sort(GridLaun
   for (int own = threadIdx.x; own < n; own += T) {
     const uint32_t p = spart[own];
     const uint32_t a = pcnt[p], z = pcnt[p + 1];
-    if (z - a > PART_MAX) continue;      // the overflow word is set: nothing of this attempt is used
     const Key key = skey[own];
     uint32_t q = a, ties = 0u;
     for (uint32_t x = a; x < z; ++x) {

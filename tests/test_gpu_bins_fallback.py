@@ -1,0 +1,76 @@
+"""The multi-CTA class where radial bins give way to the radix sort, against the
+oracle: equal radii up to what a part holds and one more, in a halo of one tile
+(one bin, a map of its own) and of several, with gas and member lists, whose
+arrays the ordering of a bin reads by the places it has found."""
+import numpy as np
+import pytest
+
+from paper_0904_3662_gb300 import synth
+from tests.gpu_util import require_gpu, run_gpu
+from tests.parity import compare, fp64_rtol
+from tests.test_gpu_bins import _nfw, _population
+
+pytestmark = pytest.mark.gpu
+
+PART = 512                                                 # members a part of a bin holds
+
+
+def _shell(rng, n, ties):
+    """n particles, the first `ties` of them at one radius, the others well inside."""
+    d = rng.standard_normal((n, 3))
+    d *= (rng.uniform(5.0, 35.0, n) / np.linalg.norm(d, axis=1))[:, None]
+    d[:ties] = np.where(rng.uniform(size=(ties, 3)) < 0.5, -1.0, 1.0) * np.array([30.0, 40.0, 50.0])
+    return d, 20.0 * rng.standard_normal((n, 3)), 100.0
+
+
+def _shuffled(pop, rng):
+    """The particle store in another order, and the member list that undoes it."""
+    perm = rng.permutation(pop.n_particles).astype(np.int64)
+    for k in ("x", "y", "z", "vx", "vy", "vz", "m", "u_th"):
+        a = getattr(pop, k)
+        if a is not None:
+            b = np.empty_like(a)
+            b[perm] = a
+            setattr(pop, k, b)
+    return perm
+
+
+def _run(pop, mode, member_idx=None):
+    require_gpu()
+    from paper_0904_3662_gb300 import ahf
+    fp64 = mode == "fp64"
+    prm = ahf.params_for(pop, precision=ahf.PREC_FP64 if fp64 else ahf.PREC_MIXED)
+    ctx = ahf.Context(0)
+    ctx.set_option(ahf.OPT_ONCHIP_MAX, 0)                  # every halo to the multi-CTA class
+    out, prm, ctx, _ = run_gpu(pop, params=prm, ctx=ctx, member_idx=member_idx)
+    tol = fp64_rtol(pop) if fp64 else 1e-5
+    compare(pop, prm, out["res"], out["bound_idx"], out["phi"], out["removed_iter"], member_idx=member_idx,
+            phi_rtol=tol, vir_rtol=tol, exact_order=fp64)
+    # the radix sort reads the keys' range back: two synchronisations more
+    # than the reads of the pass chunks (8 passes each)
+    return ctx.stats(), ctx.stats()["host_syncs"] - -(-int(out["res"]["n_iter"].max()) // 8) >= 2
+
+
+def _coord(mode):
+    return synth.COORD_F64 if mode == "fp64" else synth.COORD_F32_REL
+
+
+@pytest.mark.parametrize("mode", ["mixed", "fp64"])
+@pytest.mark.parametrize("n,ties", [(600, PART), (600, PART + 1), (2000, 2000), (5000, PART + 1)])
+def test_equal_radii_around_what_a_part_holds(n, ties, mode):
+    pop = _population([_shell(np.random.default_rng(n + ties), n, ties)], _coord(mode))
+    _, radix = _run(pop, mode)
+    assert radix == (ties > PART)
+
+
+@pytest.mark.parametrize("masses", [False, True])
+@pytest.mark.parametrize("mode", ["mixed", "fp64"])
+@pytest.mark.parametrize("gas,members", [(True, False), (False, True), (True, True)])
+def test_fallback_with_gas_and_member_lists(gas, members, mode, masses):
+    rng = np.random.default_rng(41)
+    pop = _population([_nfw(rng, 3000), _shell(rng, 5000, 900), _shell(rng, 700, 650), _nfw(rng, 300)], _coord(mode),
+                      masses)
+    if gas:
+        pop = synth.with_gas(pop, frac=0.3, u_max=1e3)
+    _, radix = _run(pop, mode, _shuffled(pop, rng) if members else None)
+    assert radix
