@@ -332,7 +332,7 @@ constexpr int CLUSTER_CELLS = 1024; // cells a cluster divides its members by
 // takes two barriers, a ranking by lane matching and a store per key byte:
 // 42 -> 20 us per halo in clusters of 2 and 4 CTAs, 46 -> 23 of 8, 55 -> 23 of 16.
 // CTA r's share is radially below CTA r + 1's; what it holds is its own (nrec;
-// not the chunk of the candidates), in order, in (kA, vA) or (kB, vB) (0 or 1
+// not the chunk of the candidates), in order, in (kA, vA) of every CTA (0
 // returned).  -1, with everything as it was, when a share would not fit.
 template <int NT, int IPT, int CS>
 __device__ int cluster_dist_sort(uint32_t* kA, uint32_t* vA, uint32_t* kB, uint32_t* vB, uint32_t* ex1, uint32_t* ex2,
@@ -475,12 +475,21 @@ __device__ int cluster_dist_sort(uint32_t* kA, uint32_t* vA, uint32_t* kB, uint3
   if (dist_sort<NT, SORT_CELLS>(kA, vA, kB, vB, ex2, ex1, hist, wtot, vA, nrec, nrec, S.min_key, S.max_key, tid))
     return 0;
   // dozens of equal radii: the counting radix sort of this CTA's share (its
-  // counters in ex1 and ex2)
+  // counters in ex1 and ex2), brought to the buffer that dist_sort leaves it in:
+  // every CTA has the order in the same arrays, at whose addresses the CTAs read
+  // one another's radii (Cl::at)
   static_assert(count_sort_words(NT) <= 2 * CAP, "counters fit");
   const uint32_t differ = S.max_key ^ S.min_key;
   const uint32_t diff = differ ? 0xffffffffu >> __clz(differ) : 0u;
-  return count_sort<NT, (run_length(CAP, NT) + 3) / 4 * 4>(kA, vA, kB, vB, ex1, wtot, nrec, run_length(nrec, NT), diff,
-                                                           0u, tid);
+  if (count_sort<NT, (run_length(CAP, NT) + 3) / 4 * 4>(kA, vA, kB, vB, ex1, wtot, nrec, run_length(nrec, NT), diff, 0u,
+                                                        tid)) {
+    for (int i = tid; i < nrec; i += NT) {
+      kA[i] = kB[i];
+      vA[i] = vB[i];
+    }
+    __syncthreads();
+  }
+  return 0;
 }
 
 constexpr int NT_1K = 128, NT_4K = 256, NT_8K = 512, NT_CL = 512;
