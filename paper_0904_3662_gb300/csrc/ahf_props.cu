@@ -120,9 +120,15 @@ __device__ __forceinline__ float block_max(float x, uint32_t* word) {
   return __uint_as_float(*word);
 }
 
-// The float M^2 / r^2 a particle is first judged by (-1: at the centre).
+__device__ __forceinline__ bool is_normal(float x) { return x >= 1.17549435e-38f && x <= 3.40282347e+38f; }
+
+// The float M^2 / r^2 a particle is first judged by: within 1e-6 of the exact
+// value while M^2, r^2 and their quotient are normal floats; where one is not
+// (SI units: r^2 ~ 1e42; masses below 1e-19), infinite, which leaves the chunk to
+// FP64.  -1: at the centre (r2 = 0).
 __device__ __forceinline__ float peak_guess(float m, float r2f, double r2) {
-  if (r2f > 0.0f) return m * m / r2f;
+  const float m2 = m * m, q = m2 / r2f;
+  if (is_normal(m2) && is_normal(r2f) && is_normal(q)) return q;
   return r2 > 0.0 ? INFINITY : -1.0f;
 }
 // What it has to reach: the chunk's largest less 1e-5 (all of them when float
@@ -212,8 +218,8 @@ __global__ void __launch_bounds__(PT) props_uniform(PropsLaunch L) {
       s[10] += phi;
       const float fx = double_to_float(d[0]), fy = double_to_float(d[1]), fz = double_to_float(d[2]);
       const float r2f = fmaf(fz, fz, fmaf(fy, fy, fx * fx));
-      const bool tiny = !(r2f > 0.0f);
-      q[j] = peak_guess((float)(int)(start + e + 1), r2f, tiny ? d[0] * d[0] + d[1] * d[1] + d[2] * d[2] : 0.0);
+      q[j] = peak_guess((float)(int)(start + e + 1), r2f,
+                        is_normal(r2f) ? 1.0 : d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
       qm = fmaxf(qm, q[j]);
     }
   }
