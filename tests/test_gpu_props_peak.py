@@ -1,11 +1,14 @@
-"""The rotation curve's peak (ahf_halo_properties) in units whose squares leave the
-range of a float, against the oracle."""
+"""The rotation curve's peak (ahf_halo_properties): in units whose squares leave
+the range of a float, against the oracle; and where thousands of particles tie
+to rounding, the same bytes from every call."""
 import dataclasses
 
+import numpy as np
 import pytest
 
 from paper_0904_3662_gb300 import synth
 from tests.gpu_util import require_gpu
+from tests.test_gpu_bins import _population
 from tests.test_gpu_props import _check_props, _run
 
 pytestmark = pytest.mark.gpu
@@ -41,3 +44,24 @@ def test_peak_with_small_masses(length, mass):
     small, kw = _scaled(pop, length, mass, 1.0)
     _, prm, _, host = _run(small, **kw)
     assert _check_props(small, prm, host, 1e-5) >= 14
+
+
+@pytest.mark.parametrize("masses", [False, True])
+def test_peak_of_a_flat_curve_is_repeatable(masses):
+    # M(<= r_i) / r_i the same to rounding for every particle: the first of the
+    # largest, whatever order the threads come in
+    torch = require_gpu()
+    from paper_0904_3662_gb300 import ahf
+    n = 2048
+    pos = np.zeros((n, 3))
+    pos[:, 0] = 0.01 * np.arange(1, n + 1)
+    pop = _population([(pos, np.zeros((n, 3)), 100.0)] * 32, synth.COORD_F64)
+    if masses:
+        pop.m = np.full(pop.n_particles, pop.m0)
+    ctx, prm, out, host = _run(pop, precision=ahf.PREC_FP64, H=0.0)
+    assert np.all(host["props"][:, 0] == n)
+    parts, hal = ahf.particles_from_population(pop), ahf.halos_from_population(pop)
+    for _ in range(20):
+        props = ctx.halo_properties(parts, hal, prm, out)
+        assert props.cpu().numpy().tobytes() == host["props"].tobytes()
+    assert np.all(host["props"] == host["props"][0])       # (32 equal haloes)
