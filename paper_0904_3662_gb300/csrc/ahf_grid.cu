@@ -503,10 +503,11 @@ __device__ __forceinline__ void merge_prepare(const GridLaunch& L, int k, unsign
 // ordering by issue slots (65 % busy).
 //
 // A bin holds BIN_MAX members at most (its CTA's shared memory).  When one would
-// hold more (thousands of equal radii, a thin shell in a void), or a part so
-// many that ordering it by counting would be slow, ctl->overflow is set, every
-// later kernel of the attempt returns at once and the host runs the radix sort
-// instead.
+// hold more (thousands of equal radii, a thin shell in a void), ctl->overflow is
+// set, every later kernel of the attempt returns at once and the host runs the
+// radix sort instead.  A bin in which a part holds so many that ordering it by
+// counting would be slow (hundreds of equal radii) is ordered by comparisons
+// (order_tied).
 
 constexpr int CELLS = 1024;              // at most
 constexpr int SAMPLE_T = 1024;
@@ -518,7 +519,7 @@ constexpr uint32_t TAB_UNIT = 2u;        // bin tables count in halves of a part
 constexpr uint32_t NO_RANK = 0xffffu;    // rank of a non-member
 static_assert(PARTS == 2 * T, "two parts a thread");
 constexpr int BIN_MAX = 3072;            // members of a bin
-constexpr uint32_t PART_MAX = 512u;      // members of a part
+constexpr uint32_t PART_MAX = 512u;      // members of a part ordered by counting
 constexpr int BIN_PAD = 32;              // words between bins' counters: atomics on one 128-byte line queue
 constexpr int AGG_BINS = 512;            // halo's bins up to which a CTA counts in shared memory first
 
@@ -2016,10 +2017,47 @@ __global__ void __launch_bounds__(HT) g_halo(GridLaunch L, int pass) {
   }
 }
 
+// The n members of a bin in order of (r, candidate position), for one in which a
+// part holds more than PART_MAX: a bitonic sort in shared memory with every
+// comparator pointing up, so that positions behind n need no padding.  78 rounds at
+// most, bound by their barriers.  Leaving such a bin to the radix sort instead sent
+// every halo of the call there, after the passes of a chunk without an active halo.
+template <typename Key>
+__device__ __noinline__ void order_tied(Key* skey, uint16_t* sidx, uint32_t* spos, int n) {
+  auto order = [&](int lo, int hi) {     // lo < hi
+    if (hi >= n) return;
+    const Key a = skey[lo], b = skey[hi];
+    const uint32_t p = spos[lo], q = spos[hi];
+    if (a < b || (a == b && p < q)) return;
+    const uint16_t x = sidx[lo];
+    skey[lo] = b;
+    skey[hi] = a;
+    spos[lo] = q;
+    spos[hi] = p;
+    sidx[lo] = sidx[hi];
+    sidx[hi] = x;
+  };
+  for (int half = 1; half < n; half <<= 1) {
+    // mirrored pairs of each block of 2 half, then pairs at distance d
+    for (int t = threadIdx.x; 2 * half * (t / half) + t % half < n; t += T) {
+      const int at = 2 * half * (t / half);
+      order(at + t % half, at + 2 * half - 1 - t % half);
+    }
+    __syncthreads();
+    for (int d = half >> 1; d > 0; d >>= 1) {
+      for (int t = threadIdx.x; 2 * d * (t / d) + t % d < n; t += T) {
+        const int at = 2 * d * (t / d) + t % d;
+        order(at, at + d);
+      }
+      __syncthreads();
+    }
+  }
+}
+
 // A bin ordered, one CTA each: its members counted in the bin's 512 parts in
 // shared memory, their keys moved there, and each member's place in its part
 // found by counting the members before it in (r, candidate).  Then, in
-// radial order, the streams (w, r), (v, m), the position (and mass, thermal
+// radial order, the streams (w, r), (v, 1/r), the position (and mass, thermal
 // energy), the exact sum m v, and the sub-tiles' sums of the initial set.
 template <typename R>
 __global__ void __launch_bounds__(T, sizeof(R) == 4 ? 4 : 3) g_bin_sort(GridLaunch L) {
@@ -2032,12 +2070,12 @@ __global__ void __launch_bounds__(T, sizeof(R) == 4 ? 4 : 3) g_bin_sort(GridLaun
   uint16_t* sidx = reinterpret_cast<uint16_t*>(skey + BIN_MAX);  // [BIN_MAX] slot -> source
   uint16_t* sout = sidx + BIN_MAX;                               // [BIN_MAX] place -> source
   uint16_t* spart = sout + BIN_MAX;                              // [BIN_MAX] slot -> part
+  uint32_t* spos = reinterpret_cast<uint32_t*>(sout);            // order_tied: candidate positions
   __shared__ uint32_t tab[CELLS + 1];
   __shared__ uint32_t pcnt[PARTS + 1];
   __shared__ uint32_t red[NWARP];
   __shared__ Acc racc[NWARP];
-  // (another CTA may set the word meanwhile: one decision for the CTA)
-  if (__syncthreads_or(bins_overflowed(L))) return;
+  if (bins_overflowed(L)) return;
   const int bin = blockIdx.x, t = bin >> 1;
   const int k = L.tile_halo[t];
   const HaloDev& H = L.halos[k];
@@ -2077,48 +2115,59 @@ __global__ void __launch_bounds__(T, sizeof(R) == 4 ? 4 : 3) g_bin_sort(GridLaun
     }
     __syncthreads();
     const uint32_t v0 = pcnt[2 * threadIdx.x], v1 = pcnt[2 * threadIdx.x + 1];
-    // (one decision for the CTA: no member of it has a place yet, and nothing
-    // below may read one)
-    const bool many = max(v0, v1) > PART_MAX;
-    if (many) L.ctl->overflow = 1;
-    if (__syncthreads_or(many)) return;
-    const uint32_t ex = block_excl(v0 + v1, red);
-    __syncthreads();
-    pcnt[2 * threadIdx.x] = ex;
-    pcnt[2 * threadIdx.x + 1] = ex + v0;
-    if (threadIdx.x == T - 1) pcnt[PARTS] = ex + v0 + v1;
-    __syncthreads();
+    // (one way for the whole CTA)
+    if (__syncthreads_or(max(v0, v1) > PART_MAX)) {
 #pragma unroll
-    for (int j = 0; j < NE; ++j) {
-      if (j * T >= n) break;
-      const int i = j * T + threadIdx.x;
-      if (i < n) {
-        const uint32_t q = pcnt[slot[j] >> 16] + (slot[j] & 0xffffu);
-        skey[q] = key[j];
-        sidx[q] = (uint16_t)i;
-        spart[q] = (uint16_t)(slot[j] >> 16);
+      for (int j = 0; j < NE; ++j) {
+        const int i = j * T + threadIdx.x;
+        if (i < n) {
+          skey[i] = key[j];
+          sidx[i] = (uint16_t)i;
+          spos[i] = binned_pos(rb[2 * i + 1].w);
+        }
+      }
+      __syncthreads();
+      order_tied(skey, sidx, spos, n);
+      for (int q = threadIdx.x; q < n; q += T) sout[q] = sidx[q];
+    } else {
+      const uint32_t ex = block_excl(v0 + v1, red);
+      __syncthreads();
+      pcnt[2 * threadIdx.x] = ex;
+      pcnt[2 * threadIdx.x + 1] = ex + v0;
+      if (threadIdx.x == T - 1) pcnt[PARTS] = ex + v0 + v1;
+      __syncthreads();
+#pragma unroll
+      for (int j = 0; j < NE; ++j) {
+        if (j * T >= n) break;
+        const int i = j * T + threadIdx.x;
+        if (i < n) {
+          const uint32_t q = pcnt[slot[j] >> 16] + (slot[j] & 0xffffu);
+          skey[q] = key[j];
+          sidx[q] = (uint16_t)i;
+          spart[q] = (uint16_t)(slot[j] >> 16);
+        }
+      }
+      __syncthreads();
+      // in slot order: a warp's members are in neighbouring parts
+      for (int own = threadIdx.x; own < n; own += T) {
+        const uint32_t p = spart[own];
+        const uint32_t a = pcnt[p], z = pcnt[p + 1];
+        const Key mine = skey[own];
+        uint32_t q = a, ties = 0u;
+        for (uint32_t x = a; x < z; ++x) {
+          const Key kx = skey[x];
+          q += kx < mine ? 1u : 0u;
+          ties += kx == mine ? 1u : 0u;
+        }
+        const uint32_t ip = sidx[own];
+        if (ties > 1u) {                 // equal radii: in candidate order
+          const uint32_t pos = binned_pos(rb[2 * ip + 1].w);
+          for (uint32_t x = a; x < z; ++x)
+            if (skey[x] == mine && binned_pos(rb[2 * (uint32_t)sidx[x] + 1].w) < pos) ++q;
+        }
+        sout[q] = (uint16_t)ip;
       }
     }
-  }
-  __syncthreads();
-  // in slot order: a warp's members are in neighbouring parts
-  for (int own = threadIdx.x; own < n; own += T) {
-    const uint32_t p = spart[own];
-    const uint32_t a = pcnt[p], z = pcnt[p + 1];
-    const Key key = skey[own];
-    uint32_t q = a, ties = 0u;
-    for (uint32_t x = a; x < z; ++x) {
-      const Key kx = skey[x];
-      q += kx < key ? 1u : 0u;
-      ties += kx == key ? 1u : 0u;
-    }
-    const uint32_t ip = sidx[own];
-    if (ties > 1u) {                     // equal radii: in candidate order
-      const uint32_t pos = binned_pos(rb[2 * ip + 1].w);
-      for (uint32_t x = a; x < z; ++x)
-        if (skey[x] == key && binned_pos(rb[2 * (uint32_t)sidx[x] + 1].w) < pos) ++q;
-    }
-    sout[q] = (uint16_t)ip;
   }
   __syncthreads();
   // the streams in radial order, a warp taking rows of 32; sums by sub-tile

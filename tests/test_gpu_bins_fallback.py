@@ -1,7 +1,8 @@
-"""The multi-CTA class where radial bins give way to the radix sort, against the
-oracle: equal radii up to what a part holds and one more, in a halo of one tile
-(one bin, a map of its own) and of several, with gas and member lists, whose
-arrays the ordering of a bin reads by the places it has found."""
+"""The multi-CTA class where radii are equal by the hundred, against the oracle:
+around what a part of a radial bin holds (its bin is then ordered by comparisons),
+in a halo of one tile (one bin, a map of its own) and of several; and by the
+thousand, more than a bin holds, where the radix sort takes over.  With gas and
+member lists, whose arrays the ordering of a bin reads by the places it has found."""
 import numpy as np
 import pytest
 
@@ -12,7 +13,8 @@ from tests.test_gpu_bins import _nfw, _population
 
 pytestmark = pytest.mark.gpu
 
-PART = 512                                                 # members a part of a bin holds
+PART = 512                                                 # members of a part ordered by counting
+BIN = 3072                                                 # members of a bin
 
 
 def _shell(rng, n, ties):
@@ -56,21 +58,59 @@ def _coord(mode):
 
 
 @pytest.mark.parametrize("mode", ["mixed", "fp64"])
-@pytest.mark.parametrize("n,ties", [(600, PART), (600, PART + 1), (2000, 2000), (5000, PART + 1)])
-def test_equal_radii_around_what_a_part_holds(n, ties, mode):
+@pytest.mark.parametrize("n,ties", [(600, PART), (600, PART + 1), (1024, 1023), (2000, 1025), (2000, 2000),
+                                    (5000, PART + 1), (9000, 1500), (9000, BIN + 1)])
+def test_equal_radii_around_what_a_part_and_a_bin_hold(n, ties, mode):
     pop = _population([_shell(np.random.default_rng(n + ties), n, ties)], _coord(mode))
     _, radix = _run(pop, mode)
-    assert radix == (ties > PART)
+    assert radix == (ties > BIN)
 
 
 @pytest.mark.parametrize("masses", [False, True])
 @pytest.mark.parametrize("mode", ["mixed", "fp64"])
 @pytest.mark.parametrize("gas,members", [(True, False), (False, True), (True, True)])
-def test_fallback_with_gas_and_member_lists(gas, members, mode, masses):
+@pytest.mark.parametrize("thousands", [False, True])
+def test_equal_radii_with_gas_and_member_lists(thousands, gas, members, mode, masses):
     rng = np.random.default_rng(41)
-    pop = _population([_nfw(rng, 3000), _shell(rng, 5000, 900), _shell(rng, 700, 650), _nfw(rng, 300)], _coord(mode),
-                      masses)
+    blocks = [_nfw(rng, 3000), _shell(rng, 5000, 900), _shell(rng, 700, 650), _nfw(rng, 300)]
+    pop = _population(blocks + [_shell(rng, 9000, 4000)] * thousands, _coord(mode), masses)
     if gas:
         pop = synth.with_gas(pop, frac=0.3, u_max=1e3)
     _, radix = _run(pop, mode, _shuffled(pop, rng) if members else None)
-    assert radix
+    assert radix == thousands
+
+
+def test_one_halo_with_equal_radii_leaves_the_others_in_bins():
+    # (the radix sort of every halo takes about as long as the whole call in bins)
+    torch = require_gpu()
+    import time
+    from paper_0904_3662_gb300 import ahf
+    rng = np.random.default_rng(43)
+    blocks = [_nfw(rng, int(n)) for n in rng.integers(300, 3000, 3000)]
+    took, outs = [], []
+    for ties in (PART, 900):
+        pop = _population(blocks[:1500] + [_shell(np.random.default_rng(3), 1200, ties)] + blocks[1500:], synth.COORD_F64)
+        prm = ahf.params_for(pop, precision=ahf.PREC_FP64)
+        ctx = ahf.Context(0)
+        parts, hal = ahf.particles_from_population(pop), ahf.halos_from_population(pop)
+        out = ctx.alloc_outputs(pop.n_halos, pop.n_particles, precision=ahf.PREC_FP64)
+        best = 1e9
+        for _ in range(6):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            ctx.unbind_batch(parts, hal, prm, out=out)
+            torch.cuda.synchronize()
+            best = min(best, time.perf_counter() - t)
+        took.append(best)
+        res = ahf.results_to_numpy(out["res"])
+        host = [out[k].cpu().numpy() for k in ("bound_idx", "phi", "removed_iter")]
+        tol = fp64_rtol(pop)
+        compare(pop, prm, res, *host, halos=[0, 700, 1499, 1500, 1501, 3000], phi_rtol=tol, vir_rtol=tol,
+                exact_order=True)
+        outs.append((res, host))
+    (ra, ha), (rb, hb) = outs
+    rest = np.arange(3001) != 1500
+    assert ra[rest].tobytes() == rb[rest].tobytes()
+    slot = np.repeat(rest, pop.count)
+    np.testing.assert_array_equal(ha[2][slot], hb[2][slot])
+    assert took[1] < 1.5 * took[0], took
