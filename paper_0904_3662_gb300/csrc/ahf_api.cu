@@ -671,9 +671,10 @@ int run_grid(ahf_ctx* c, GridLaunch& G, const ahf_params* prm, cudaStream_t s, i
     AHF_CUDA(cudaStreamSynchronize(s));
     c->stats.host_syncs += 1;
     if (!radix && c->flag_host[2]) {
-      // a radial bin overflowed (the passes above had no active halo): the
-      // radix sort orders any radii
+      // a radial bin overflowed (the passes above had no active halo, and do
+      // not count): the radix sort orders any radii
       radix = true;
+      c->stats.grid_iterations -= pass - 1;
       pass = 1;
       streams(false);
       if ((rc = grid_reset(G, s))) return rc;

@@ -80,6 +80,17 @@ def test_equal_radii_with_gas_and_member_lists(thousands, gas, members, mode, ma
     assert radix == thousands
 
 
+@pytest.mark.parametrize("mode", ["mixed", "fp64"])
+def test_abandoned_bins_do_not_count_as_iterations(mode):
+    st = {}
+    for ties in (PART, BIN + 1):
+        pop = _population([_shell(np.random.default_rng(7), 6000, ties)], _coord(mode))
+        st[ties], radix = _run(pop, mode)
+        assert radix == (ties > BIN)
+    # (8 passes to a chunk; each halo needs one chunk)
+    assert st[PART]["grid_iterations"] == st[BIN + 1]["grid_iterations"] == 8
+
+
 def test_one_halo_with_equal_radii_leaves_the_others_in_bins():
     # (the radix sort of every halo takes about as long as the whole call in bins)
     torch = require_gpu()
