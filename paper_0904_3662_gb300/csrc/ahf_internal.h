@@ -124,7 +124,7 @@ struct SkipRec {
 struct GridCtl {
   int work_n[2];                     // sub-tiles to process in the passes of each parity
   int overflow;                      // a radial bin would hold more members than it can
-  int pad0;
+  int no_bins;                       // so the sample foretold (before any member is counted)
   unsigned long long key_or, key_and;  // OR and AND of every radius key
   int pad[8];
 };

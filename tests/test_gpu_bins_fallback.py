@@ -125,3 +125,35 @@ def test_one_halo_with_equal_radii_leaves_the_others_in_bins():
     slot = np.repeat(rest, pop.count)
     np.testing.assert_array_equal(ha[2][slot], hb[2][slot])
     assert took[1] < 1.5 * took[0], took
+
+
+@pytest.mark.parametrize("mode", ["mixed", "fp64"])
+def test_most_of_a_large_halo_at_one_radius(mode):
+    # (counted one by one on one address, 1.8e6 members took five times the untied call)
+    torch = require_gpu()
+    import time
+    from paper_0904_3662_gb300 import ahf
+    fp64 = mode == "fp64"
+    n = 2_000_000
+    took = []
+    for ties in (0, 1_800_000):
+        rng = np.random.default_rng(47)
+        p, v, r = _shell(rng, n, ties)
+        order = rng.permutation(n)
+        pop = _population([(p[order], v[order], r)], _coord(mode))
+        prm = ahf.params_for(pop, precision=ahf.PREC_FP64 if fp64 else ahf.PREC_MIXED)
+        ctx = ahf.Context(0)
+        parts, hal = ahf.particles_from_population(pop), ahf.halos_from_population(pop)
+        out = ctx.alloc_outputs(1, n, precision=prm.precision)
+        best = 1e9
+        for _ in range(6):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            ctx.unbind_batch(parts, hal, prm, out=out)
+            torch.cuda.synchronize()
+            best = min(best, time.perf_counter() - t)
+        took.append(best)
+    tol = fp64_rtol(pop) if fp64 else 1e-5
+    compare(pop, prm, ahf.results_to_numpy(out["res"]), *[out[k].cpu().numpy() for k in ("bound_idx", "phi", "removed_iter")],
+            phi_rtol=tol, vir_rtol=tol, exact_order=fp64)
+    assert took[1] < 3.0 * took[0], took
