@@ -83,49 +83,42 @@ __device__ __forceinline__ double block_sums(const double s[NV], double* red /* 
   return t;
 }
 
-// A candidate for the peak: M^2 / r^2 by its bits, which order as it does, and its
-// place in the list (k < 0: none).  Each quotient is rounded once by itself, so the
-// larger, on ties the first in the list, is the same in whatever sequence a set is
-// taken; with cross products M'^2 r^2 > M^2 r'^2, which do not order a set where
-// thousands tie to rounding (a flat curve), and the candidates as they arrived, the
-// peak differed between calls.
-struct Peak {
-  unsigned long long q = 0;
-  long long k = -1;
-  // Takes (q2, k2) if it comes first.
-  __device__ __forceinline__ bool take(unsigned long long q2, long long k2) {
+// The place in the list of the peak among the CTA's threads: each brings the first
+// of its largest M^2 / r^2 (k < 0: none), as cross products find it in list order.
+// Between threads the quotients decide, rounded once each, on ties the first in
+// the list, which is the same however the threads are taken; cross products
+// M'^2 r^2 > M^2 r'^2 do not order a set where thousands tie to rounding (a flat
+// curve), and with the candidates as they arrived the peak differed between calls.
+// (A quotient for every particle instead: 20,000 haloes of 40 with a mass each
+// 1.4 -> 2.2 ms.)  -1: none; a NaN mass makes no candidate.
+__device__ __forceinline__ long long block_peak(double m, double r2, long long k) {
+  __shared__ unsigned long long sq[PT / 32];
+  __shared__ long long sk[PT / 32];
+  unsigned long long q = 0;              // the quotient's bits, which order as it does
+  auto take = [&](unsigned long long q2, long long k2) {
     const bool before = k2 >= 0 && (k < 0 || q2 > q || (q2 == q && k2 < k));
     q = before ? q2 : q;
     k = before ? k2 : k;
-    return before;
-  }
-  // (a NaN mass makes no candidate)
-  __device__ __forceinline__ bool take(double m, double r2, long long k2) {
-    const double x = m * m / r2;
-    return x >= 0.0 && take((unsigned long long)__double_as_longlong(x), k2);
-  }
-};
-
-// The place of the first among the CTA's threads' candidates (-1: none).
-__device__ __forceinline__ long long block_peak(Peak p) {
-  __shared__ unsigned long long sq[PT / 32];
-  __shared__ long long sk[PT / 32];
-  if (__any_sync(FULL_MASK, p.k >= 0)) {
+  };
+  if (__any_sync(FULL_MASK, k >= 0)) {
+    const double x = k >= 0 ? m * m / r2 : 0.0;
+    if (x >= 0.0) q = (unsigned long long)__double_as_longlong(x);
+    else k = -1;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long q = __shfl_xor_sync(FULL_MASK, p.q, o);
-      const long long k = __shfl_xor_sync(FULL_MASK, p.k, o);
-      p.take(q, k);
+      const unsigned long long q2 = __shfl_xor_sync(FULL_MASK, q, o);
+      const long long k2 = __shfl_xor_sync(FULL_MASK, k, o);
+      take(q2, k2);
     }
   }
   if ((threadIdx.x & 31) == 0) {
-    sq[threadIdx.x >> 5] = p.q;
-    sk[threadIdx.x >> 5] = p.k;
+    sq[threadIdx.x >> 5] = q;
+    sk[threadIdx.x >> 5] = k;
   }
   __syncthreads();
 #pragma unroll
-  for (int w = 0; w < PT / 32; ++w) p.take(sq[w], sk[w]);
-  return p.k;
+  for (int w = 0; w < PT / 32; ++w) take(sq[w], sk[w]);
+  return k;
 }
 
 // The largest of one float >= 0 per thread over the CTA.
@@ -138,7 +131,8 @@ __device__ __forceinline__ float block_max(float x, uint32_t* word) {
   return __uint_as_float(*word);
 }
 
-__device__ __forceinline__ bool is_normal(float x) { return x >= 1.17549435e-38f && x <= 3.40282347e+38f; }
+// x > 0, neither subnormal nor infinite nor NaN
+__device__ __forceinline__ bool is_normal(float x) { return __float_as_uint(x) - 0x800000u < 0x7f000000u; }
 
 // The float M^2 / r^2 a particle is first judged by: within 1e-6 of the exact
 // value while M^2, r^2 and their quotient are normal floats; where one is not
@@ -256,8 +250,8 @@ __global__ void __launch_bounds__(PT) props_uniform(PropsLaunch L) {
     out[14] = red[10];
     out[15] = (double)ne;
   }
-  Peak best;
   double bm = 0.0, br = 0.0;
+  long long bk = -1;
 #pragma unroll
   for (int j = 0; j < PER_T; ++j) {
     if (j * PT >= ne) break;
@@ -267,13 +261,14 @@ __global__ void __launch_bounds__(PT) props_uniform(PropsLaunch L) {
     load_f64<CT>(L, H, list[e], d, v, m);
     const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
     const double cum = (double)(start + e + 1);
-    if (r2 > 0.0 && best.take(cum, r2, start + e)) {
+    if (r2 > 0.0 && (bk < 0 || cum * cum * br > bm * bm * r2)) {
       bm = cum;
       br = r2;
+      bk = start + e;
     }
   }
-  const long long peak = block_peak(best);
-  if (peak < 0 ? threadIdx.x == 0 : best.k == peak) {
+  const long long peak = block_peak(bm, br, bk);
+  if (peak < 0 ? threadIdx.x == 0 : bk == peak) {
     out[16] = bm * L.p.m0;
     out[17] = br;
     out[18] = (double)peak;
@@ -385,18 +380,19 @@ __global__ void __launch_bounds__(PT) props_vmax(PropsLaunch L) {
   }
   const float least = peak_least(block_max(qm, &word));
   // the largest M(<= r_i) / r_i of the run (first one on ties)
-  Peak best;
   double best_m = 0.0, best_r2 = 0.0;
+  long long best_k = -1;
 #pragma unroll
   for (int j = 0; j < PER_T; ++j) {
     if (q[j] < least || q[j] < 0.0f) continue;
-    if (r2[j] > 0.0 && best.take(m[j], r2[j], k0 + j)) {
+    if (r2[j] > 0.0 && (best_k < 0 || m[j] * m[j] * best_r2 > best_m * best_m * r2[j])) {
       best_m = m[j];
       best_r2 = r2[j];
+      best_k = k0 + j;
     }
   }
-  const long long peak = block_peak(best);
-  if (peak < 0 ? threadIdx.x == 0 : best.k == peak) {
+  const long long peak = block_peak(best_m, best_r2, best_k);
+  if (peak < 0 ? threadIdx.x == 0 : best_k == peak) {
     double* out = L.part + (size_t)c * PROPS_PART;
     out[16] = best_m;
     out[17] = best_r2;
