@@ -83,42 +83,45 @@ __device__ __forceinline__ double block_sums(const double s[NV], double* red /* 
   return t;
 }
 
-// The place in the list of the peak among the CTA's threads: each brings the first
-// of its largest M^2 / r^2 (k < 0: none), as cross products find it in list order.
-// Between threads the quotients decide, rounded once each, on ties the first in
-// the list, which is the same however the threads are taken; cross products
+// Whether this thread holds the peak: each brings the first of its largest
+// M^2 / r^2 at place k of the list (k < 0: none), as cross products find it in list
+// order.  Between threads the quotients decide, rounded once each, on ties the
+// first in the list, which is the same however the threads are taken; cross products
 // M'^2 r^2 > M^2 r'^2 do not order a set where thousands tie to rounding (a flat
 // curve), and with the candidates as they arrived the peak differed between calls.
 // (A quotient for every particle instead: 20,000 haloes of 40 with a mass each
-// 1.4 -> 2.2 ms.)  -1: none; a NaN mass makes no candidate.
-__device__ __forceinline__ long long block_peak(double m, double r2, long long k) {
+// 1.4 -> 2.2 ms.)  Thread 0's none when there is no candidate; a NaN mass makes none.
+__device__ __forceinline__ bool block_peak(double m, double r2, long long k) {
   __shared__ unsigned long long sq[PT / 32];
   __shared__ long long sk[PT / 32];
-  unsigned long long q = 0;              // the quotient's bits, which order as it does
-  auto take = [&](unsigned long long q2, long long k2) {
-    const bool before = k2 >= 0 && (k < 0 || q2 > q || (q2 == q && k2 < k));
-    q = before ? q2 : q;
-    k = before ? k2 : k;
+  const int n = __syncthreads_count(k >= 0);
+  if (n <= 1) return n ? k >= 0 : threadIdx.x == 0;      // mostly one thread's
+  unsigned long long best = 0;           // the quotient's bits, which order as it does
+  long long at = k;
+  auto take = [&](unsigned long long q, long long k2) {
+    const bool before = k2 >= 0 && (at < 0 || q > best || (q == best && k2 < at));
+    best = before ? q : best;
+    at = before ? k2 : at;
   };
   if (__any_sync(FULL_MASK, k >= 0)) {
-    const double x = k >= 0 ? m * m / r2 : 0.0;
-    if (x >= 0.0) q = (unsigned long long)__double_as_longlong(x);
-    else k = -1;
+    const double q = k >= 0 ? m * m / r2 : 0.0;
+    if (q >= 0.0) best = (unsigned long long)__double_as_longlong(q);
+    else at = -1;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long q2 = __shfl_xor_sync(FULL_MASK, q, o);
-      const long long k2 = __shfl_xor_sync(FULL_MASK, k, o);
+      const unsigned long long q2 = __shfl_xor_sync(FULL_MASK, best, o);
+      const long long k2 = __shfl_xor_sync(FULL_MASK, at, o);
       take(q2, k2);
     }
   }
   if ((threadIdx.x & 31) == 0) {
-    sq[threadIdx.x >> 5] = q;
-    sk[threadIdx.x >> 5] = k;
+    sq[threadIdx.x >> 5] = best;
+    sk[threadIdx.x >> 5] = at;
   }
   __syncthreads();
 #pragma unroll
   for (int w = 0; w < PT / 32; ++w) take(sq[w], sk[w]);
-  return k;
+  return at < 0 ? threadIdx.x == 0 : at == k;
 }
 
 // The largest of one float >= 0 per thread over the CTA.
@@ -267,11 +270,10 @@ __global__ void __launch_bounds__(PT) props_uniform(PropsLaunch L) {
       bk = start + e;
     }
   }
-  const long long peak = block_peak(bm, br, bk);
-  if (peak < 0 ? threadIdx.x == 0 : bk == peak) {
+  if (block_peak(bm, br, bk)) {
     out[16] = bm * L.p.m0;
     out[17] = br;
-    out[18] = (double)peak;
+    out[18] = (double)bk;
   }
 }
 
@@ -391,12 +393,11 @@ __global__ void __launch_bounds__(PT) props_vmax(PropsLaunch L) {
       best_k = k0 + j;
     }
   }
-  const long long peak = block_peak(best_m, best_r2, best_k);
-  if (peak < 0 ? threadIdx.x == 0 : best_k == peak) {
+  if (block_peak(best_m, best_r2, best_k)) {
     double* out = L.part + (size_t)c * PROPS_PART;
     out[16] = best_m;
     out[17] = best_r2;
-    out[18] = (double)peak;
+    out[18] = (double)best_k;
   }
 }
 
