@@ -1404,6 +1404,7 @@ int match_impl(ahf_ctx* c, int64_t n_ids, const int64_t* ids_a, const int64_t* o
   L.n_a = (int)n_a;
   L.ids_b = (const long long*)ids_b; L.off_b = (const long long*)off_b; L.cnt_b = (const long long*)cnt_b;
   L.n_b = (int)n_b;
+  L.sms = c->sms;
   L.err = c->err_dev;
   L.best = (long long*)best; L.shared = (long long*)shared; L.xi = xi;
   AHF_CUDA(launch_match(L, s));

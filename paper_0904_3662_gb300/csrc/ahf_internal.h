@@ -378,6 +378,7 @@ struct MatchLaunch {
   const long long *ids_b, *off_b, *cnt_b;
   int n_b;
   int *label;                            // [n_ids] workspace
+  int sms;                               // multiprocessors of the device
   int *err;
   long long *best, *shared;
   double *xi;

@@ -451,18 +451,28 @@ __global__ void props_final(PropsLaunch L) {
 
 // ---- matching ----------------------------------------------------------------
 
+constexpr int M_UNROLL = 4;              // ids in flight per thread
+
 // The ids of halo blockIdx.x, spread over gridDim.y CTAs.
 __global__ void __launch_bounds__(PT) match_label(MatchLaunch L) {
   const int b = blockIdx.x;
   const long long off = L.off_b[b], cnt = L.cnt_b[b];
-  for (long long k = (long long)blockIdx.y * PT + threadIdx.x; k < cnt; k += (long long)gridDim.y * PT) {
-    const long long id = L.ids_b[off + k];
-    if (id < 0 || id >= L.n_ids) {
-      atomicOr(L.err, ERR_ID_RANGE);
-      continue;
+  const long long step = (long long)gridDim.y * PT;
+  for (long long k0 = (long long)blockIdx.y * PT + threadIdx.x; k0 < cnt; k0 += M_UNROLL * step) {
+    long long id[M_UNROLL];
+    int old[M_UNROLL];
+#pragma unroll
+    for (int j = 0; j < M_UNROLL; ++j) id[j] = k0 + j * step < cnt ? L.ids_b[off + k0 + j * step] : 0;
+#pragma unroll
+    for (int j = 0; j < M_UNROLL; ++j) {
+      old[j] = b;
+      if (k0 + j * step >= cnt) continue;
+      if (id[j] < 0 || id[j] >= L.n_ids) atomicOr(L.err, ERR_ID_RANGE);
+      else old[j] = atomicCAS(&L.label[id[j]], -1, b);
     }
-    const int old = atomicCAS(&L.label[id], -1, b);
-    if (old != -1 && old != b) atomicOr(L.err, ERR_SHARED_ID);
+#pragma unroll
+    for (int j = 0; j < M_UNROLL; ++j)
+      if (old[j] != -1 && old[j] != b) atomicOr(L.err, ERR_SHARED_ID);
   }
 }
 
@@ -471,7 +481,6 @@ __global__ void __launch_bounds__(PT) match_label(MatchLaunch L) {
 // id queued on one counter, and one thread's search of the table cost as much;
 // 182 -> 53 us for 1,500 haloes of 1.2e6 ids, caches cold).
 constexpr int MT = 512;
-constexpr int M_UNROLL = 4;              // ids in flight per thread
 
 __global__ void __launch_bounds__(MT) match_best(MatchLaunch L) {
   __shared__ int key[MATCH_TABLE];
@@ -592,10 +601,15 @@ cudaError_t launch_properties(const PropsLaunch& L, cudaStream_t s) {
 }
 
 cudaError_t launch_match(const MatchLaunch& L, cudaStream_t s) {
-  // some 38,000 CTAs in all while haloes are few, 64 per halo at most: the list
-  // lengths are on the device, and one CTA took 130 us over a halo of 41,000 (29 us)
-  if (L.n_b > 0)
-    match_label<<<dim3((unsigned)L.n_b, (unsigned)std::min(64, std::max(1, 38912 / L.n_b))), PT, 0, s>>>(L);
+  // The list lengths are on the device.  One CTA took 130 us over a halo of 41,000
+  // ids, so a halo gets up to 64 (of 4 ids a thread) while that is 64 an SM in all
+  // at most.  (Four times as many, of an id a thread, took as long over long lists
+  // but had mostly nothing to do for short ones: 600 haloes of 100 ids, a call
+  // alone, 63 us; one CTA a halo 55; now 50.)
+  if (L.n_b > 0) {
+    const int shares = std::min(64, std::max(1, 64 * L.sms / L.n_b));
+    match_label<<<dim3((unsigned)L.n_b, (unsigned)shares), PT, 0, s>>>(L);
+  }
   if (L.n_a > 0) match_best<<<L.n_a, MT, 0, s>>>(L);
   return cudaGetLastError();
 }
