@@ -688,6 +688,9 @@ int run_grid(ahf_ctx* c, GridLaunch& G, const ahf_params* prm, cudaStream_t s, i
       std::memcpy(&andb, c->flag_host + 2, 8);
       AHF_CUDA(grid_sort(G, s, orb, andb));
       c->stats.launches += 2 + G.sort_launches;
+      // (the sort's phase ends here, the iterations' begins)
+      if ((rc = phase_end(c, PH_GRID_SORT, s))) return rc;
+      if ((rc = phase_begin(c, PH_GRID_ITER, s, 0, 0))) return rc;
       continue;
     }
     if (pass > prm->max_iter || c->flag_host[pass & 1] == 0) break;

@@ -91,6 +91,20 @@ def test_abandoned_bins_do_not_count_as_iterations(mode):
     assert st[PART]["grid_iterations"] == st[BIN + 1]["grid_iterations"] == 8
 
 
+def test_radix_sort_after_bins_is_timed_as_sort():
+    require_gpu()
+    from paper_0904_3662_gb300 import ahf
+    pop = _population([_shell(np.random.default_rng(53), 300_000, 100_000)], synth.COORD_F64)
+    ctx = ahf.Context(0)
+    ctx.set_option(ahf.OPT_TIMING, 1)
+    run_gpu(pop, params=ahf.params_for(pop, precision=ahf.PREC_FP64, max_iter=1), ctx=ctx)
+    st = ctx.stats()
+    sort, iterate = (ahf.PHASE_NAMES.index(k) for k in ("grid_gather_sort", "grid_iterate"))
+    assert st["phase_halos"][sort] == st["phase_halos"][iterate] == 1
+    # eight radix passes against one pass of the iteration
+    assert st["phase_ms"][sort] > 2.0 * st["phase_ms"][iterate]
+
+
 def test_one_halo_with_equal_radii_leaves_the_others_in_bins():
     # (the radix sort of every halo takes about as long as the whole call in bins)
     torch = require_gpu()
