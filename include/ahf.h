@@ -249,7 +249,9 @@ int ahf_profile_batch(ahf_ctx *ctx, const ahf_particles *p, const ahf_halo *halo
  * the multi-CTA passes gave up waiting for its tensor copy into shared
  * memory (AHF_OPT_WAIT_LIMIT; the results of that call are then undefined).
  * The device error word is cleared by the call.  No kernel waits for
- * another CTA. */
+ * another CTA outside its own cluster, except that the launches of several
+ * on-chip size classes end in order: a launch's last worker waits for the end
+ * of the launch before it, whose CTAs are all on SMs by then. */
 int ahf_sync(ahf_ctx *ctx);
 
 /* ahf_unbind_batch and ahf_profile_batch in one call: the same arguments
@@ -351,7 +353,9 @@ int ahf_unbind_profile_batch(ahf_ctx *ctx, const ahf_particles *p, const ahf_hal
 typedef struct ahf_stats {
   int64_t launches;                    /* kernels launched by the call        */
   int64_t host_syncs;                  /* host synchronisations in the call   */
-  int64_t grid_iterations;             /* multi-CTA iterations launched       */
+  int64_t grid_iterations;             /* multi-CTA iterations launched (not those
+                                          of an attempt at the radial order that
+                                          the radix sort replaced)            */
   int64_t phase_halos[AHF_N_PHASES];
   int64_t phase_candidates[AHF_N_PHASES];
   double phase_ms[AHF_N_PHASES];

@@ -1052,7 +1052,6 @@ __device__ __forceinline__ int sm_id() {
   return s;
 }
 
-// Record trace field f of halo h (no-op when tracing is off).
 // Chained launches (OnchipLaunch::done): let the next launch of the stream start
 // beside this one (no effect unless it asks for that) ...
 __device__ __forceinline__ void chain_open() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -1065,6 +1064,7 @@ __device__ __forceinline__ void chain_close(int* done, int n) {
   if (done && atomicAdd(done, 1) == n - 1) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// Record trace field f of halo h (no-op when tracing is off).
 __device__ __forceinline__ void trace_mark(long long* trace, int h, int f) {
   if (trace) trace[(size_t)h * AHF_TRACE_FIELDS + f] = global_ns();
 }

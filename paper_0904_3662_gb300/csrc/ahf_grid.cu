@@ -10,26 +10,26 @@
 //            (v, m) with w = v + H d (64 bytes in the all-FP64 mode)
 //   sort     members distributed into radial bins by rank of arrival (counted
 //            by the prepare), each bin then ordered on chip by one CTA, which
-//            writes the radial-order streams (w, r), (v, m), so no later step
+//            writes the radial-order streams (w, r), (v, 1/r), so no later step
 //            touches the particle store.  Radii that the bins cannot hold
-//            (hundreds equal, a thin shell in a void) take a segmented stable LSD
+//            (thousands equal, a thin shell in a void) take a segmented stable LSD
 //            radix sort of (key, position) with 8-bit digits instead
 //   init     exact sums of the initial set per sub-tile (with the bins) and per
 //            halo, v_bulk
-//   passes   ONE streaming kernel per iteration: each tile takes the exact
-//            prefix sums M(<r) and sum m/r of the tiles before it from the
-//            tile prefixes of the current set, evaluates phi (Appendix A),
-//            the escape test and the removals, and subtracts what it removed
-//            from its own sums; the last tile of a halo to finish turns the
-//            tiles' sums into the prefixes of the set left, the halo's
-//            totals, v_bulk and its convergence
+//   passes   two kernels per iteration.  A streaming one: each sub-tile of an
+//            active halo takes the exact prefix sums M(<r) and sum m/r of the
+//            tiles before it from the tile prefixes of the current set,
+//            evaluates phi (Appendix A), the escape test and the removals, and
+//            subtracts what it removed from its own sums.  Then one CTA or warp
+//            per halo (g_halo) turns the sub-tiles' sums into the prefixes of
+//            the set left, the halo's totals, v_bulk, its convergence and its
+//            part of the next pass's list
 //   final    bound lists, phi, compacted radii and inclusive masses, the
 //            first virial crossing, the records, and the profile rows by
 //            binary search over the compacted radii
 //
 // No CTA ever waits for another one: a tile reads only prefixes that an
-// earlier kernel finished, and each halo's bookkeeping is done by whichever
-// of its tiles finishes last (an atomic count).
+// earlier kernel finished.
 
 // Exact sums: long long fixed point in the mixed mode (the same scales and
 // bits as the on-chip classes), __int128 in the all-FP64 mode, where a
@@ -3048,7 +3048,6 @@ void launch_halo_init(const GridLaunch& L, cudaStream_t s) {
 // The distribution into radial bins (see g_sample).
 template <typename R>
 cudaError_t bins_t(GridLaunch& L, cudaStream_t s) {
-  L.sort_passes = 0;
   L.sort_launches = 0;
   if (L.n_tiles == 0) {
     g_scales<R><<<blocks_for(L.n_halos, 128), 128, 0, s>>>(L);
@@ -3096,7 +3095,6 @@ cudaError_t sort_t(GridLaunch& L, cudaStream_t s, unsigned long long or_bits, un
   for (int d = 0; d < (int)sizeof(Key); ++d)
     if ((diff >> (8 * d)) & 0xffull) digits[nd++] = d;
   if (L.n_tiles == 0) nd = 0;
-  L.sort_passes = nd;
   L.sort_launches = 0;
   if (L.n_tiles == 0) return cudaGetLastError();
   Key *ki = (Key*)L.key_a, *ko = (Key*)L.key_b;

@@ -123,7 +123,8 @@ struct SkipRec {
 // Device control words of one multi-CTA call.
 struct GridCtl {
   int work_n[2];                     // sub-tiles to process in the passes of each parity
-  int overflow;                      // a radial bin would hold more members than it can
+  int overflow;                      // a radial bin would hold more members than it can: set by the
+                                     // prepare, which counts them, or foretold (no_bins)
   int no_bins;                       // so the sample foretold (before any member is counted)
   unsigned long long key_or, key_and;  // OR and AND of every radius key
   int pad[8];
@@ -224,7 +225,7 @@ struct GridLaunch {
   void* ms_b;              // masses by bin
   uint32_t *bin_n, *bin_at;  // per bin (two per tile): members (a 128-byte line each, in
                            // tile_hist), first position in the halo
-  void* vr;                // radial order: (v, m); NULL after the radix sort (then by
+  void* vr;                // radial order: (v, 1/r); NULL after the radix sort (then (v, m) by
                            // candidate, in rec)
   void *wr_bins, *vr_bins; // wr and vr after the bins (in rec, which the bins are done with)
   void* wr_radix;          // wr after the radix sort
@@ -261,7 +262,6 @@ struct GridLaunch {
                            // haloes for the passes of each parity: (sub-tile, halo, first
                            // flat element, members in it)
   int iter_grid;           // CTAs of the persistent iteration pass
-  int sort_passes;         // radix passes the last grid_sort launched (0: bins)
   int sort_launches;       // kernel launches of the last grid_bins or grid_sort
   ProfileRows rows;        // rows.prof != NULL: profile rows from the final pass
 };

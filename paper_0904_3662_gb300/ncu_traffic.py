@@ -8,15 +8,22 @@ that ncu writes (`--csv --log-file`) into the table bench.py reads
 the phase's kernel sources, so that a number taken on older kernels is not
 reported for newer ones.
 
-The capture (on the GPU machine, after the same command exited 0 without ncu):
+The captures (each after the same command exited 0 without ncu): one kernel each
+and a few launches, on a case that holds little device memory, since a list of
+several metrics takes several passes per launch and restores the memory between
+them.  For an on-chip size class of the 2,000-halo batch, e.g. the 16-CTA cluster:
 
     ncu --metrics gpu__time_duration.sum,dram__bytes_read.sum,dram__bytes_write.sum,smsp__inst_executed.sum \\
-        --clock-control none --csv --log-file launches.csv \\
+        --clock-control none --kernel-name-base demangled -k "regex:unbind_kernel<.*16>" -s 3 -c 2 \\
+        --csv --log-file launches.csv \\
         python bench.py --steps 2 --warmup 3 --no-plain --no-e2e --no-cpu-baseline --no-graphs --no-tune
 
-and then, anywhere:
+and then, anywhere, once per list (each adds or replaces the entries it holds):
 
     python -m paper_0904_3662_gb300.ncu_traffic launches.csv --workload batch
+
+A list of every launch of a whole workload takes gpu__time_duration.sum alone (one
+pass).
 
 Phases: each on-chip size class is one kernel launch per call (the figure is
 the mean over its launches); each multi-CTA phase is several kernels per call
